@@ -102,8 +102,9 @@ typedef struct {
     long long cell_updates;   /* fluid cells x (drag + relaxation + standard steps) since creation */
     size_t device_bytes;      /* device memory held by the handle */
     long long kernel_launches; /* CUDA kernels launched by this handle since creation */
-    int mg_first_cta_level;   /* first multigrid level held in one CTA's shared memory */
-    int mg_cta_global_level;  /* level worked by that CTA with coefficients in global memory, -1 when none */
+    int mg_first_cta_level;   /* first multigrid level of at most cta_cells cells (oscar_schedule): it and the
+                                 coarser ones are worked in the shared memory of one thread-block cluster */
+    int mg_cta_global_level;  /* first of the larger levels that the cluster works too, -1 when none */
 } oscar_stats_t;
 
 typedef struct oscar_instance *oscar_handle;
@@ -203,17 +204,17 @@ int oscar_stats(oscar_handle h, oscar_stats_t *out);
  * Defaults at creation: {2, 2, 2, 1024, 8, 0, 1}. */
 typedef struct {
     int mg_nu;          /* red-black Gauss-Seidel sweep pairs per smoothing step, finest level: 1..4 */
-    int mg_nu_mid;      /* the same on the levels between the finest and the coarse CTA: 1..4 */
-    int mg_nu_cta;      /* the same on the levels held by the single coarse CTA: 1..6 */
-    int cta_cells;      /* levels of at most this many cells (and fitting its shared memory) go to the
-                           coarse CTA: 1..1024 */
-    int coarse_refresh; /* the coarsest CTA level's explicit inverse is formed on the first PISO set-up of
+    int mg_nu_mid;      /* the same on the coarser levels of more than cta_cells cells: 1..4 */
+    int mg_nu_cta;      /* the same on the levels of at most cta_cells cells: 1..6 */
+    int cta_cells;      /* levels of at most this many cells (and fitting the shared memory) are worked by one
+                           thread-block cluster: 1..1024 */
+    int coarse_refresh; /* the explicit inverse of the cluster's coarsest level is formed on the first PISO set-up of
                            a step call and every coarse_refresh-th after it, kept in between: 1..1000 */
     int block_x;        /* cap on the x extent of the 256-thread blocks of cell kernels: 0 (none), 32, 64,
                            128 or 256 */
-    int cta_global;     /* 1: the level just above the coarse CTA's levels (not the finest) is worked by
-                           the same CTA, its x and b in shared memory and its coefficients read from
-                           global memory, when that fits; 0: by per-level kernels */
+    int cta_global;     /* 1: the cluster has several CTAs and also takes larger levels (not the finest) when
+                           they fit, and a small 2D grid's pressure solve runs whole in one cluster; 0: a
+                           cluster of one CTA, with the levels of at most cta_cells cells only */
 } oscar_schedule;
 
 /* Read the schedule of an instance. */
@@ -260,8 +261,9 @@ int oscar_profile_read(oscar_handle h, int index, int *count_out, char *name_out
  * run from their (rebuilt) CUDA graphs as usual; the time they add over the
  * same steps of an identical instance, divided by the launches they add
  * (oscar_stats kernel_launches), is the in-graph duration of one such sweep
- * with its operands where the step leaves them. enable = 0 restores normal
- * steps. Waits for the stream. OSCAR_E_INVALID_ARG while an asynchronous step
+ * with its operands where the step leaves them. (A small 2D instance whose
+ * solves run whole in one cluster launches no such sweeps: nothing is added.)
+ * enable = 0 restores normal steps. Waits for the stream. OSCAR_E_INVALID_ARG while an asynchronous step
  * is pending. */
 int oscar_profile_repeat(oscar_handle h, int enable);
 

@@ -190,7 +190,7 @@ static void carve(Instance &I, Carver &C) {
         L.res = C.take(n * es);
     }
     I.stage_dev = (double *)C.take(I.stage_len * sizeof(double));
-    I.cta_img = C.take(kCtaImageBytes);
+    I.cl_inv = C.take(kClInvBytes);
     I.partials = (double *)C.take((size_t)kRedSlots * I.red_stride * sizeof(double));
     I.scal = (double *)C.take(S_COUNT * sizeof(double));
     I.ctl = (int *)C.take(C_COUNT * sizeof(int));
@@ -372,6 +372,10 @@ int oscar_create(const oscar_params *p, const uint8_t *solid, const double *alph
     bool streams_ok = true;
     for (int q = 0; q < 4; ++q)
         if (cudaStreamCreateWithFlags(&I.side[q], cudaStreamNonBlocking) != cudaSuccess) streams_ok = false;
+    if (cudaStreamCreateWithFlags(&I.aux, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&I.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&I.ev_join, cudaEventDisableTiming) != cudaSuccess)
+        streams_ok = false;
     if (!streams_ok || cudaMallocHost(&I.scal_host, S_COUNT * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&I.ctl_host, C_COUNT * sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&I.stage_host, stage * sizeof(double)) != cudaSuccess) {
@@ -408,6 +412,9 @@ int oscar_destroy(oscar_handle h) {
     }
     for (int q = 0; q < 4; ++q)
         if (I.side[q]) cudaStreamDestroy(I.side[q]);
+    if (I.aux) cudaStreamDestroy(I.aux);
+    if (I.ev_fork) cudaEventDestroy(I.ev_fork);
+    if (I.ev_join) cudaEventDestroy(I.ev_join);
     if (I.own_stream && I.stream) cudaStreamDestroy(I.stream);
     if (I.ctl_host) cudaFreeHost(I.ctl_host);
     if (I.prof) {
@@ -557,24 +564,26 @@ int oscar_set_schedule(oscar_handle h, const oscar_schedule *s) {
     if (s->cta_global != 0 && s->cta_global != 1) return OSCAR_E_INVALID_ARG;
     int rc = sync_bounded(I.stream, kSyncTimeoutSec);
     if (rc) return rc;
-    const int lc0 = I.lc0, lg = I.lg, cg = I.cta_global;
-    const size_t sm = I.cta_smem, ib = I.cta_img_bytes;
-    I.cta_global = s->cta_global;
-    rc = I.prec == OSCAR_FP64 ? Solver<double>::choose_cta(I, s->cta_cells) : Solver<float>::choose_cta(I, s->cta_cells);
-    if (rc) {   // keep the previous schedule
-        I.lc0 = lc0;
-        I.lg = lg;
-        I.cta_global = cg;
-        I.cta_smem = sm;
-        I.cta_img_bytes = ib;
+    // the layout of the cluster's levels depends on the sweeps as well: set
+    // everything, then choose, and go back to the previous schedule on failure
+    oscar_schedule old;
+    oscar_get_schedule(h, &old);
+    auto apply = [&](const oscar_schedule &v) {
+        I.mg_nu = v.mg_nu;
+        I.mg_nu_c = v.mg_nu_mid;
+        I.mg_nu_cta = v.mg_nu_cta;
+        I.cta_cells = v.cta_cells;
+        I.coarse_refresh = v.coarse_refresh;
+        I.block_x = v.block_x;
+        I.cta_global = v.cta_global;
+        return I.prec == OSCAR_FP64 ? Solver<double>::choose_cta(I, v.cta_cells)
+                                    : Solver<float>::choose_cta(I, v.cta_cells);
+    };
+    rc = apply(*s);
+    if (rc) {
+        apply(old);
         return rc;
     }
-    I.mg_nu = s->mg_nu;
-    I.mg_nu_c = s->mg_nu_mid;
-    I.mg_nu_cta = s->mg_nu_cta;
-    I.cta_cells = s->cta_cells;
-    I.coarse_refresh = s->coarse_refresh;
-    I.block_x = s->block_x;
     if (I.prec == OSCAR_FP64) Solver<double>::release_graphs(I);
     else Solver<float>::release_graphs(I);
     return 0;

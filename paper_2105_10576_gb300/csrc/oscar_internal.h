@@ -14,7 +14,7 @@ constexpr int kMaxLevels = 24;
 constexpr int kRedBlocks = 1216;      // 152 SMs x 8: fixed grid of every reduction (deterministic order)
 constexpr int kRedSlots = 16;         // partial-sum slots
 constexpr double kSyncTimeoutSec = 600.0;
-constexpr size_t kCtaImageBytes = 224 * 1024;   // shared-memory budget of the coarse CTA
+constexpr size_t kClInvBytes = 128 * 128 * sizeof(double);   // explicit inverse of a level of at most 128 cells
 
 // Scalar slots in the device scalar array (double).
 enum Slot {
@@ -123,11 +123,15 @@ struct Instance {
     // reductions
     double *partials;      // kRedSlots * red_stride
     int red_stride;        // partials per slot: max(kRedBlocks, blocks of a cell launch)
-    int lc0;               // first multigrid level solved by the single-CTA coarse kernel
-    size_t cta_smem;       // shared memory of the coarse kernel
-    size_t cta_img_bytes;  // bytes of the coarse levels' image (the start of that shared memory)
-    int lg;                // level worked by the coarse CTA with global coefficients, -1 when none
-    void *cta_img;         // shared-memory image of the coarse levels (kCtaImageBytes, built per PISO set-up)
+    int lc0;               // first multigrid level of at most cta_cells cells
+    int lg;                // first of the levels above lc0 that the cluster works too, -1 when none
+    int cl_nc;             // CTAs of the V-cycle's cluster
+    size_t cl_smem;        // shared memory of each of them
+    int solve_nc;          // CTAs of the whole-solve cluster, 0 when solves run as launches
+    size_t solve_smem;
+    void *cl_inv;          // explicit inverse of the coarsest level (kClInvBytes)
+    cudaStream_t aux;      // branch of the operator set-up
+    cudaEvent_t ev_fork, ev_join;
     int pending;           // kind (0 drag, 1 relax, 2 standard) of a launched step not yet waited for, or -1
     double pending_dt;
     int pending_N;
@@ -145,12 +149,12 @@ struct Instance {
     int cg_iters_last;
     long long cell_updates;
     int mg_nu, mg_nu_c, mg_coarse_sweeps;   // sweeps on the finest level, on coarser levels, on the coarsest
-    int mg_nu_cta;         // sweeps on the levels held by the coarse CTA
+    int mg_nu_cta;         // sweeps on the levels of at most cta_cells cells
     int repeat_fine;       // measurement: finest-level plain half sweeps issued twice (oscar_profile_repeat)
     int coarse_refresh;    // the coarsest level's inverse is formed every this many PISO set-ups
-    int cta_cells;         // levels of at most this many cells go to the coarse CTA
+    int cta_cells;         // levels of at most this many cells go to the cluster (one CTA's worth)
     int block_x;           // cap on the x extent of cell-kernel blocks (0: none)
-    int cta_global;        // 1: the level above the CTA's may go to the CTA with global coefficients
+    int cta_global;        // 1: clusters of several CTAs, which also take larger levels; 0: one CTA
     long long nlaunch;     // kernel launches issued by the host (eager or into a capture)
     long long nexec;       // kernels executed on the device (graph executions counted by loop trips)
     Profiler *prof;
@@ -182,7 +186,7 @@ template <typename T> struct Solver {
     static int field_from_device(Instance &I, int which, const double *src, size_t n);
     static int phase_volume(Instance &I, double *out);
     static void release_graphs(Instance &I);
-    static int choose_cta(Instance &I, long long cap);   // first CTA level and its shared memory
+    static int choose_cta(Instance &I, long long cap);   // the cluster's levels, CTAs and shared memory
 };
 
 int sync_bounded(cudaStream_t s, double timeout_sec);

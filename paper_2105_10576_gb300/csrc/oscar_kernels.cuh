@@ -32,8 +32,7 @@ namespace oscar {
 enum : int { FT_NONE = 0, FT_INTERIOR = 1, FT_WALL = 2, FT_INLET = 3, FT_OUTLET = 4 };
 constexpr uint32_t INFO_FLUID = 1u << 31;
 constexpr int BS = 256;
-constexpr int kCtaCells = 1024;      // levels at or below this size run in one CTA
-constexpr int kMaxCL = 16;
+constexpr int kCtaCells = 1024;      // largest cta_cells of a schedule
 constexpr int kApplyRows = 2;    // rows per thread of k_cg_pz_apply
 constexpr int kUpdateRows = 4;   // rows per thread of k_cg_update
 
@@ -1756,66 +1755,6 @@ __global__ void k_mg_diag(GridD g, const uint8_t *__restrict__ fluid, MG3<M> cc,
     idiag[c] = acc > M(0) ? M(1) / acc : M(0);
 }
 
-// The V-cycle on the coarse levels in one CTA, with every level held in
-// shared memory. The face coefficients are copied in asynchronously
-// (cp.async) and rearranged once per launch into per-cell form: the six
-// neighbour coefficients (zero across the domain boundary), the diagonal
-// (sum of the six face coefficients, as k_mg_diag) and its reciprocal, the
-// packed cell coordinates and, per colour, the list of fluid cells. x carries
-// a zero pad of one plane on each side, so the stencil reads need no bounds
-// tests. A smoothing step is then a handful of shared-memory loads and FMAs
-// per cell. Same symmetric schedule as the per-level kernels (pre-smoothing
-// red-black, post-smoothing black-red, symmetric sweeps on the coarsest
-// level); the residual for the restriction is formed cell-parallel first.
-constexpr int kCtaThreads = 1024;
-constexpr int kExactCells = 128;   // coarsest CTA level solved exactly when at most this size
-constexpr int kGlCells = 2048;     // largest level the CTA works with global coefficients (larger ones
-                                   // ran slower there than as per-level launches: 4 or more cells per
-                                   // thread and seven L2 loads per cell and sweep)
-template <typename M> struct CLevel {
-    GridD g;
-    const M *c[3];          // global face coefficients
-    const uint8_t *fluid;
-    int r[3];               // ratios to the next level (1 or 2)
-    float rnx, rny, rhx;    // 1/nx, 1/ny, 1/ceil(nx/2) for the cell decomposition
-    int nh;                 // entries of a colour list: ceil(nx/2) ny nz
-    // shared-memory byte offsets: x (past its pad), b, diagonal, reciprocal,
-    // neighbour coefficients (2 DIM per cell), packed coordinates, colour
-    // lists, fluid flags, staging of the face arrays
-    int ox, ob, od, oi, ow, opk, ol[2], ofl, os[3];
-};
-// The level just above the coarse CTA's levels, worked by the same CTA with
-// its x and b in shared memory and its coefficients, diagonal, inverse
-// diagonal and fluid flags read from global memory (the level is too large for
-// the per-cell form, small enough for its x and b). Same operations as the
-// per-level kernels: red-black sweeps from x = 0, residual and restriction
-// into the CTA's first level, prolongation, reverse-order sweeps.
-template <typename M> struct GLevel {
-    int active;
-    GridD g;
-    MG3<M> c;                  // face coefficients
-    const M *diag, *idiag;
-    const uint8_t *fluid;
-    int r[3];                  // ratios to the CTA's first level
-    float rhx, rny;            // 1/ceil(nx/2), 1/ny (colour-cell decomposition)
-    int ox, ob;                // shared-memory byte offsets of x and b
-    int nu;                    // sweep pairs per smoothing step
-    const M *b_glob;           // b of the level (written by the preceding restriction)
-    M *x_glob;                 // x of the level after the post-smoothing
-};
-template <typename M> struct CLevels {
-    GLevel<M> G;
-    int n, nu, nu_top, coarse_sweeps;
-    int ors;           // residual scratch (cells of the largest level)
-    // exact = 1: the coarsest level (at most kExactCells cells) is solved with
-    // its explicit inverse, stored row-major at oinv (built by
-    // k_mg_coarse_pack every refresh-th call, kept in between)
-    int exact, oinv, refresh;
-    const M *b_top;    // global b of the top level
-    M *x_top;          // global x of the top level
-    CLevel<M> L[kMaxCL];
-};
-
 // idx -> (a, b, c) with idx = a + n0 * (b + n1 * c), without integer
 // division (float reciprocals, corrected by one step; exact below 2^22)
 __device__ __forceinline__ void split3(int idx, int n0, float rn0, int n1, float rn1, int &a, int &b, int &c) {
@@ -1825,451 +1764,6 @@ __device__ __forceinline__ void split3(int idx, int n0, float rn0, int n1, float
     c = (int)(((float)r + 0.5f) * rn1);
     b = r - c * n1;
     if (b < 0) { --c; b += n1; } else if (b >= n1) { ++c; b -= n1; }
-}
-
-template <int B> struct CpAsync;
-template <> struct CpAsync<4> {
-    __device__ static __forceinline__ void copy(void *dst, const void *src) {
-        unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(src) : "memory");
-    }
-};
-template <> struct CpAsync<8> {
-    __device__ static __forceinline__ void copy(void *dst, const void *src) {
-        unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(src) : "memory");
-    }
-};
-template <> struct CpAsync<16> {   // both addresses 16-byte aligned; cached in L2 only
-    __device__ static __forceinline__ void copy(void *dst, const void *src) {
-        unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src) : "memory");
-    }
-};
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-constexpr uint32_t kPkFluid = 1u << 31;
-__device__ __forceinline__ void pk_ijk(uint32_t pk, int &i, int &j, int &k) {
-    i = (int)(pk & 1023u);
-    j = (int)((pk >> 10) & 1023u);
-    k = (int)((pk >> 20) & 1023u);
-}
-
-// sum of the neighbour terms of one row
-template <int DIM, typename M>
-__device__ __forceinline__ M cta_off(const M *__restrict__ w, const M *x, int cell, int nx, int nxy) {
-    M off = w[0] * x[cell - 1] + w[1] * x[cell + 1];
-    off += w[2] * x[cell - nx] + w[3] * x[cell + nx];
-    if (DIM == 3) off += w[4] * x[cell - nxy] + w[5] * x[cell + nxy];
-    return off;
-}
-
-// one colour of a red-black sweep, by threads t0, t0 + st, ... (no barrier)
-template <int DIM, typename M>
-__device__ __forceinline__ void cta_sweep(const CLevel<M> &L, unsigned char *sm, int colour, int t0, int st) {
-    M *x = (M *)(sm + L.ox);
-    const M *b = (const M *)(sm + L.ob), *iv = (const M *)(sm + L.oi), *w = (const M *)(sm + L.ow);
-    const unsigned short *lst = (const unsigned short *)(sm + L.ol[colour]);
-    const int nx = L.g.nx, nxy = L.g.nx * L.g.ny;
-    for (int h = t0; h < L.nh; h += st) {
-        const int cell = lst[h];
-        if (cell == 0xFFFF) continue;
-        x[cell] = (b[cell] + cta_off<DIM, M>(w + 2 * DIM * cell, x, cell, nx, nxy)) * iv[cell];
-    }
-}
-
-// Levels of at most this many cells are worked by warp 0 alone, with warp
-// barriers between their phases instead of block barriers.
-constexpr int kWarpCells = 128;
-
-// Set-up of the coarse levels in shared memory (loads and per-cell form);
-// with load_b the top level's b comes from P.b_top, else it is cleared (and
-// filled by the caller).
-template <int DIM, typename M>
-__device__ __forceinline__ void cta_prepare(const CLevels<M> &P, unsigned char *sm, bool load_b) {
-    const int t = threadIdx.x, nt = blockDim.x;
-    // 1. loads: face arrays and b of the top level asynchronously, fluid
-    //    flags directly; x (with pads) and the coarser b cleared
-    for (int l = 0; l < P.n; ++l) {
-        const CLevel<M> &L = P.L[l];
-        const GridD &g = L.g;
-        const int nf[3] = {(g.nx + 1) * g.ny * g.nz, g.nx * (g.ny + 1) * g.nz, g.nx * g.ny * (g.nz + 1)};
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            M *dst = (M *)(sm + L.os[a]);
-            for (int q = t; q < nf[a]; q += nt) CpAsync<sizeof(M)>::copy(dst + q, L.c[a] + q);
-        }
-        if (l == 0 && load_b)
-            for (int q = t; q < g.ncell; q += nt) CpAsync<sizeof(M)>::copy((M *)(sm + L.ob) + q, P.b_top + q);
-    }
-    for (int l = 0; l < P.n; ++l) {
-        const CLevel<M> &L = P.L[l];
-        const int n = L.g.ncell, pad = L.g.nx * L.g.ny;
-        for (int q = t; q < n; q += nt) (sm + L.ofl)[q] = L.fluid[q];
-        M *x = (M *)(sm + L.ox);
-        for (int q = t - pad; q < n + pad; q += nt) x[q] = M(0);
-        if (l > 0 || !load_b)
-            for (int q = t; q < n; q += nt) ((M *)(sm + L.ob))[q] = M(0);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    // 2. per-cell form
-    for (int l = 0; l < P.n; ++l) {
-        const CLevel<M> &L = P.L[l];
-        const GridD &g = L.g;
-        const uint8_t *fl = sm + L.ofl;
-        for (int q = t; q < g.ncell; q += nt) {
-            int i, j, k;
-            split3(q, g.nx, L.rnx, g.ny, L.rny, i, j, k);
-            const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
-            M *w = (M *)(sm + L.ow) + 2 * DIM * q;
-            M d = M(0);
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                const M *cc = (const M *)(sm + L.os[a]);
-                const M cl = cc[flo(g, a, i, j, k)], ch = cc[fhi(g, a, i, j, k)];
-                d += cl + ch;
-                w[2 * a] = ijk[a] > 0 ? cl : M(0);
-                w[2 * a + 1] = ijk[a] < n[a] - 1 ? ch : M(0);
-            }
-            ((M *)(sm + L.od))[q] = d;
-            ((M *)(sm + L.oi))[q] = d > M(0) ? M(1) / d : M(0);
-            ((uint32_t *)(sm + L.opk))[q] = (uint32_t)i | ((uint32_t)j << 10) | ((uint32_t)k << 20) | (fl[q] ? kPkFluid : 0u);
-        }
-        const int hx = (g.nx + 1) >> 1;
-        for (int h = t; h < L.nh; h += nt) {
-            int ti, j, k;
-            split3(h, hx, L.rhx, g.ny, L.rny, ti, j, k);
-#pragma unroll
-            for (int colour = 0; colour < 2; ++colour) {
-                const int i = 2 * ti + ((j + k + colour) & 1);
-                const int cell = i + g.nx * (j + g.ny * k);
-                ((unsigned short *)(sm + L.ol[colour]))[h] = (i < g.nx && fl[cell]) ? (unsigned short)cell : 0xFFFF;
-            }
-        }
-    }
-}
-
-// The V-cycle over the levels prepared by cta_prepare; ends with a block
-// barrier, the top level's x in shared memory.
-template <int DIM, typename M>
-__device__ __forceinline__ void cta_vcycle(const CLevels<M> &P, unsigned char *sm) {
-    const int t = threadIdx.x, nt = blockDim.x;
-    // phase bookkeeping: a block barrier wherever this or the previous phase
-    // involves the whole block, a warp barrier between two warp-0 phases
-    bool prev_blk = true;
-    int t0 = t, st = nt;
-    bool active = true;
-#define phase(L)                                                   \
-    do {                                                           \
-        const bool blk_ = (L).g.ncell > kWarpCells;                \
-        if (prev_blk || blk_) __syncthreads(); else __syncwarp();  \
-        prev_blk = blk_;                                           \
-        st = blk_ ? nt : 32;                                       \
-        active = blk_ || t < 32;                                   \
-    } while (0)
-    M *rs = (M *)(sm + P.ors);
-    for (int l = 0; l < P.n - 1; ++l) {
-        const CLevel<M> &L = P.L[l];
-        const CLevel<M> &C = P.L[l + 1];
-        const int nu = l == 0 ? P.nu_top : P.nu;
-        for (int s = 0; s < nu; ++s) {
-            phase(L); if (active) cta_sweep<DIM, M>(L, sm, 0, t0, st);
-            phase(L); if (active) cta_sweep<DIM, M>(L, sm, 1, t0, st);
-        }
-        phase(L);
-        if (active) {   // residual b - M x, cell-parallel
-            const M *x = (const M *)(sm + L.ox), *b = (const M *)(sm + L.ob), *d = (const M *)(sm + L.od);
-            const M *w = (const M *)(sm + L.ow);
-            const uint32_t *pk = (const uint32_t *)(sm + L.opk);
-            const int nx = L.g.nx, nxy = L.g.nx * L.g.ny;
-            for (int q = t0; q < L.g.ncell; q += st)
-                rs[q] = (pk[q] & kPkFluid) ? b[q] - (d[q] * x[q] - cta_off<DIM, M>(w + 2 * DIM * q, x, q, nx, nxy)) : M(0);
-        }
-        phase(L);
-        if (active) {   // restriction: sum over the children
-            const uint32_t *pkc = (const uint32_t *)(sm + C.opk);
-            M *bc = (M *)(sm + C.ob);
-            const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz;
-            for (int q = t0; q < C.g.ncell; q += st) {
-                int I, J, K;
-                pk_ijk(pkc[q], I, J, K);
-                const int i0 = I * L.r[0], j0 = J * L.r[1], k0 = K * L.r[2];
-                const int i1 = min(i0 + L.r[0], nx), j1 = min(j0 + L.r[1], ny), k1 = min(k0 + L.r[2], nz);
-                M acc = M(0);
-                for (int kk = k0; kk < k1; ++kk)
-                    for (int jj = j0; jj < j1; ++jj)
-                        for (int ii = i0; ii < i1; ++ii) acc += rs[ii + nx * (jj + ny * kk)];
-                bc[q] = acc;
-            }
-        }
-    }
-    const CLevel<M> &Lc = P.L[P.n - 1];
-    if (P.exact) {   // x = A^-1 b on the coarsest level: a warp per row, lanes over the columns
-        const int ne = Lc.g.ncell;
-        const M *inv = (const M *)(sm + P.oinv), *bc = (const M *)(sm + Lc.ob);
-        M *xc = (M *)(sm + Lc.ox);
-        __syncthreads();
-        const int lane = t & 31, warp = t >> 5, nwarp = nt >> 5;
-        for (int row = warp; row < ne; row += nwarp) {
-            M acc = M(0);
-            for (int jj = lane; jj < ne; jj += 32) acc += inv[row * ne + jj] * bc[jj];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) xc[row] = acc;
-        }
-        prev_blk = true;   // the next phase starts with a block barrier
-    } else {
-        for (int s = 0; s < P.coarse_sweeps; ++s) {
-            phase(Lc); if (active) cta_sweep<DIM, M>(Lc, sm, 0, t0, st);
-            phase(Lc); if (active) cta_sweep<DIM, M>(Lc, sm, 1, t0, st);
-        }
-        for (int s = 0; s < P.coarse_sweeps; ++s) {
-            phase(Lc); if (active) cta_sweep<DIM, M>(Lc, sm, 1, t0, st);
-            phase(Lc); if (active) cta_sweep<DIM, M>(Lc, sm, 0, t0, st);
-        }
-    }
-    for (int l = P.n - 2; l >= 0; --l) {
-        const CLevel<M> &L = P.L[l];
-        const CLevel<M> &C = P.L[l + 1];
-        phase(L);
-        if (active) {   // prolongation (piecewise constant)
-            const uint32_t *pk = (const uint32_t *)(sm + L.opk);
-            const M *xc = (const M *)(sm + C.ox);
-            M *x = (M *)(sm + L.ox);
-            const int s0 = L.r[0] >> 1, s1 = L.r[1] >> 1, s2 = L.r[2] >> 1;
-            for (int q = t0; q < L.g.ncell; q += st) {
-                const uint32_t v = pk[q];
-                if (!(v & kPkFluid)) continue;
-                int i, j, k;
-                pk_ijk(v, i, j, k);
-                x[q] += xc[(i >> s0) + C.g.nx * ((j >> s1) + C.g.ny * (k >> s2))];
-            }
-        }
-        const int nu = l == 0 ? P.nu_top : P.nu;
-        for (int s = 0; s < nu; ++s) {
-            phase(L); if (active) cta_sweep<DIM, M>(L, sm, 1, t0, st);
-            phase(L); if (active) cta_sweep<DIM, M>(L, sm, 0, t0, st);
-        }
-    }
-#undef phase
-    __syncthreads();
-}
-
-// one colour of a red-black sweep of the global-coefficient level (threads t0, t0 + st, ...)
-template <int DIM, typename M>
-__device__ __forceinline__ void gl_sweep(const GLevel<M> &G, unsigned char *sm, int colour) {
-    M *x = (M *)(sm + G.ox);
-    const M *b = (const M *)(sm + G.ob);
-    const int hx = (G.g.nx + 1) >> 1, nh = hx * G.g.ny * G.g.nz;
-    for (int h = threadIdx.x; h < nh; h += blockDim.x) {
-        int ti, j, k;
-        split3(h, hx, G.rhx, G.g.ny, G.rny, ti, j, k);
-        const int i = 2 * ti + ((j + k + colour) & 1);
-        if (i >= G.g.nx) continue;
-        const int cell = i + G.g.nx * (j + G.g.ny * k);
-        M w[2 * DIM];
-        mg_row_coeffs<DIM, M>(G.g, G.c, i, j, k, w);
-        x[cell] = (b[cell] + mg_row_off<DIM, M>(G.g, w, x, cell, i, j, k)) * G.idiag[cell];
-    }
-}
-
-// b of the CTA's first level C = the sum over its children of the fluid
-// residual b - (diag x - off) of the global-coefficient level
-template <int DIM, typename M>
-__device__ __forceinline__ void gl_restrict(const GLevel<M> &G, const CLevel<M> &C, unsigned char *sm) {
-    const M *x = (const M *)(sm + G.ox), *b = (const M *)(sm + G.ob);
-    M *bc = (M *)(sm + C.ob);
-    const uint32_t *pkc = (const uint32_t *)(sm + C.opk);
-    for (int q = threadIdx.x; q < C.g.ncell; q += blockDim.x) {
-        int I, J, K;
-        pk_ijk(pkc[q], I, J, K);
-        const int i0 = I * G.r[0], j0 = J * G.r[1], k0 = K * G.r[2];
-        const int i1 = min(i0 + G.r[0], G.g.nx), j1 = min(j0 + G.r[1], G.g.ny), k1 = min(k0 + G.r[2], G.g.nz);
-        M acc = M(0);
-        for (int kk = k0; kk < k1; ++kk)
-            for (int jj = j0; jj < j1; ++jj)
-                for (int ii = i0; ii < i1; ++ii) {
-                    const int cell = ii + G.g.nx * (jj + G.g.ny * kk);
-                    if (!G.fluid[cell]) continue;
-                    M w[2 * DIM];
-                    mg_row_coeffs<DIM, M>(G.g, G.c, ii, jj, kk, w);
-                    acc += b[cell] - (G.diag[cell] * x[cell] - mg_row_off<DIM, M>(G.g, w, x, cell, ii, jj, kk));
-                }
-        bc[q] = acc;
-    }
-}
-
-// x += the piecewise-constant prolongation of the CTA's first level's x
-template <int DIM, typename M>
-__device__ __forceinline__ void gl_prolong(const GLevel<M> &G, const CLevel<M> &C, unsigned char *sm) {
-    M *x = (M *)(sm + G.ox);
-    const M *xc = (const M *)(sm + C.ox);
-    const int s0 = G.r[0] >> 1, s1 = G.r[1] >> 1, s2 = G.r[2] >> 1;
-    for (int q = threadIdx.x; q < G.g.ncell; q += blockDim.x) {
-        int i, j, k;
-        split3(q, G.g.nx, 1.0f / (float)G.g.nx, G.g.ny, G.rny, i, j, k);
-        x[q] += xc[(i >> s0) + C.g.nx * ((j >> s1) + C.g.ny * (k >> s2))];
-    }
-}
-
-// The shared-memory image of the coarse levels (cta_prepare with x = 0 and
-// b = 0), built once per set of coefficients (once per PISO set-up) and stored
-// in global memory, so that every V-cycle starts from one contiguous copy
-// instead of redoing the loads and the per-cell rearrangement.
-// With P.exact, the pack also forms (on its first call of a step call and
-// every P.refresh-th call after it) the coarsest level's matrix (diagonal d,
-// off-diagonals -w from its per-cell form; rows of cells that are solid or
-// have no coefficients decouple) and inverts it in place by Gauss-Jordan
-// elimination without pivoting (the matrix is symmetric positive definite: the
-// fluid is connected to the Dirichlet outlet); a pivot that vanishes (a
-// fluid pocket cut off from the outlet, whose block is singular) drops its row
-// and column.
-template <int DIM, typename M>
-__global__ void __launch_bounds__(kCtaThreads, 1) k_mg_coarse_pack(CLevels<M> P, uint4 *__restrict__ img, int n16,
-                                                                   int *__restrict__ ctl) {
-    griddep_wait();
-    extern __shared__ __align__(16) unsigned char sm[];
-    // the inverse is formed on the first call of a step call and on every
-    // refresh-th one after it; in between the stored inverse is kept
-    __shared__ int invert_s;
-    if (threadIdx.x == 0) {
-        const int n = ctl[C_PACK];
-        invert_s = P.exact && (n % P.refresh == 0);
-        ctl[C_PACK] = n + 1;
-    }
-    cta_prepare<DIM, M>(P, sm, false);
-    __syncthreads();
-    const bool invert = invert_s;
-    if (invert) {
-        const CLevel<M> &Lc = P.L[P.n - 1];
-        const int ne = Lc.g.ncell, t = threadIdx.x, nt = blockDim.x;
-        M *A = (M *)(sm + P.oinv);
-        const M *d = (const M *)(sm + Lc.od), *w = (const M *)(sm + Lc.ow);
-        const uint32_t *pk = (const uint32_t *)(sm + Lc.opk);
-        const int nx = Lc.g.nx, nxy = Lc.g.nx * Lc.g.ny;
-        for (int q = t; q < ne * ne; q += nt) A[q] = M(0);
-        __syncthreads();
-        for (int c = t; c < ne; c += nt) {
-            const bool live = (pk[c] & kPkFluid) && d[c] > M(0);
-            A[c * ne + c] = live ? d[c] : M(0);
-            if (!live) continue;
-            const int offs[6] = {-1, 1, -nx, nx, -nxy, nxy};
-#pragma unroll
-            for (int f = 0; f < 2 * DIM; ++f) {
-                const M wf = w[2 * DIM * c + f];
-                const int nb = c + offs[f];
-                if (wf != M(0) && nb >= 0 && nb < ne) A[c * ne + nb] = -wf;
-            }
-        }
-        // Gauss-Jordan: thread t owns column j = t % ne and the rows g0, g0 + ng,
-        // g0 + 2 ng, ... (g0 = t / ne, ng = nt / ne groups), so a warp touches
-        // consecutive columns of one row (no bank conflicts) and reads the
-        // pivot-column entry of a row as a broadcast. Per pivot: the pivot row
-        // and column entries a thread needs go to registers, a barrier, then
-        // every owned entry gets the rank-one update and the thread fixes up
-        // its entries of the pivot row and column. The single CTA is bound by
-        // instruction issue here (n^3 updates), so the update is one FMA per
-        // entry on a strided pointer. The result is only the coarsest
-        // level's solve inside the preconditioner.
-        // rows per thread: ne / floor(nt / ne) <= 16 for ne <= 128 and nt = 1024
-        constexpr int kRows = (kExactCells * kExactCells + kCtaThreads - 1) / kCtaThreads;
-        static_assert(kRows == 16, "row bound of the Gauss-Jordan mapping");
-        const int ng = nt / ne;
-        const int j = t % ne, g0 = t / ne;
-        const int nrow = t < ng * ne ? (ne - g0 + ng - 1) / ng : 0;   // rows owned
-        const int rs = ng * ne;                                         // stride between them
-        M *const colp = A + g0 * ne + j;
-        for (int k = 0; k < ne; ++k) {
-            __syncthreads();
-            const M pv = A[k * ne + k];
-            const bool skip = !(pv > M(0));   // decoupled (or singular) row: zero row and column
-            const M inv = skip ? M(0) : M(1) / pv;
-            M aik[kRows];
-            const M *colk = A + g0 * ne + k;
-#pragma unroll
-            for (int q = 0; q < kRows; ++q) aik[q] = q < nrow ? colk[q * rs] : M(0);
-            const M akj = nrow > 0 ? A[k * ne + j] : M(0);
-            __syncthreads();
-            if (nrow == 0) continue;
-            const bool own_k = (k - g0) % ng == 0 && k >= g0;   // the pivot row is one of mine
-            const int qk = (k - g0) / ng;
-            if (skip) {
-#pragma unroll
-                for (int q = 0; q < kRows; ++q)
-                    if (q < nrow && j == k) colp[q * rs] = M(0);
-                if (own_k) colp[qk * rs] = M(0);
-                continue;
-            }
-            const M nkj = akj * inv;   // the normalised pivot-row entry
-#pragma unroll
-            for (int q = 0; q < kRows; ++q)
-                if (q < nrow) colp[q * rs] = fma(-aik[q], nkj, colp[q * rs]);
-            if (j == k) {
-#pragma unroll
-                for (int q = 0; q < kRows; ++q)
-                    if (q < nrow) colp[q * rs] = -aik[q] * inv;
-            }
-            if (own_k) colp[qk * rs] = j == k ? inv : nkj;
-        }
-        __syncthreads();
-    }
-    // the image, without the inverse's bytes when it was not formed
-    const int q0 = P.exact ? P.oinv / 16 : n16;
-    const int q1 = P.exact ? (P.oinv + P.L[P.n - 1].g.ncell * P.L[P.n - 1].g.ncell * (int)sizeof(M) + 15) / 16 : n16;
-    for (int q = threadIdx.x; q < n16; q += blockDim.x)
-        if (invert || q < q0 || q >= q1) img[q] = reinterpret_cast<const uint4 *>(sm)[q];
-}
-
-// The coarse V-cycle: the image (fixed during a solve) is copied in before the
-// grid-dependency wait, then b of the top level, written by the preceding
-// restriction, after it.
-// With P.G.active the CTA first pre-smooths the global-coefficient level and
-// restricts its residual into its first level, and after that level's
-// V-cycle prolongates back and post-smooths (see GLevel).
-template <int DIM, typename M>
-__global__ void __launch_bounds__(kCtaThreads, 1) k_mg_coarse(CLevels<M> P, const uint4 *__restrict__ img, int n16) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    // every 16-byte piece of the image in flight at once (asynchronous copies)
-    for (int q = threadIdx.x; q < n16; q += blockDim.x) CpAsync<16>::copy(sm + 16 * (size_t)q, img + q);
-    cp_async_wait_all();
-    const GLevel<M> &G = P.G;
-    if (G.active) {   // x of the level starts at 0
-        M *gx = (M *)(sm + G.ox);
-        for (int q = threadIdx.x; q < G.g.ncell; q += blockDim.x) gx[q] = M(0);
-    }
-    griddep_wait();
-    if (G.active) {
-        M *gb = (M *)(sm + G.ob);
-        for (int q = threadIdx.x; q < G.g.ncell; q += blockDim.x) gb[q] = G.b_glob[q];
-        for (int s = 0; s < G.nu; ++s) {
-            __syncthreads();
-            gl_sweep<DIM, M>(G, sm, 0);
-            __syncthreads();
-            gl_sweep<DIM, M>(G, sm, 1);
-        }
-        __syncthreads();
-        gl_restrict<DIM, M>(G, P.L[0], sm);
-    } else {
-        M *bt = (M *)(sm + P.L[0].ob);
-        for (int q = threadIdx.x; q < P.L[0].g.ncell; q += blockDim.x) bt[q] = P.b_top[q];
-    }
-    __syncthreads();
-    cta_vcycle<DIM, M>(P, sm);
-    if (G.active) {
-        gl_prolong<DIM, M>(G, P.L[0], sm);
-        for (int s = 0; s < G.nu; ++s) {
-            __syncthreads();
-            gl_sweep<DIM, M>(G, sm, 1);
-            __syncthreads();
-            gl_sweep<DIM, M>(G, sm, 0);
-        }
-        __syncthreads();
-        const M *gx = (const M *)(sm + G.ox);
-        for (int q = threadIdx.x; q < G.g.ncell; q += blockDim.x) G.x_glob[q] = gx[q];
-    } else {
-        for (int q = threadIdx.x; q < P.L[0].g.ncell; q += blockDim.x) P.x_top[q] = ((const M *)(sm + P.L[0].ox))[q];
-    }
 }
 
 }  // namespace oscar

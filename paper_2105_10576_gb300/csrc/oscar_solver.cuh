@@ -13,7 +13,7 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include "oscar_kernels.cuh"
+#include "oscar_cluster.cuh"
 
 namespace oscar {
 
@@ -36,19 +36,31 @@ inline int nblk(long long n) { return (int)((n + BS - 1) / BS); }
 
 // Kernel launch with programmatic stream serialization: the next kernel's
 // launch overlaps the tail of this one (each kernel waits in griddep_wait()).
+// nc > 1: a cluster of that many CTAs. pdl = false: full dependencies (the
+// first kernel after a fork or a join of streams).
 template <typename... KArgs, typename... Args>
-inline void launchk(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+inline void launchx(bool pdl, int nc, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                    Args &&...args) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (nc > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)nc;
+        attr[na].val.clusterDim.y = attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = na;
     if (Profiler *P = t_prof) {   // in-step timing (eager steps only; never while capturing)
         int slot = prof_begin(P, st, (const void *)kern, grid, block);
         cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
@@ -56,6 +68,10 @@ inline void launchk(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, 
     } else {
         cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
     }
+}
+template <typename... KArgs, typename... Args>
+inline void launchk(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    launchx(true, 1, kern, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -157,6 +173,21 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
     }
 }
 
+// Which levels and grids go to a cluster, and of how many CTAs. The V-cycle's
+// cluster takes levels of at most vcycle_cells x cta_cells cells (default 8192
+// in FP32: 16 SMs then work about 512 cells each, where a launch per half sweep
+// is still bound by its latency; in FP64 they are bound by FP64 issue above
+// 1024 cells). A 2D grid of at most solve_cells is solved whole in one cluster
+// when its vectors fit the shared memory.
+constexpr int kVcycleCtas = 16, kVcycleThreads = 512, kSolveCtas = 16, kSolveThreads = 256;
+template <typename T> struct ClRule;
+template <> struct ClRule<float> {
+    static constexpr long long vcycle_cells = 8, solve_cells = 65536;
+};
+template <> struct ClRule<double> {
+    static constexpr long long vcycle_cells = 1, solve_cells = 16384;
+};
+
 template <typename T> struct Impl {
     using M = T;
     using V = T;
@@ -223,104 +254,126 @@ template <typename T> struct Impl {
     // --- multigrid -----------------------------------------------------------
     static MG3<M> mg3(const Level &L) { MG3<M> c; for (int a = 0; a < 3; ++a) c.a[a] = (const M *)L.c[a]; return c; }
 
+    // operators of every level and the coarsest one's inverse, on stream st
     template <int DIM>
-    static int mg_coeffs_d(Instance &I) {
+    static int mg_coeffs_d(Instance &I, cudaStream_t st) {
         for (int l = 0; l < I.nlev; ++l) {
             Level &L = I.lev[l];
             GridD g = to_dev(L.g);
             L3 LL = launch3(L.g);
             if (l == 0) {
-                launchk(k_mg_diag<DIM, M>, LL.grid, LL.block, 0, I.stream, g, L.fluid, mg3(L), (M *)L.diag,
+                launchx(false, 1, k_mg_diag<DIM, M>, LL.grid, LL.block, 0, st, g, L.fluid, mg3(L), (M *)L.diag,
                         (M *)L.idiag), ++I.nlaunch;
             } else {
                 Level &F = I.lev[l - 1];
                 P3<M> cc;
                 for (int a = 0; a < 3; ++a) cc.a[a] = (M *)L.c[a];
-                launchk(k_mg_level_operator<DIM, M>, LL.grid, LL.block, 0, I.stream, to_dev(F.g), g, F.r[0], F.r[1],
+                launchk(k_mg_level_operator<DIM, M>, LL.grid, LL.block, 0, st, to_dev(F.g), g, F.r[0], F.r[1],
                         F.r[2], mg3(F), cc, (const uint8_t *)L.fluid, (M *)L.diag, (M *)L.idiag), ++I.nlaunch;
             }
         }
-        {   // the coarse CTA's shared-memory image for this set of coefficients
-            CLevels<M> P;
-            cta_levels(I, P, I.lc0);
-            launchk(k_mg_coarse_pack<DIM, M>, 1, kCtaThreads, I.cta_img_bytes, I.stream, P, (uint4 *)I.cta_img,
-                    (int)(I.cta_img_bytes / 16), I.ctl), ++I.nlaunch;
-        }
+        const Level &E = I.lev[exact_level(I, top_level(I))];
+        if constexpr (sizeof(M) == sizeof(float))
+            launchk(k_mg_inverse_dense<DIM>, 1, kGjThreads, 0, st, to_dev(E.g), mg3(E), (const M *)E.diag,
+                    (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, I.ctl), ++I.nlaunch;
+        else
+            launchk(k_mg_inverse_band<DIM, M>, 1, 128, inverse_smem(E.g), st, to_dev(E.g), mg3(E), (const M *)E.diag,
+                    (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, I.ctl), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
         return 0;
     }
 
-    // levels l0.. of the single-CTA coarse kernel with their shared-memory
-    // layout; returns the bytes of shared memory they need
-    static size_t cta_levels(Instance &I, CLevels<M> &P, int l0, size_t base = 0, bool allow_exact = true) {
-        memset(&P.G, 0, sizeof(P.G));
-        P.n = I.nlev - l0;
-        P.exact = 0;
-        P.oinv = 0;
-        P.refresh = I.coarse_refresh;
-        if (allow_exact)   // stop at the first level small enough for an exact solve
-            for (int q = 0; q < P.n; ++q)
-                if (I.lev[l0 + q].g.ncell <= kExactCells) { P.n = q + 1; P.exact = 1; break; }
-        P.nu = I.mg_nu_cta;
-        P.nu_top = l0 == 0 ? I.mg_nu : I.mg_nu_cta;
-        P.coarse_sweeps = I.mg_coarse_sweeps;
-        size_t off = base;
-        auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 15) & ~(size_t)15; return (int)o; };
-        size_t nmax = 0;
-        for (int q = 0; q < P.n && q < kMaxCL; ++q) {
-            Level &L = I.lev[l0 + q];
-            CLevel<M> &C = P.L[q];
-            C.g = to_dev(L.g);
-            for (int a = 0; a < 3; ++a) C.c[a] = (const M *)L.c[a];
-            C.fluid = L.fluid;
-            for (int a = 0; a < 3; ++a) C.r[a] = L.r[a];
-            C.rnx = 1.0f / (float)L.g.nx;
-            C.rny = 1.0f / (float)L.g.ny;
-            C.rhx = 1.0f / (float)((L.g.nx + 1) / 2);
-            C.nh = ((L.g.nx + 1) / 2) * L.g.ny * L.g.nz;
-            size_t n = L.g.ncell, pad = (size_t)L.g.nx * L.g.ny, dim = L.g.dim;
-            nmax = n > nmax ? n : nmax;
-            C.ox = take((n + 2 * pad) * sizeof(M)) + (int)(pad * sizeof(M));
-            C.ob = take(n * sizeof(M));
-            C.od = take(n * sizeof(M));
-            C.oi = take(n * sizeof(M));
-            C.ow = take(2 * dim * n * sizeof(M));
-            C.opk = take(n * sizeof(uint32_t));
-            C.ol[0] = take(C.nh * sizeof(unsigned short));
-            C.ol[1] = take(C.nh * sizeof(unsigned short));
-            C.ofl = take(n);
-            for (int a = 0; a < 3; ++a) C.os[a] = take(a < L.g.dim ? (size_t)L.g.nf[a] * sizeof(M) : 0);
-        }
-        P.ors = take(nmax * sizeof(M));
-        if (P.exact) {
-            const int ne = I.lev[l0 + P.n - 1].g.ncell;
-            P.oinv = take((size_t)ne * ne * sizeof(M));
-        }
-        return P.n > kMaxCL ? (size_t)-1 : off;
+    // --- the cluster's levels ------------------------------------------------
+    // first level worked by the V-cycle's cluster
+    static int top_level(const Instance &I) { return I.lg >= 0 ? I.lg : I.lc0; }
+    // the level solved with its explicit inverse below level l0
+    static int exact_level(const Instance &I, int l0) {
+        int l = l0;
+        while (l < I.nlev - 1 && I.lev[l].g.ncell > kExactCells) ++l;
+        return l;
+    }
+    static size_t inverse_smem(const GridH &g) {
+        int e[3] = {g.nx, g.ny, g.nz};
+        std::sort(e, e + 3);
+        const size_t n = g.ncell;
+        return (kExactCells * (size_t)(e[0] * e[1] + 1) + n * n) * sizeof(M);
     }
 
-    // the global-coefficient level lg of the coarse CTA, its x and b placed in
-    // shared memory after the image of the CTA's levels
-    static void gl_fill(Instance &I, CLevels<M> &P, int lg) {
-        GLevel<M> &G = P.G;
-        const Level &L = I.lev[lg];
-        G.active = 1;
-        G.g = to_dev(L.g);
-        G.c = mg3(L);
-        G.diag = (const M *)L.diag;
-        G.idiag = (const M *)L.idiag;
-        G.fluid = L.fluid;
-        for (int a = 0; a < 3; ++a) G.r[a] = L.r[a];
-        G.rhx = 1.0f / (float)((L.g.nx + 1) / 2);
-        G.rny = 1.0f / (float)L.g.ny;
-        const size_t base = (I.cta_img_bytes + 15) & ~(size_t)15;
-        G.ox = (int)base;
-        G.ob = (int)(base + (((size_t)L.g.ncell * sizeof(M) + 15) & ~(size_t)15));
-        G.nu = I.mg_nu_c;
-    }
-    static size_t gl_bytes(const Instance &I, int lg, size_t img) {
-        const size_t n = (size_t)I.lev[lg].g.ncell * sizeof(M);
-        return ((img + 15) & ~(size_t)15) + 2 * ((n + 15) & ~(size_t)15);
+    // Levels l0 .. of a cluster of at most nc_max CTAs and their shared-memory
+    // layout; returns the bytes each CTA needs, (size_t)-1 when the levels
+    // cannot be worked by a cluster. With A the vectors of a whole solve are
+    // laid out too.
+    static size_t cl_fill(const Instance &I, ClLevels<M> &P, int l0, int nc_max, ClSolve *A = nullptr) {
+        memset(&P, 0, sizeof(P));
+        const int le = exact_level(I, A ? top_level(I) : l0);   // one inverse serves both kernels
+        P.n = le - l0 + 1;
+        if (P.n > kMaxCL || I.lev[le].g.ncell > kExactCells) return (size_t)-1;
+        P.cols = I.lev[le].g.nx;
+        P.nc = 1;
+        while (2 * P.nc <= nc_max && 2 * P.nc <= P.cols) { P.nc *= 2; ++P.lnc; }
+        P.inv = (const M *)I.cl_inv;
+        size_t off = 0, rs = 0;
+        auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 15) & ~(size_t)15; return (int)o; };
+        int w[kMaxCL], sh = 0;
+        for (int q = P.n - 1; q >= 0; --q) {   // slabs, from the coarsest level
+            const Level &L = I.lev[l0 + q];
+            if (q < P.n - 1 && L.r[0] == 2) ++sh;
+            P.L[q].sh = sh;
+            w[q] = 0;
+            for (int r = 0; r < P.nc; ++r) {
+                const int s0 = std::min(((r * P.cols) >> P.lnc) << sh, L.g.nx);
+                const int s1 = std::min((((r + 1) * P.cols) >> P.lnc) << sh, L.g.nx);
+                w[q] = std::max(w[q], s1 - s0);
+            }
+        }
+        int E = A ? 1 : 0;   // a solve applies the operator to z
+        for (int q = 0; q < P.n; ++q) {
+            const Level &L = I.lev[l0 + q];
+            ClLevel<M> &C = P.L[q];
+            const bool last = q == P.n - 1;
+            C.nx = L.g.nx; C.ny = L.g.ny; C.nz = L.g.nz;
+            C.rx = L.r[0]; C.ry = L.r[1]; C.rz = L.r[2];
+            C.paired = l0 + q >= I.lc0;
+            C.nu = l0 + q == 0 ? I.mg_nu : (l0 + q < I.lc0 ? I.mg_nu_c : I.mg_nu_cta);
+            C.E = E;
+            C.D = last ? E : E + 4 * C.nu - 2;
+            // the ghosts held: at most the whole domain, at least the column beyond it
+            C.G = P.nc == 1 ? 1 : std::min(C.nx, std::max(1, C.D));
+            E = (E + 2 * C.nu + C.rx - 1) / C.rx;
+            C.ncol = w[q] + 2 * C.G;
+            C.ps = (C.ny * C.nz) | 1;
+            const size_t n = (size_t)C.ncol * C.ps;
+            if (n > 65534) return (size_t)-1;   // list entries hold 16-bit cell numbers
+            C.nloc = (int)n;
+            C.ce = ((C.ny + 1) / 2) * C.nz;
+            C.rncol = 1.0f / (float)C.ncol;
+            C.rny = 1.0f / (float)C.ny;
+            C.rhj = 1.0f / (float)((C.ny + 1) / 2);
+            for (int a = 0; a < 3; ++a) C.c[a] = (const M *)L.c[a];
+            C.idiag = (const M *)L.idiag;
+            C.ox = take(n * sizeof(M));
+            C.ob = take(n * sizeof(M));
+            C.oi = take(n * sizeof(M));
+            for (int a = 0; a < L.g.dim; ++a) C.oc[a] = take(n * sizeof(M));
+            const size_t nh = (size_t)C.ncol * C.ce * sizeof(unsigned short);
+            C.ol[0] = take(nh);
+            C.ol[1] = take(nh);
+            if (!last) C.op = take(nh);
+            if (!last) rs = std::max(rs, (size_t)w[q] * C.ps);
+        }
+        const ClLevel<M> &Lc = P.L[P.n - 1];
+        const size_t ne = I.lev[le].g.ncell;
+        P.ors = take(rs * sizeof(M));
+        P.obx = take(ne * sizeof(M));
+        P.oinv = take(std::min((size_t)Lc.ncol * Lc.ny * Lc.nz, ne) * ne * sizeof(M));
+        if (A) {
+            P.ored = take((512 + 2 * 4 * kMaxCluster) * sizeof(double));
+            const size_t n = (size_t)(w[0] + 2) * P.L[0].ps;
+            A->op = take(n * sizeof(M));
+            A->oap = take(n * sizeof(M));
+            A->oe = sizeof(M) == sizeof(float) ? take(n * sizeof(M)) : A->oap;
+        }
+        return off;
     }
 
     // x / b of level l (level 0 works in place on the Krylov vectors z / r)
@@ -379,13 +432,13 @@ template <typename T> struct Impl {
     }
 
     // z = V-cycle(r): pre-smoothing red-black, post-smoothing black-red
-    // (symmetric, so a valid CG preconditioner); levels from lc0 down run in
-    // one CTA. The first colour-0 half sweep of each level above the CTA is
+    // (symmetric, so a valid CG preconditioner); levels from top_level down run
+    // in one cluster. The first colour-0 half sweep of each level above it is
     // done by the kernel that produces its right-hand side (k_cg_init /
     // k_cg_update for the finest level, the restriction for the others).
     template <int DIM>
     static int vcycle_d(Instance &I, V *r, V *z) {
-        const int lk = I.lg >= 0 ? I.lg : I.lc0;   // first level not worked by per-level kernels
+        const int lk = top_level(I);   // first level not worked by per-level kernels
         for (int l = 0; l < lk; ++l) {
             Level &L = I.lev[l], &C = I.lev[l + 1];
             M *x = lx(I, l, z), *b = lb(I, l, r);
@@ -397,17 +450,10 @@ template <typename T> struct Impl {
             resid_restrict<DIM>(I, L, C, x, b, lb(I, l + 1, r), lx(I, l + 1, z), l + 1 < lk ? 1 : 0);
         }
         {
-            CLevels<M> P;
-            cta_levels(I, P, I.lc0);
-            P.b_top = lb(I, I.lc0, r);
-            P.x_top = lx(I, I.lc0, z);
-            if (I.lg >= 0) {
-                gl_fill(I, P, I.lg);
-                P.G.b_glob = lb(I, I.lg, r);
-                P.G.x_glob = lx(I, I.lg, z);
-            }
-            launchk(k_mg_coarse<DIM, M>, 1, kCtaThreads, I.cta_smem, I.stream, P, (const uint4 *)I.cta_img,
-                    (int)(I.cta_img_bytes / 16)), ++I.nlaunch;
+            ClLevels<M> P;
+            cl_fill(I, P, lk, I.cl_nc);
+            launchx(true, P.nc, k_mg_cluster<DIM, M>, P.nc, kVcycleThreads, I.cl_smem, I.stream, P,
+                    (const M *)lb(I, lk, r), lx(I, lk, z)), ++I.nlaunch;
         }
         for (int l = lk - 1; l >= 0; --l) {
             M *x = lx(I, l, z), *b = lb(I, l, r);
@@ -444,7 +490,7 @@ template <typename T> struct Impl {
         V *r = (V *)I.cg_r, *z = (V *)I.cg_z, *p = (V *)I.cg_p, *Ap = (V *)I.cg_Ap;
         long long n0 = I.nlaunch;
         OSCAR_TRY(vcycle_d<DIM>(I, r, z));
-        if (I.lc0 == 0)   // the whole V-cycle ran in the coarse CTA: r.z on its own
+        if (top_level(I) == 0)   // the whole V-cycle ran in the cluster: r.z on its own
             launchk(k_cg_dot_rz<V>, kRedBlocks, BS, 0, I.stream, n, r, z, I.partials, I.ticket, I.scal), ++I.nlaunch;
         if constexpr (sizeof(V) == sizeof(float)) {
             L3 LA = launch_rpt(I.g, kApplyRows);
@@ -470,8 +516,27 @@ template <typename T> struct Impl {
     // defect correction around an FP32 PCG for the correction e.
     template <int DIM>
     static int pcg_d(Instance &I, double *q, const double *b, bool with_E) {
-        size_t nbytes = (size_t)I.g.ncell * sizeof(V);
-        (void)nbytes;
+        if (DIM == 2 && I.solve_nc) {
+            ClLevels<M> P;
+            ClSolve A;
+            memset(&A, 0, sizeof(A));
+            cl_fill(I, P, 0, I.solve_nc, &A);
+            A.g = to_dev(I.g);
+            A.info = I.info;
+            A.w64 = w64(I);
+            A.q = q;
+            A.b = b;
+            A.r64 = I.cg_r64;
+            A.scal = I.scal;
+            A.ctl = I.ctl;
+            A.rtol = I.P.cg_rtol;
+            A.inv_nf = with_E ? 1.0 / (double)I.n_fluid : 0.0;
+            A.maxit = I.P.cg_maxit;
+            A.by = (int)launch3(I.g).block.y;
+            launchx(!with_E, P.nc, k_solve_cluster<T>, P.nc, kSolveThreads, I.solve_smem, I.stream, P, A), ++I.nlaunch;
+            OSCAR_LAUNCH_CHECK();
+            return 0;
+        }
         if constexpr (sizeof(T) == sizeof(double)) {
             cudaGraphConditionalHandle h;
             OSCAR_TRY(cond_handle(I, &h));
@@ -524,7 +589,12 @@ template <typename T> struct Impl {
             launchk(k_face_coeffs<2, T>, F[2].grid, F[2].block, 0, I.stream, g, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
                                                                         tp(cf[2]), tp(I.fst[2]), cf64_out(I, 2)), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
-        OSCAR_TRY(mg_coeffs_d<DIM>(I));
+        // the multigrid operators are first needed by the solve: they are built
+        // on a branch beside the first momentum prediction
+        if (cudaEventRecord(I.ev_fork, I.stream) != cudaSuccess || cudaStreamWaitEvent(I.aux, I.ev_fork, 0) != cudaSuccess)
+            return OSCAR_E_CUDA;
+        OSCAR_TRY(mg_coeffs_d<DIM>(I, I.aux));
+        if (cudaEventRecord(I.ev_join, I.aux) != cudaSuccess) return OSCAR_E_CUDA;
         P3<T> Gp0 = p3(&I.G[0]), Gp1 = p3(&I.G[3]), Gp2 = p3(&I.G[6]);
         C3<T> Gc0 = c3(&I.G[0]), Gc1 = c3(&I.G[3]), Gc2 = c3(&I.G[6]);
         for (int corr = 0; corr < I.P.n_piso; ++corr) {
@@ -536,9 +606,12 @@ template <typename T> struct Impl {
                     (T)vin0, p3(I.phis), I.cg_b), ++I.nlaunch;
             // E_k, the normalised initial residual of the first corrector
             // (Section 3.2), is formed by the solve's initial-residual kernel
-            if (corr == 0)
-                launchk(k_sum_to<double>, kRedBlocks, BS, 0, I.stream, g.ncell, q, 1.0, I.partials, I.ticket, I.scal,
-                                                                  S_QSUM), ++I.nlaunch;
+            if (corr == 0) {
+                if (cudaStreamWaitEvent(I.stream, I.ev_join, 0) != cudaSuccess) return OSCAR_E_CUDA;
+                if (!(DIM == 2 && I.solve_nc))   // the one-launch solve sums q itself
+                    launchx(false, 1, k_sum_to<double>, kRedBlocks, BS, 0, I.stream, g.ncell, q, 1.0, I.partials,
+                            I.ticket, I.scal, S_QSUM), ++I.nlaunch;
+            }
             OSCAR_LAUNCH_CHECK();
             OSCAR_TRY(pcg_d<DIM>(I, q, I.cg_b, corr == 0));
             launchk(k_correct<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.phis), c3(cf), q, p3(phi),
@@ -761,6 +834,7 @@ template <typename T> struct Impl {
 };
 
 template <typename T> void Solver<T>::release_graphs(Instance &I) {
+    I.n_cg_body = I.n_outer_body = 0;   // set again by the next capture
     for (int k = 0; k < 3; ++k) {
         GraphSlot &G = I.gslot[k];
         if (G.valid) {
@@ -771,29 +845,37 @@ template <typename T> void Solver<T>::release_graphs(Instance &I) {
     }
 }
 
-// The coarse CTA takes the levels of at most `cap` cells (at most 1024: one
-// per thread) whose subtree fits the shared-memory budget.
+// The cluster takes the levels of at most `cap` cells whose subtree fits its
+// shared memory; with cta_global it has several CTAs and takes the levels of
+// at most kVcycleCells * cap cells (never the finest one, whose x and b are the
+// Krylov vectors), and a small 2D grid's whole solve runs in one cluster.
 template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
-    CLevels<T> P;
-    const size_t budget = kCtaImageBytes;
+    ClLevels<T> P;
+    const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
+    const int nc = I.cta_global ? kVcycleCtas : 1;
+    const int keep = I.lc0;
+    auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
     int lc0 = I.nlev - 1;
-    while (lc0 > 0 && I.lev[lc0 - 1].g.ncell <= cap && Impl<T>::cta_levels(I, P, lc0 - 1) <= budget) --lc0;
-    const size_t sm = Impl<T>::cta_levels(I, P, lc0);
-    if (sm > budget) return OSCAR_E_INVALID_ARG;
-    I.lc0 = lc0;
-    I.cta_img_bytes = (sm + 15) & ~(size_t)15;
-    I.cta_smem = I.cta_img_bytes;
-    I.lg = -1;
-    // the level above may join the CTA with its coefficients in global memory
-    // when its x and b fit beside the image (never the finest level, whose x
-    // and b are the Krylov vectors of the CG kernels)
-    if (I.cta_global && lc0 - 1 >= 1 && I.lev[lc0 - 1].g.ncell <= kGlCells) {
-        const size_t tot = Impl<T>::gl_bytes(I, lc0 - 1, I.cta_img_bytes);
-        if (tot <= budget) {
-            I.lg = lc0 - 1;
-            I.cta_smem = tot;
-        }
+    for (;;) {   // the layout depends on which levels take mg_nu_cta sweeps
+        I.lc0 = lc0;
+        if (!fits(lc0)) break;
+        if (lc0 == 0 || I.lev[lc0 - 1].g.ncell > cap) { --lc0; break; }
+        --lc0;
+    }
+    I.lc0 = ++lc0;   // the last one that fitted
+    if (lc0 == I.nlev) { I.lc0 = keep; return OSCAR_E_INVALID_ARG; }
+    int lg = lc0;
+    if (I.cta_global)
+        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1)) --lg;
+    I.lg = lg < lc0 ? lg : -1;
+    I.cl_smem = Impl<T>::cl_fill(I, P, lg, nc);
+    I.cl_nc = P.nc;
+    I.solve_nc = 0;
+    if (I.cta_global && I.g.dim == 2 && I.g.ncell <= ClRule<T>::solve_cells) {
+        ClSolve A;
+        I.solve_smem = Impl<T>::cl_fill(I, P, 0, kSolveCtas, &A);
+        if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) I.solve_nc = P.nc;   // even slab starts
     }
     return 0;
 }
@@ -814,20 +896,17 @@ template <typename T> int Solver<T>::setup(Instance &I, const uint8_t *solid_dev
     }
     OSCAR_LAUNCH_CHECK();
     OSCAR_TRY(choose_cta(I, I.cta_cells));
-    const size_t budget = kCtaImageBytes;
-    // the attribute belongs to the kernel, not to this instance: it is set to
-    // the budget (never lowered), so that instances of other sizes, created
-    // while this one runs, cannot shrink it below what this one launches with
-    cudaError_t e = I.g.dim == 3 ? cudaFuncSetAttribute(k_mg_coarse<3, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        (int)budget)
-                                 : cudaFuncSetAttribute(k_mg_coarse<2, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        (int)budget);
-    if (e == cudaSuccess)
-        e = I.g.dim == 3 ? cudaFuncSetAttribute(k_mg_coarse_pack<3, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)budget)
-                         : cudaFuncSetAttribute(k_mg_coarse_pack<2, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)budget);
-    if (e != cudaSuccess) return OSCAR_E_CUDA;
+    // the attributes belong to the kernels, not to this instance: they are set
+    // to the budget (never lowered), so that instances of other sizes, created
+    // while this one runs, cannot shrink them below what this one launches with
+    const void *inv = I.g.dim == 3 ? (const void *)k_mg_inverse_band<3, T> : (const void *)k_mg_inverse_band<2, T>;
+    const void *vcy = I.g.dim == 3 ? (const void *)k_mg_cluster<3, T> : (const void *)k_mg_cluster<2, T>;
+    const void *sol = (const void *)k_solve_cluster<T>;
+    for (const void *f : {inv, vcy, sol}) {
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return OSCAR_E_CUDA;
+    }
     int rc = Impl<T>::interface_(I, I.alpha);
     I.nexec += I.nlaunch - l0;
     return rc;
