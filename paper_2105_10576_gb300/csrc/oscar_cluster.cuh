@@ -484,29 +484,14 @@ __device__ __forceinline__ void cl_sum(const ClLevels<M> &P, unsigned char *sm, 
     buf ^= 1;
 }
 // the same for one value of the vectors' type: FP64 as above, FP32 in
-// compensated pairs (reduce_last_sum); the total is valid in thread 0
-struct ClAcc64 {          // a thread's sum of group values
-    double s = 0.0;
-    __device__ __forceinline__ void add(double v) { s += v; }
-};
-struct ClAcc32 {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        float sn, se;
-        two_sum(s, v, sn, se);
-        s = sn;
-        e += se;
-    }
-};
-template <typename T> struct ClAcc { using type = ClAcc64; };
-template <> struct ClAcc<float> { using type = ClAcc32; };
+// compensated pairs; the total is valid in thread 0
 template <typename M>
-__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, ClAcc64 a) {
+__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc64 a) {
     cl_sum(P, sm, rank, buf, &a.s, 1);
     return a.s;
 }
 template <typename M>
-__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, ClAcc32 a) {
+__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc32 a) {
     float2 *slot = (float2 *)((double *)(sm + P.ored) + 512 + buf * 4 * kMaxCluster);
     const int t = threadIdx.x;
     float s = a.s, e = a.e;
@@ -628,7 +613,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
         do {
             cl_vcycle<2, T>(P, sm, rank);
             __syncthreads();
-            typename ClAcc<T>::type dz;   // r.z: a colour-0 cell with its row partner (level 0 on its own: cell by cell)
+            typename DotAcc<T>::type dz;   // r.z: a colour-0 cell with its row partner (level 0 on its own: cell by cell)
             for (int g = t; g < ((S.w + 1) >> 1) * L.ny; g += blockDim.x) {
                 const int tp = g / L.ny, j = g - tp * L.ny, lo = (2 * tp + L.G) * ps + j, odd = (S.s + j) & 1;
                 const bool two = 2 * tp + 1 < S.w;
@@ -646,7 +631,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
                 K.beta_f = (float)K.beta;
             }
             __syncthreads();
-            typename ClAcc<T>::type dp;
+            typename DotAcc<T>::type dp;
             const T *c0 = (const T *)(sm + L.oc[0]), *c1 = (const T *)(sm + L.oc[1]);
             if constexpr (MIXED) {   // p = z + beta p, Ap = M z + beta Ap, p.Ap
                 const T be = K.beta_f;
@@ -693,7 +678,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             }
             __syncthreads();
             const T al = MIXED ? (T)K.alpha_f : (T)K.alpha;
-            typename ClAcc<T>::type dr;
+            typename DotAcc<T>::type dr;
             CL_ROW_GROUPS(kUpdateRows) {   // x += alpha p, r -= alpha Ap, r.r
                 T a = T(0);
 #pragma unroll

@@ -19,7 +19,7 @@ constexpr size_t kClInvBytes = 128 * 128 * sizeof(double);   // explicit inverse
 // Scalar slots in the device scalar array (double).
 enum Slot {
     S_BB = 0, S_RR, S_RZ0, S_RZ1, S_PAP, S_QSUM, S_RES, S_NRM, S_DUMAX, S_VOL, S_TARGET, S_E, S_DU, S_TEST,
-    S_ITARGET, S_ALPHA, S_BETA, S_ALPHA_F, S_BETA_F, S_TMP, S_AREA0, S_AREA1, S_COUNT
+    S_ITARGET, S_AREA0, S_AREA1, S_COUNT
 };
 
 // Integer control words on the device (relaxation and PCG loop state).
@@ -122,6 +122,7 @@ struct Instance {
     Level lev[kMaxLevels];
     // reductions
     double *partials;      // kRedSlots * red_stride
+    int nrz;               // partials of r.z left by the last kernel that formed them (while issuing a step)
     int red_stride;        // partials per slot: max(kRedBlocks, blocks of a cell launch)
     int lc0;               // first multigrid level of at most cta_cells cells
     int lg;                // first of the levels above lc0 that the cluster works too, -1 when none
@@ -164,7 +165,6 @@ struct Instance {
     int depth;             // current nesting depth while capturing
     int capturing;
     long long n_cg_body;   // kernels per PCG iteration
-    long long n_outer_body; // kernels per defect-correction trip outside the PCG body
     long long cg_bodies_captured;
     int *ctl;              // device control words
     int *ctl_host;         // pinned: initial control words (read by the graph) and read-back

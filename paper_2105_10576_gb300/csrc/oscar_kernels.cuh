@@ -133,6 +133,21 @@ inline L3 launch_rpt(const GridH &g, int rpt) {
     return l;
 }
 
+// launch_rpt with at most about kDotBlocks blocks: a block takes the row
+// groups blockIdx.y, blockIdx.y + gridDim.y, ... (at most gy of them)
+constexpr int kDotBlocks = 608;   // 152 SMs x 4
+struct L3G : L3 { int groups; };
+inline L3G launch_groups(int nx, int rows, int rpt) {
+    L3G l;
+    static_cast<L3 &>(l) = launch3(nx, rows, 1);
+    const int by = (int)l.block.y, gx = (int)l.grid.x;
+    l.groups = (rows + by * rpt - 1) / (by * rpt);
+    const int m = std::max(1, (int)(((long long)l.groups * gx + kDotBlocks - 1) / kDotBlocks));
+    l.grid = dim3(gx, (l.groups + m - 1) / m, 1);
+    l.nblocks = (int)(l.grid.x * l.grid.y);
+    return l;
+}
+
 // Row loop of the stencil reductions (launch_rows): the thread at x = i takes
 // every (gridDim.y * blockDim.y)-th row, row = j + ny k, so that a thread sums
 // several cells before the block reduction.
@@ -248,20 +263,6 @@ __device__ __forceinline__ void block_pair_f(float &s, float &e) {
         warp_sum_pair(s, e);
     }
 }
-// CG scalars: the finishing block stores alpha / beta in FP64 and an FP32
-// copy in the slot's f-twin, so FP32 kernels read them without FP64 work
-__device__ __forceinline__ void put_scalar(double *scal, int slot, int fslot, double v) {
-    scal[slot] = v;
-    *reinterpret_cast<float *>(scal + fslot) = (float)v;
-}
-template <typename V> __device__ __forceinline__ V get_scalar(const double *scal, int slot, int fslot);
-template <> __device__ __forceinline__ float get_scalar<float>(const double *scal, int, int fslot) {
-    return *reinterpret_cast<const float *>(scal + fslot);
-}
-template <> __device__ __forceinline__ double get_scalar<double>(const double *scal, int slot, int) {
-    return scal[slot];
-}
-
 __device__ __forceinline__ bool block_leader() { return threadIdx.x == 0 && threadIdx.y == 0; }
 
 // Single-pass reduction: every block stores its partial(s); the block that
@@ -336,51 +337,59 @@ __device__ __forceinline__ bool reduce_last4(double *v, int nv, double *__restri
     return true;
 }
 
-// reduce_last for one sum of FP32 thread values (compensated block sums,
-// FP64 across blocks); the total is returned in v (all threads of the last
-// block). An FP64 value goes through reduce_last.
-__device__ __forceinline__ bool reduce_last_sum(float v, double &out, double *__restrict__ part,
-                                                unsigned *__restrict__ ticket, int nb) {
-    // block partials stay compensated pairs (stored as float2 in the FP64
-    // partial slots) and the finishing block sums them the same way, so the
-    // whole reduction runs in FP32 instructions up to the final FP64 sum
-    float s = v, e = 0.f;
-    block_pair_f(s, e);
-    __shared__ int last_f;
-    __shared__ double tot_f;
-    if (block_leader()) {
-        reinterpret_cast<float2 *>(part)[BLOCK_ID()] = make_float2(s, e);
-        __threadfence();
-        unsigned t = atomicAdd(ticket, 1u);
-        last_f = (t == (unsigned)(nb - 1)) ? 1 : 0;
-    }
-    __syncthreads();
-    if (!last_f) return false;
-    __threadfence();
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
-    float as = 0.f, ae = 0.f;
-    for (int q = tid; q < nb; q += nt) {
-        const float2 pv = __ldcg(reinterpret_cast<const float2 *>(part) + q);
+// Dot products of the CG. A thread sums groups of cells in the vectors' type
+// (the groups of its kernel) and the groups in compensated pairs (FP32) or
+// plainly (FP64); a block stores one partial and ends. The kernel that needs
+// the total sums the partials itself, every block in the same order, beside
+// its own loads. That leaves out a finishing block: a fence and an atomic in
+// every block, 1.4 us, and a last block that sums 2048 partials alone while
+// the next kernel waits, 2.8 us of the 9.2 us of the r.z sweep at 256x64x64.
+// With at most about kDotBlocks partials a thread of a 256-thread block loads
+// three.
+struct DotAcc64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s += v; }
+};
+struct DotAcc32 {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float v) {
         float sn, se;
-        two_sum(as, pv.x, sn, se);
-        as = sn;
-        ae += se + pv.y;
+        two_sum(s, v, sn, se);
+        s = sn;
+        e += se;
     }
-    block_pair_f(as, ae);
-    if (block_leader()) {
-        tot_f = (double)as + (double)ae;
-        *ticket = 0u;
-    }
-    __syncthreads();
-    out = tot_f;
-    return true;
+};
+template <typename V> struct DotAcc { using type = DotAcc64; };
+template <> struct DotAcc<float> { using type = DotAcc32; };
+__device__ __forceinline__ void dot_store(DotAcc32 a, double *part) {
+    block_pair_f(a.s, a.e);
+    if (block_leader()) reinterpret_cast<float2 *>(part)[BLOCK_ID()] = make_float2(a.s, a.e);
 }
-__device__ __forceinline__ bool reduce_last_sum(double v, double &out, double *__restrict__ part,
-                                                unsigned *__restrict__ ticket, int nb) {
-    double dummy = 0.0;
-    const bool last = reduce_last(v, dummy, 1, false, part, 0, ticket, nb);
-    out = v;
-    return last;
+__device__ __forceinline__ void dot_store(DotAcc64 a, double *part) {
+    const double v = block_sum(a.s);
+    if (block_leader()) part[BLOCK_ID()] = v;
+}
+// total of nb partials of vectors of type V, valid in the block leader (every
+// thread calls it)
+template <typename V> __device__ __forceinline__ double dot_total(const double *part, int nb);
+template <> __device__ __forceinline__ double dot_total<float>(const double *part, int nb) {
+    const int nt = blockDim.x * blockDim.y, t = threadIdx.x + blockDim.x * threadIdx.y;
+    float s = 0.f, e = 0.f;
+    for (int q = t; q < nb; q += nt) {
+        const float2 v = __ldcg(reinterpret_cast<const float2 *>(part) + q);
+        float sn, se;
+        two_sum(s, v.x, sn, se);
+        s = sn;
+        e += se + v.y;
+    }
+    block_pair_f(s, e);
+    return (double)s + (double)e;
+}
+template <> __device__ __forceinline__ double dot_total<double>(const double *part, int nb) {
+    const int nt = blockDim.x * blockDim.y, t = threadIdx.x + blockDim.x * threadIdx.y;
+    double s = 0.0;
+    for (int q = t; q < nb; q += nt) s += __ldcg(part + q);
+    return block_sum(s);
 }
 
 // Loop-control decisions taken by the finishing block: each writes
@@ -408,6 +417,8 @@ __device__ __forceinline__ void residual_control(double *scal, int *ctl, double 
         set_cond(ctl, h, !bad && rn > target);
         return;
     }
+    scal[S_RZ0] = 0.0;   // the FP32 iteration starts afresh
+    ctl[C_IT] = 0;
     if (mode == 1) {
         scal[S_TARGET] = rtol * (bn > 0.0 ? bn : rn);
         ctl[C_OUT] = 0;
@@ -1086,15 +1097,6 @@ __global__ void k_sum_to(int n, const T *__restrict__ x, double scale, double *_
     if (reduce_last(acc, dummy, 1, false, part, 0, ticket, gridDim.x) && block_leader()) scal[slot] = acc * scale;
 }
 
-template <typename T>
-__global__ void k_sum_field(int n, const T *__restrict__ x, double scale, double *__restrict__ part) {
-    griddep_wait();
-    double acc = 0.0;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) acc += (double)x[c];
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = acc * scale;
-}
-
 // u_sum += v and max |v - vold|; the finishing block applies the early exit
 // of Section 3.2: stop after sub-step k if k = N or the test value (E_k, or
 // max |du_cr| / U) is below the tolerance
@@ -1138,8 +1140,7 @@ __global__ void k_relax_accum(int n, const uint32_t *__restrict__ info, C3<T> v,
 // CG. The residual of the outer (FP64) system is r = b - M q with q and b in
 // FP64; the Krylov vectors are of type V (double on the FP64 path, float on
 // the mixed path). Dot products are accumulated per thread in V (a thread
-// takes several cells) and across threads and blocks in FP64; the finishing block of each reduction also
-// computes the CG scalars and takes the loop decisions.
+// takes several cells) and across threads and blocks in compensated FP32 pairs or FP64.
 // ---------------------------------------------------------------------------
 // The kernel also starts the first V-cycle: z receives the colour-0 half
 // sweep of the finest level from z = 0 (z = r / diagonal on colour 0, 0 on
@@ -1198,13 +1199,48 @@ __global__ void k_cg_init(GridD g, const uint32_t *__restrict__ info, C3<double>
     }
 }
 
-// Ap = M p and p.Ap; the finishing block sets alpha = (r.z) / (p.Ap)
+// beta = (r.z) / (r.z)_old (0 on the first iteration) from the partials of
+// r.z, rounded to V, in every thread of the block; the first block stores r.z
+// and counts the iteration
+template <typename V>
+__device__ __forceinline__ V cg_beta(const double *rz_part, int nrz, double *scal, int *ctl) {
+    __shared__ V beta_s;
+    const double rz = dot_total<V>(rz_part, nrz);
+    if (block_leader()) {
+        const double ro = scal[S_RZ0];
+        beta_s = (V)(ro != 0.0 ? rz / ro : 0.0);
+        if (BLOCK_ID() == 0) {
+            scal[S_RZ1] = rz;
+            ctl[C_IT] += 1;
+            ctl[C_ITSUM] += 1;
+        }
+    }
+    __syncthreads();
+    return beta_s;
+}
+// alpha = (r.z) / (p.Ap); the first block keeps r.z for the next beta
+template <typename V>
+__device__ __forceinline__ V cg_alpha(const double *pap_part, int npap, double *scal) {
+    __shared__ V alpha_s;
+    const double pap = dot_total<V>(pap_part, npap);
+    if (block_leader()) {
+        const double rz = scal[S_RZ1];
+        alpha_s = (V)(rz / pap);
+        if (BLOCK_ID() == 0) {
+            scal[S_PAP] = pap;
+            scal[S_RZ0] = rz;
+        }
+    }
+    __syncthreads();
+    return alpha_s;
+}
+
+// FP64 path: Ap = M p and p.Ap
 template <int DIM, typename T, typename V>
 __global__ void k_cg_apply_dot(GridD g, const uint32_t *__restrict__ info, C3<T> cf, const V *__restrict__ p,
-                               V *__restrict__ Ap, double *__restrict__ part, unsigned *__restrict__ ticket, int nb,
-                               double *__restrict__ scal) {
+                               V *__restrict__ Ap, double *__restrict__ part) {
     griddep_wait();
-    V accv = V(0);
+    typename DotAcc<V>::type acc;
     ROW_LOOP(g) {
         ROW_CELL(g);
         if (i >= g.nx) continue;
@@ -1214,184 +1250,202 @@ __global__ void k_cg_apply_dot(GridD g, const uint32_t *__restrict__ info, C3<T>
         } else {
             V y = poisson_row<DIM, T, V>(g, inf, c, i, j, k, cf, p);
             Ap[c] = y;
-            accv += p[c] * y;
+            acc.add(p[c] * y);
         }
     }
-    double acc;
-    if (reduce_last_sum(accv, acc, part, ticket, nb) && block_leader()) {
-        scal[S_PAP] = acc;
-        put_scalar(scal, S_ALPHA, S_ALPHA_F, scal[S_RZ1] / acc);
-    }
+    dot_store(acc, part);
 }
 
 // Mixed path: p = z + beta p and Ap = M z + beta Ap (the search direction
 // update folded into the operator apply: M p = M z + beta M p_old, so every
 // thread writes only its own cell), then p.Ap; beta = 0 starts afresh. Each
-// thread takes RPT rows (launch_rpt); the cell flags and face coefficients,
-// fixed during a solve, are loaded before the grid dependency wait, the
-// vectors after it, all rows at once.
+// thread takes RPT rows of a group (launch_groups), loaded together; the cell
+// flags and face coefficients, fixed during a solve, are loaded before the
+// grid dependency wait for its first group, the vectors after it.
 template <int DIM, typename T, typename V, int RPT>
-__global__ void k_cg_pz_apply(GridD g, const uint32_t *__restrict__ info, C3<T> cf, const V *__restrict__ z,
-                              V *__restrict__ p, V *__restrict__ Ap, double *__restrict__ part,
-                              unsigned *__restrict__ ticket, int nb, double *__restrict__ scal) {
+__global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, const uint32_t *__restrict__ info, C3<T> cf, const V *__restrict__ z,
+                              V *__restrict__ p, V *__restrict__ Ap, const double *__restrict__ rz_part, int nrz,
+                              double *__restrict__ part, int groups, double *__restrict__ scal, int *__restrict__ ctl) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int nrow = g.ny * g.nz;
-    const int row0 = blockIdx.y * blockDim.y * RPT + threadIdx.y;
     uint32_t inf[RPT];
     T w[RPT][2 * DIM];
-#pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        inf[u] = 0;
-        if (i < g.nx && row < nrow) {
-            const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
-            inf[u] = info[c];
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                w[u][2 * a] = cf.a[a][flo(g, a, i, j, k)];
-                w[u][2 * a + 1] = cf.a[a][fhi(g, a, i, j, k)];
-            }
-        }
-    }
-    griddep_wait();
-    const V be = get_scalar<V>(scal, S_BETA, S_BETA_F);
-    const bool fresh = be == V(0);
     V zc[RPT], zn[RPT][2 * DIM], po[RPT], ao[RPT];
+    auto load_fixed = [&](int row0) {
 #pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        if (i < g.nx && row < nrow) {
-            const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
-            const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
-            zc[u] = z[c];
-            po[u] = p[c];
-            ao[u] = Ap[c];
+        for (int u = 0; u < RPT; ++u) {
+            const int row = row0 + u * blockDim.y;
+            inf[u] = 0;
+            if (i < g.nx && row < nrow) {
+                const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
+                inf[u] = info[c];
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    w[u][2 * a] = cf.a[a][flo(g, a, i, j, k)];
+                    w[u][2 * a + 1] = cf.a[a][fhi(g, a, i, j, k)];
+                }
+            }
+        }
+    };
+    auto load_vectors = [&](int row0) {
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            const int row = row0 + u * blockDim.y;
+            if (i < g.nx && row < nrow) {
+                const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
+                const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
+                zc[u] = z[c];
+                po[u] = p[c];
+                ao[u] = Ap[c];
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    const int off = noff(g, a);
+                    zn[u][2 * a] = ijk[a] > 0 ? z[c - off] : V(0);
+                    zn[u][2 * a + 1] = ijk[a] < n[a] - 1 ? z[c + off] : V(0);
+                }
+            }
+        }
+    };
+    int grp = blockIdx.y;
+    const int step = blockDim.y * RPT;
+    load_fixed(grp * step + threadIdx.y);
+    griddep_wait();
+    load_vectors(grp * step + threadIdx.y);
+    const V be = cg_beta<V>(rz_part, nrz, scal, ctl);
+    const bool fresh = be == V(0);
+    typename DotAcc<V>::type acc;
+    for (;;) {
+        V accv = V(0);
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            const int row = grp * step + threadIdx.y + u * blockDim.y;
+            if (i >= g.nx || row >= nrow) continue;
+            const int c = i + g.nx * row;
+            const V pn = fresh ? zc[u] : zc[u] + be * po[u];
+            p[c] = pn;
+            if (!(inf[u] & INFO_FLUID)) {
+                Ap[c] = V(0);
+                continue;
+            }
+            V y = V(0);   // same terms and order as poisson_row
 #pragma unroll
             for (int a = 0; a < DIM; ++a) {
-                const int off = noff(g, a);
-                zn[u][2 * a] = ijk[a] > 0 ? z[c - off] : V(0);
-                zn[u][2 * a + 1] = ijk[a] < n[a] - 1 ? z[c + off] : V(0);
+#pragma unroll
+                for (int s2 = 0; s2 < 2; ++s2) {
+                    const int t = ftype(inf[u], a, s2);
+                    if (t == FT_INTERIOR) y += (V)w[u][2 * a + s2] * (zc[u] - zn[u][2 * a + s2]);
+                    else if (t == FT_OUTLET) y += (V)w[u][2 * a + s2] * zc[u];
+                }
             }
+            const V an = fresh ? y : y + be * ao[u];
+            Ap[c] = an;
+            accv += pn * an;
         }
+        acc.add(accv);
+        grp += gridDim.y;
+        if (grp >= groups) break;
+        load_fixed(grp * step + threadIdx.y);
+        load_vectors(grp * step + threadIdx.y);
     }
-    V accv = V(0);
-#pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        if (i >= g.nx || row >= nrow) continue;
-        const int c = i + g.nx * row;
-        const V pn = fresh ? zc[u] : zc[u] + be * po[u];
-        p[c] = pn;
-        if (!(inf[u] & INFO_FLUID)) {
-            Ap[c] = V(0);
-            continue;
-        }
-        V y = V(0);   // same terms and order as poisson_row
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-#pragma unroll
-            for (int s2 = 0; s2 < 2; ++s2) {
-                const int t = ftype(inf[u], a, s2);
-                if (t == FT_INTERIOR) y += (V)w[u][2 * a + s2] * (zc[u] - zn[u][2 * a + s2]);
-                else if (t == FT_OUTLET) y += (V)w[u][2 * a + s2] * zc[u];
-            }
-        }
-        const V an = fresh ? y : y + be * ao[u];
-        Ap[c] = an;
-        accv += pn * an;
-    }
-    double acc;
-    if (reduce_last_sum(accv, acc, part, ticket, nb) && block_leader()) {
-        scal[S_PAP] = acc;
-        put_scalar(scal, S_ALPHA, S_ALPHA_F, scal[S_RZ1] / acc);
-    }
+    dot_store(acc, part);
 }
 
-// x += alpha p, r -= alpha Ap, and z = the first colour-0 half sweep of the
-// next V-cycle (as in k_cg_init); the finishing block tests ||r|| against
-// scal[target_slot] and decides whether the PCG loop continues. RPT rows per
-// thread (launch_rpt), loaded together. xfresh: x starts from 0 in the first
+// x += alpha p, r -= alpha Ap, z = the first colour-0 half sweep of the next
+// V-cycle (as in k_cg_init), and r.r. RPT rows per thread and group
+// (launch_groups), loaded together. xfresh: x starts from 0 in the first
 // iteration (x is not read then), so it needs no clearing beforehand.
 template <typename V, int RPT>
-__global__ void k_cg_update(GridD g, V *__restrict__ x, V *__restrict__ r, const V *__restrict__ p,
+__global__ void __launch_bounds__(256) k_cg_update(GridD g, V *__restrict__ x, V *__restrict__ r, const V *__restrict__ p,
                             const V *__restrict__ Ap, const V *__restrict__ idiag0, V *__restrict__ z,
-                            double *__restrict__ part, unsigned *__restrict__ ticket, double *__restrict__ scal,
-                            int *__restrict__ ctl, int maxit, int target_slot, int xfresh,
-                            cudaGraphConditionalHandle h) {
+                            const double *__restrict__ pap_part, int npap, double *__restrict__ part, int groups,
+                            double *__restrict__ scal, const int *__restrict__ ctl, int xfresh) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int nrow = g.ny * g.nz;
-    const int row0 = blockIdx.y * blockDim.y * RPT + threadIdx.y;
-    V id[RPT];
+    V id[RPT], xo[RPT], ro[RPT], pc[RPT], ac[RPT];
+    auto load_fixed = [&](int row0) {
 #pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        id[u] = (i < g.nx && row < nrow) ? idiag0[i + g.nx * row] : V(0);
-    }
-    griddep_wait();
-    const V al = get_scalar<V>(scal, S_ALPHA, S_ALPHA_F);
-    // with xfresh, the first iteration of a solve (iteration counter still 0:
-    // every block reads it before the finishing block counts) starts x from 0
-    const bool x0 = xfresh && ctl[C_IT] == 0;
-    V xo[RPT], ro[RPT], pc[RPT], ac[RPT];
-#pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        if (i < g.nx && row < nrow) {
-            const int c = i + g.nx * row;
-            xo[u] = x0 ? V(0) : x[c];
-            ro[u] = r[c];
-            pc[u] = p[c];
-            ac[u] = Ap[c];
+        for (int u = 0; u < RPT; ++u) {
+            const int row = row0 + u * blockDim.y;
+            id[u] = (i < g.nx && row < nrow) ? idiag0[i + g.nx * row] : V(0);
         }
-    }
-    V accv = V(0);
+    };
+    int grp = blockIdx.y;
+    const int step = blockDim.y * RPT;
+    load_fixed(grp * step + threadIdx.y);
+    griddep_wait();
+    // with xfresh, the first iteration of a solve (counted by the kernel before) starts x from 0
+    const bool x0 = xfresh && ctl[C_IT] == 1;
+    auto load_vectors = [&](int row0) {
 #pragma unroll
-    for (int u = 0; u < RPT; ++u) {
-        const int row = row0 + u * blockDim.y;
-        if (i >= g.nx || row >= nrow) continue;
-        const int c = i + g.nx * row;
-        const int k = row / g.ny, j = row - k * g.ny;
-        x[c] = x0 ? al * pc[u] : xo[u] + al * pc[u];
-        const V rc = ro[u] - al * ac[u];
-        r[c] = rc;
-        z[c] = ((i + j + k) & 1) == 0 ? rc * id[u] : V(0);
-        accv += rc * rc;
+        for (int u = 0; u < RPT; ++u) {
+            const int row = row0 + u * blockDim.y;
+            if (i < g.nx && row < nrow) {
+                const int c = i + g.nx * row;
+                xo[u] = x0 ? V(0) : x[c];
+                ro[u] = r[c];
+                pc[u] = p[c];
+                ac[u] = Ap[c];
+            }
+        }
+    };
+    load_vectors(grp * step + threadIdx.y);
+    const V al = cg_alpha<V>(pap_part, npap, scal);
+    typename DotAcc<V>::type acc;
+    for (;;) {
+        V accv = V(0);
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            const int row = grp * step + threadIdx.y + u * blockDim.y;
+            if (i >= g.nx || row >= nrow) continue;
+            const int c = i + g.nx * row;
+            const int k = row / g.ny, j = row - k * g.ny;
+            x[c] = x0 ? al * pc[u] : xo[u] + al * pc[u];
+            const V rc = ro[u] - al * ac[u];
+            r[c] = rc;
+            z[c] = ((i + j + k) & 1) == 0 ? rc * id[u] : V(0);
+            accv += rc * rc;
+        }
+        acc.add(accv);
+        grp += gridDim.y;
+        if (grp >= groups) break;
+        load_fixed(grp * step + threadIdx.y);
+        load_vectors(grp * step + threadIdx.y);
     }
-    double acc;
-    if (reduce_last_sum(accv, acc, part, ticket, gridDim.x * gridDim.y) && block_leader()) {
-        scal[S_RR] = acc;
-        int it = ++ctl[C_IT];
-        ctl[C_ITSUM] += 1;
-        double rn = sqrt(acc);
-        scal[S_RZ0] = scal[S_RZ1];
-        bool bad = !isfinite(rn);
-        if (bad) ctl[C_NAN] = 1;
-        bool more = !bad && rn > scal[target_slot];
-        if (more && it >= maxit) { ctl[C_NOTCONV] = 1; more = false; }
-        set_cond(ctl, h, more);
-    }
+    dot_store(acc, part);
 }
 
-// r.z; the finishing block sets beta = (r.z)_new / (r.z)_old (0 on the first iteration)
+// FP64 path, one block: ||r|| from the partials of r.r against the target;
+// decides whether the PCG loop continues
 template <typename V>
-__global__ void k_cg_dot_rz(int n, const V *__restrict__ x, const V *__restrict__ y, double *__restrict__ part,
-                            unsigned *__restrict__ ticket, double *__restrict__ scal) {
+__global__ void k_cg_check(const double *__restrict__ rr_part, int nrr, double *__restrict__ scal, int *__restrict__ ctl,
+                           int maxit, cudaGraphConditionalHandle h) {
     griddep_wait();
-    V accv = V(0);
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) accv += x[c] * y[c];
-    double acc;
-    if (reduce_last_sum(accv, acc, part, ticket, gridDim.x) && block_leader()) {
-        double ro = scal[S_RZ0];
-        scal[S_RZ1] = acc;
-        put_scalar(scal, S_BETA, S_BETA_F, ro != 0.0 ? acc / ro : 0.0);
-    }
+    const double rr = dot_total<V>(rr_part, nrr);
+    if (!block_leader()) return;
+    scal[S_RR] = rr;
+    const double rn = sqrt(rr);
+    const bool bad = !isfinite(rn);
+    if (bad) ctl[C_NAN] = 1;
+    bool more = !bad && rn > scal[S_TARGET];
+    if (more && ctl[C_IT] >= maxit) { ctl[C_NOTCONV] = 1; more = false; }
+    set_cond(ctl, h, more);
+}
+
+// r.z, cell by cell (when the whole V-cycle ran in the cluster)
+template <typename V>
+__global__ void k_cg_dot_rz(int n, const V *__restrict__ x, const V *__restrict__ y, double *__restrict__ part) {
+    griddep_wait();
+    typename DotAcc<V>::type acc;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) acc.add(x[c] * y[c]);
+    dot_store(acc, part);
 }
 
 // p = z + beta p
 template <typename V>
-__global__ void k_cg_pupdate(int n, const double *__restrict__ scal, const V *__restrict__ z, V *__restrict__ p) {
+__global__ void k_cg_pupdate(int n, const V *__restrict__ z, V *__restrict__ p, const double *__restrict__ rz_part, int nrz,
+                             double *__restrict__ scal, int *__restrict__ ctl) {
     griddep_wait();
-    const V be = get_scalar<V>(scal, S_BETA, S_BETA_F);
+    const V be = cg_beta<V>(rz_part, nrz, scal, ctl);
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) p[c] = z[c] + be * p[c];
 }
 
@@ -1438,19 +1492,45 @@ __device__ __forceinline__ void poisson_row_comp(const GridD &g, uint32_t inf, i
     }
 }
 
-// End of an outer defect-correction trip (mixed path): q += e in FP64, and the
-// FP64 residual updated recursively, r64 -= M e, with M e from the
-// compensated apply above (so r64 stays b - M q to FP64 accuracy, without
-// re-evaluating the operator on q in FP64); then r = (float) r64, z = the
-// first colour-0 half sweep of the next V-cycle, ||r||^2, and the loop
-// decision of residual_control(mode 2).
+// Mixed path, the last kernel of an iteration: every block forms ||r|| from
+// the partials of r.r (the same value everywhere) and decides whether the FP32
+// iteration goes on; if so, that is all. Otherwise the defect-correction trip
+// ends: q += e in FP64, and the FP64 residual updated recursively, r64 -= M e,
+// with M e from the compensated apply above (so r64 stays b - M q to FP64
+// accuracy, without re-evaluating the operator on q in FP64); then
+// r = (float) r64, z = the first colour-0 half sweep of the next V-cycle,
+// ||r||^2, and the loop decision of residual_control(mode 2). With the trip's
+// end inside the iteration a solve is one loop: a loop of iterations inside
+// one of trips costs 5 us to enter and to leave per trip, more than the
+// 1.5 us of the iterations that only check. The values the decision reads are
+// written by the last block to finish at the earliest.
 template <int DIM>
 __global__ void k_cg_refine(GridD g, const uint32_t *__restrict__ info, C3<float> cf, const float *__restrict__ e,
                             double *__restrict__ q, double *__restrict__ r64, float *__restrict__ r,
-                            const float *__restrict__ idiag0, float *__restrict__ z, double *__restrict__ part,
-                            int stride, unsigned *__restrict__ ticket, int nb, double *__restrict__ scal,
-                            int *__restrict__ ctl, double rtol, cudaGraphConditionalHandle h) {
+                            const float *__restrict__ idiag0, float *__restrict__ z, const double *__restrict__ rr_part,
+                            int nrr, double *__restrict__ part, int stride, unsigned *__restrict__ ticket, int nb,
+                            double *__restrict__ scal, int *__restrict__ ctl, double rtol, int maxit,
+                            cudaGraphConditionalHandle h) {
     griddep_wait();
+    __shared__ int more_s;
+    {
+        const double rr = dot_total<float>(rr_part, nrr);
+        if (block_leader()) {
+            const double rn = sqrt(rr);
+            const bool bad = !isfinite(rn);
+            bool more = !bad && rn > scal[S_ITARGET];
+            const bool capped = more && ctl[C_IT] >= maxit;
+            if (capped) more = false;
+            if (BLOCK_ID() == 0) {
+                if (bad) ctl[C_NAN] = 1;
+                if (capped) ctl[C_NOTCONV] = 1;
+                if (more) set_cond(ctl, h, true);
+            }
+            more_s = more;
+        }
+        __syncthreads();
+        if (more_s) return;
+    }
     double rr = 0.0, dummy = 0.0;
     ROW_LOOP(g) {
         ROW_CELL(g);
@@ -1563,41 +1643,47 @@ __global__ void k_mg_rbgs(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__
 
 // The last half sweep of the finest level (colour 0) fused with r.z: the
 // thread of colour cell i also takes its row partner i ^ 1 (colour 1, final
-// already), so every cell is counted once; the finishing block sets
-// beta = (r.z)_new / (r.z)_old as k_cg_dot_rz does.
+// already), so every cell is counted once. A block takes several rows
+// (launch_groups over the colour's cells).
 template <int DIM, typename M>
-__global__ void k_mg_rbgs_dot(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__restrict__ x,
-                              const M *__restrict__ b, int colour, double *__restrict__ part,
-                              unsigned *__restrict__ ticket, double *__restrict__ scal) {
+__global__ void __launch_bounds__(256) k_mg_rbgs_dot(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__restrict__ x,
+                              const M *__restrict__ b, int colour, int groups, double *__restrict__ part) {
     const int ti = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int k = blockIdx.z;
-    const int i = 2 * ti + ((j + k + colour) & 1);
-    const bool ok = i < g.nx && j < g.ny;
-    const int cell = i + g.nx * (j + g.ny * k);
-    const int ip = i ^ 1;
-    const bool okp = ip < g.nx && j < g.ny;
-    const int cellp = ip + g.nx * (j + g.ny * k);
+    const int nrow = g.ny * g.nz;
+    int grp = blockIdx.y;
     M w[2 * DIM], id = M(0);
-    if (ok) {
-        mg_row_coeffs<DIM, M>(g, cc, i, j, k, w);
-        id = idiag[cell];
-    }
+    int row, j, k, i;
+    bool ok;
+    auto load_fixed = [&]() {
+        row = grp * blockDim.y + threadIdx.y;
+        k = row / g.ny;
+        j = row - k * g.ny;
+        i = 2 * ti + ((j + k + colour) & 1);
+        ok = i < g.nx && row < nrow;
+        if (ok) {
+            mg_row_coeffs<DIM, M>(g, cc, i, j, k, w);
+            id = idiag[i + g.nx * row];
+        }
+    };
+    load_fixed();
     griddep_wait();
-    M acc = M(0);
-    if (ok) {
-        const M bc = b[cell];
-        const M xn = (bc + mg_row_off<DIM, M>(g, w, x, cell, i, j, k)) * id;
-        x[cell] = xn;
-        acc = bc * xn;
+    typename DotAcc<M>::type sum;
+    for (;;) {
+        const int cell = i + g.nx * row, ip = i ^ 1, cellp = ip + g.nx * row;
+        M acc = M(0);
+        if (ok) {
+            const M bc = b[cell];
+            const M xn = (bc + mg_row_off<DIM, M>(g, w, x, cell, i, j, k)) * id;
+            x[cell] = xn;
+            acc = bc * xn;
+        }
+        if (ip < g.nx && row < nrow) acc += b[cellp] * x[cellp];
+        sum.add(acc);
+        grp += gridDim.y;
+        if (grp >= groups) break;
+        load_fixed();
     }
-    if (okp) acc += b[cellp] * x[cellp];
-    double a64;
-    if (reduce_last_sum(acc, a64, part, ticket, gridDim.x * gridDim.y * gridDim.z) && block_leader()) {
-        double ro = scal[S_RZ0];
-        scal[S_RZ1] = a64;
-        put_scalar(scal, S_BETA, S_BETA_F, ro != 0.0 ? a64 / ro : 0.0);
-    }
+    dot_store(sum, part);
 }
 
 // coarse b = sum over children of the fine residual b - M x. With first set,

@@ -75,17 +75,10 @@ inline void launchk(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 }
 
 // ---------------------------------------------------------------------------
-// control kernels (one thread). The other loop decisions are taken by the
-// finishing block of the reductions (see k_cg_init, k_cg_update,
+// control kernel (one thread). The other loop decisions are taken by the
+// finishing block of the reductions (see k_cg_init, k_cg_check, k_cg_refine,
 // k_relax_accum).
 // ---------------------------------------------------------------------------
-static __global__ void k_inner_start(double *scal, int *ctl, cudaGraphConditionalHandle h) {
-    griddep_wait();
-    scal[S_RZ0] = 0.0;
-    ctl[C_IT] = 0;
-    set_cond(ctl, h, true);
-}
-
 static __global__ void k_relax_init(int *ctl, cudaGraphConditionalHandle h) {
     griddep_wait(); set_cond(ctl, h, ctl[C_N] > 0); }
 
@@ -201,6 +194,8 @@ template <typename T> struct Impl {
     // FP64 copy of the level-0 coefficients of direction a (mixed path only)
     static double *cf64_out(Instance &I, int a) { return sizeof(T) == sizeof(double) ? nullptr : I.cf64[a]; }
     static P3<T> p3(void *const *p) { P3<T> r; for (int a = 0; a < 3; ++a) r.a[a] = (T *)p[a]; return r; }
+    // partial sums of the CG's dot products and of k_cg_refine, each in slots of its own
+    enum { kPartRz = 4, kPartPap, kPartRr, kPartRefine };
     static double *part(Instance &I, int slot) { return I.partials + (size_t)slot * I.red_stride; }
 
 
@@ -386,10 +381,12 @@ template <typename T> struct Impl {
         Level &L = I.lev[l];
         GridD g = to_dev(L.g);
         L3 LL = launch3((L.g.nx + 1) / 2, L.g.ny, L.g.nz);
-        if (with_dot)
-            launchk(k_mg_rbgs_dot<DIM, M>, LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, colour,
-                    I.partials, I.ticket, I.scal), ++I.nlaunch;
-        else
+        if (with_dot) {
+            const L3G LD = launch_groups((L.g.nx + 1) / 2, L.g.ny * L.g.nz, 1);
+            launchk(k_mg_rbgs_dot<DIM, M>, LD.grid, LD.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, colour,
+                    LD.groups, part(I, kPartRz)), ++I.nlaunch;
+            I.nrz = LD.nblocks;
+        } else
             for (int rep = 0; rep < (l == 0 && I.repeat_fine ? 2 : 1); ++rep)   // a repeat is idempotent
                 launchk(k_mg_rbgs<DIM, M, false>, LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x,
                         b, colour, g, 0, 0, 0, (const M *)nullptr), ++I.nlaunch;
@@ -481,39 +478,43 @@ template <typename T> struct Impl {
                 I.scal, I.ctl, I.P.cg_rtol, mode, h, with_E ? 1.0 / (double)I.n_fluid : 0.0), ++I.nlaunch;
     }
 
-    // one PCG iteration on M x = r with Krylov vectors z, p, Ap (type V)
+    // one PCG iteration on M x = r with Krylov vectors z, p, Ap (type V), up to
+    // the update; nrr: partials of r.r left in kPartRr
     template <int DIM>
-    static int pcg_body(Instance &I, V *x, int target_slot, cudaGraphConditionalHandle h, int xfresh) {
+    static int pcg_body(Instance &I, V *x, int xfresh, int *nrr) {
         GridD g = to_dev(I.g);
-        L3 L = launch_rows(I.g, kRedBlocks);
-        int n = I.g.ncell;
+        const int n = I.g.ncell, rows = I.g.ny * I.g.nz;
         V *r = (V *)I.cg_r, *z = (V *)I.cg_z, *p = (V *)I.cg_p, *Ap = (V *)I.cg_Ap;
-        long long n0 = I.nlaunch;
         OSCAR_TRY(vcycle_d<DIM>(I, r, z));
-        if (top_level(I) == 0)   // the whole V-cycle ran in the cluster: r.z on its own
-            launchk(k_cg_dot_rz<V>, kRedBlocks, BS, 0, I.stream, n, r, z, I.partials, I.ticket, I.scal), ++I.nlaunch;
+        if (top_level(I) == 0) {   // the whole V-cycle ran in the cluster: r.z on its own
+            I.nrz = std::min(kDotBlocks, nblk(n));
+            launchk(k_cg_dot_rz<V>, I.nrz, BS, 0, I.stream, n, r, z, part(I, kPartRz)), ++I.nlaunch;
+        }
+        int npap;
         if constexpr (sizeof(V) == sizeof(float)) {
-            L3 LA = launch_rpt(I.g, kApplyRows);
+            const L3G LA = launch_groups(I.g.nx, rows, kApplyRows);
+            npap = LA.nblocks;
             launchk(k_cg_pz_apply<DIM, T, V, kApplyRows>, LA.grid, LA.block, 0, I.stream, g, I.info, c3(I.lev[0].c),
-                    (const V *)z, p, Ap, I.partials, I.ticket, LA.nblocks, I.scal), ++I.nlaunch;
+                    (const V *)z, p, Ap, part(I, kPartRz), I.nrz, part(I, kPartPap), LA.groups, I.scal, I.ctl), ++I.nlaunch;
         } else {   // FP64 path: the search direction as written, M p applied directly
-            launchk(k_cg_pupdate<V>, kRedBlocks, BS, 0, I.stream, n, I.scal, z, p), ++I.nlaunch;
+            launchk(k_cg_pupdate<V>, std::min(kDotBlocks, nblk(n)), BS, 0, I.stream, n, (const V *)z, p,
+                    part(I, kPartRz), I.nrz, I.scal, I.ctl), ++I.nlaunch;
+            const L3 L = launch_rows(I.g, kDotBlocks);
+            npap = L.nblocks;
             launchk(k_cg_apply_dot<DIM, T, V>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.lev[0].c), p, Ap,
-                    I.partials, I.ticket, L.nblocks, I.scal), ++I.nlaunch;
+                    part(I, kPartPap)), ++I.nlaunch;
         }
-        L3 LU = launch_rpt(I.g, kUpdateRows);
+        const L3G LU = launch_groups(I.g.nx, rows, kUpdateRows);
         launchk(k_cg_update<V, kUpdateRows>, LU.grid, LU.block, 0, I.stream, g, x, r, p, Ap, (const V *)I.lev[0].idiag,
-                z, I.partials, I.ticket, I.scal, I.ctl, I.P.cg_maxit, target_slot, xfresh, h), ++I.nlaunch;
-        if (I.capturing) {
-            I.n_cg_body = I.nlaunch - n0;
-            I.cg_bodies_captured += 1;
-        }
+                z, part(I, kPartPap), npap, part(I, kPartRr), LU.groups, I.scal, (const int *)I.ctl, xfresh), ++I.nlaunch;
+        *nrr = LU.nblocks;
         OSCAR_LAUNCH_CHECK();
         return 0;
     }
 
     // Pressure solve M q = b. FP64 path: PCG on q itself. Mixed path: FP64
-    // defect correction around an FP32 PCG for the correction e.
+    // defect correction around an FP32 PCG for the correction e, as one loop of
+    // PCG iterations (k_cg_refine ends a trip).
     template <int DIM>
     static int pcg_d(Instance &I, double *q, const double *b, bool with_E) {
         if (DIM == 2 && I.solve_nc) {
@@ -537,36 +538,34 @@ template <typename T> struct Impl {
             OSCAR_LAUNCH_CHECK();
             return 0;
         }
-        if constexpr (sizeof(T) == sizeof(double)) {
-            cudaGraphConditionalHandle h;
-            OSCAR_TRY(cond_handle(I, &h));
-            residual64<DIM>(I, q, b, 0, h, (V *)I.cg_p, nullptr, nullptr, with_E);
-            return loop_while(I, h, [&]() -> int { return pcg_body<DIM>(I, (V *)q, S_TARGET, h, 0); });
-        } else {
-        cudaGraphConditionalHandle ho;
-        OSCAR_TRY(cond_handle(I, &ho));
-        // the inner solve starts e and p from 0 itself (xfresh, beta = 0), so
-        // neither is cleared; the FP64 residual is evaluated once, then updated
-        // by k_cg_refine at the end of every trip
-        residual64<DIM>(I, q, b, 1, ho, nullptr, nullptr, I.cg_r64, with_E);
-        return loop_while(I, ho, [&]() -> int {
-            long long n0 = I.nlaunch, cg0 = I.cg_bodies_captured;
-            cudaGraphConditionalHandle hi;
-            OSCAR_TRY(cond_handle(I, &hi));
-            launchk(k_inner_start, 1, 1, 0, I.stream, I.scal, I.ctl, hi), ++I.nlaunch;
-            OSCAR_TRY(loop_while(I, hi, [&]() -> int { return pcg_body<DIM>(I, (V *)I.cg_e, S_ITARGET, hi, 1); }));
-            if constexpr (sizeof(V) == sizeof(float)) {
-                GridD g = to_dev(I.g);
-                L3 L = launch_rows(I.g, kRedBlocks);
-                launchk(k_cg_refine<DIM>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.lev[0].c), (const float *)I.cg_e,
-                        q, I.cg_r64, (float *)I.cg_r, (const float *)I.lev[0].idiag, (float *)I.cg_z, I.partials,
-                        I.red_stride, I.ticket, L.nblocks, I.scal, I.ctl, I.P.cg_rtol, ho), ++I.nlaunch;
+        constexpr bool mixed = sizeof(T) == sizeof(float);
+        cudaGraphConditionalHandle h;
+        OSCAR_TRY(cond_handle(I, &h));
+        // mixed: the iteration starts e and p from 0 itself (xfresh, beta = 0),
+        // so neither is cleared; the FP64 residual is evaluated once, then
+        // updated by k_cg_refine at the end of every trip
+        residual64<DIM>(I, q, b, mixed ? 1 : 0, h, mixed ? nullptr : (V *)I.cg_p, nullptr, mixed ? I.cg_r64 : nullptr, with_E);
+        return loop_while(I, h, [&]() -> int {
+            const long long n0 = I.nlaunch;
+            int nrr = 0;
+            OSCAR_TRY(pcg_body<DIM>(I, mixed ? (V *)I.cg_e : (V *)q, mixed ? 1 : 0, &nrr));
+            if constexpr (mixed) {
+                const L3 L = launch_rows(I.g, kRedBlocks);
+                launchk(k_cg_refine<DIM>, L.grid, L.block, 0, I.stream, to_dev(I.g), I.info, c3(I.lev[0].c),
+                        (const float *)I.cg_e, q, I.cg_r64, (float *)I.cg_r, (const float *)I.lev[0].idiag,
+                        (float *)I.cg_z, part(I, kPartRr), nrr, part(I, kPartRefine), I.red_stride, I.ticket, L.nblocks,
+                        I.scal, I.ctl, I.P.cg_rtol, I.P.cg_maxit, h), ++I.nlaunch;
+            } else {
+                launchk(k_cg_check<V>, 1, BS, 0, I.stream, part(I, kPartRr), nrr, I.scal, I.ctl, I.P.cg_maxit, h),
+                    ++I.nlaunch;
             }
-            if (I.capturing) I.n_outer_body = (I.nlaunch - n0) - (I.cg_bodies_captured - cg0) * I.n_cg_body;
+            if (I.capturing) {
+                I.n_cg_body = I.nlaunch - n0;
+                I.cg_bodies_captured += 1;
+            }
             OSCAR_LAUNCH_CHECK();
             return 0;
         });
-        }
     }
 
     // --- PISO (Section 2.2) --------------------------------------------------
@@ -699,18 +698,12 @@ template <typename T> struct Impl {
         launchk(k_relax_init, 1, 1, 0, I.stream, I.ctl, h), ++I.nlaunch;
         *n_pre = I.nlaunch - s0;
         long long b0 = I.nlaunch, cg0 = I.cg_bodies_captured;
-        long long ob0 = I.cg_bodies_captured;
-        int outer_bodies_before = 0;
-        (void)ob0;
-        (void)outer_bodies_before;
-        int npiso_solves = 0;
         int rc = loop_while(I, h, [&]() -> int {
             OSCAR_TRY(transport(I, I.phi_cr, dt));
             OSCAR_TRY(interface_(I, I.alpha_new));
             OSCAR_TRY(sum_faces(I, I.phi_vd, I.phi_cr, I.phic));
             OSCAR_TRY(copy_fields(I, I.vold, I.u_cr, 0));
             OSCAR_TRY(piso(I, I.u_cr, I.p_cr, I.phi_cr, true, 0.0, dt));
-            npiso_solves += I.P.n_piso;
             OSCAR_TRY(commit_alpha(I));
             if (area) OSCAR_TRY(relax_energy(I, S_AREA1));
             P3<double> us;
@@ -728,8 +721,7 @@ template <typename T> struct Impl {
             return 0;
         });
         // launches of one sub-step outside the loop bodies of its pressure solves
-        long long outer = sizeof(T) == sizeof(double) ? 0 : (long long)npiso_solves * I.n_outer_body;
-        *n_body = (I.nlaunch - b0) - (I.cg_bodies_captured - cg0) * I.n_cg_body - outer;
+        *n_body = (I.nlaunch - b0) - (I.cg_bodies_captured - cg0) * I.n_cg_body;
         return rc;
     }
 
@@ -750,10 +742,7 @@ template <typename T> struct Impl {
         if (kind == 0) rc = body_drag(I, dt);
         else if (kind == 1) rc = body_relax(I, dt, &n_pre, &n_body);
         else rc = body_standard(I, dt);
-        if (kind != 1) {
-            long long outer = sizeof(T) == sizeof(double) ? 0 : (long long)I.P.n_piso * I.n_outer_body;
-            n_pre = (I.nlaunch - s0) - (I.cg_bodies_captured - cg0) * I.n_cg_body - outer;
-        }
+        if (kind != 1) n_pre = (I.nlaunch - s0) - (I.cg_bodies_captured - cg0) * I.n_cg_body;
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(I.stream, &graph);
         I.capturing = 0;
@@ -820,9 +809,7 @@ template <typename T> struct Impl {
         int its = I.ctl_host[C_ITSUM];
         int trips = kind == 1 ? I.ctl_host[C_K] : 1;
         if (!eager_now(I)) {
-            long long outer_trips = sizeof(T) == sizeof(double) ? 0 : (long long)I.ctl_host[C_OSUM];
-            I.nexec += G.n_pre + (long long)(kind == 1 ? trips : 0) * G.n_body + (long long)its * I.n_cg_body +
-                       outer_trips * I.n_outer_body;
+            I.nexec += G.n_pre + (long long)(kind == 1 ? trips : 0) * G.n_body + (long long)its * I.n_cg_body;
         }
         I.cg_iters_last = its;
         I.cg_iters_total += its;
@@ -834,7 +821,7 @@ template <typename T> struct Impl {
 };
 
 template <typename T> void Solver<T>::release_graphs(Instance &I) {
-    I.n_cg_body = I.n_outer_body = 0;   // set again by the next capture
+    I.n_cg_body = 0;   // set again by the next capture
     for (int k = 0; k < 3; ++k) {
         GraphSlot &G = I.gslot[k];
         if (G.valid) {
