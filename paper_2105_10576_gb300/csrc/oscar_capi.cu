@@ -191,6 +191,7 @@ static void carve(Instance &I, Carver &C) {
     }
     I.stage_dev = (double *)C.take(I.stage_len * sizeof(double));
     I.cl_inv = C.take(kClInvBytes);
+    I.cl_image = C.take(kClImageBytes);
     I.partials = (double *)C.take((size_t)kRedSlots * I.red_stride * sizeof(double));
     I.scal = (double *)C.take(S_COUNT * sizeof(double));
     I.ctl = (int *)C.take(C_COUNT * sizeof(int));

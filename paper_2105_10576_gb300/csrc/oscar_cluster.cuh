@@ -52,19 +52,23 @@ template <typename M> struct ClLevel {
     int G, D, E;             // columns beyond the slab: held on each side, on which b is needed, on which x is needed
     int ncol, ps, nloc;      // local columns (widest slab), column stride, local cells
     int ce;                  // entries of a column in a colour list: ceil(ny / 2) nz
-    float rncol, rny, rhj;   // reciprocals for the cell decomposition
+    float rncol, rny, rce;   // reciprocals for the cell decomposition
     const M *c[3], *idiag;
-    // shared-memory byte offsets: x, b, reciprocal diagonal, low-face
-    // coefficients per direction, colour lists (local indices by column), the
-    // coarse local index of each colour-0 entry
-    int ox, ob, oi, oc[3], ol[2], op;
+    // shared-memory byte offsets: reciprocal diagonal, low-face coefficients
+    // per direction, colour lists (local indices by column), the coarse local
+    // index of each colour-0 entry, slab starts of all ranks; x, b
+    int oi, oc[3], ol[2], op, os;
+    int ox, ob;
 };
 template <typename M> struct ClLevels {
     int n, nc, lnc;          // levels, CTAs (a power of two) and their log2
     int cols;                // columns of the coarsest level
-    int ors, obx, oinv;      // residual scratch, gathered right-hand side and inverse rows of the coarsest level
+    int img;                 // bytes of the image: what is fixed for a set of coefficients, at the start of shared memory
+    int oinv, orow;          // in the image: the inverse's rows that the CTA works, and the local cell of each
+    int ors, obx;            // residual scratch, gathered right-hand side of the coarsest level
     int ored;                // reduction scratch
     const M *inv;            // explicit inverse of the coarsest level (row-major)
+    unsigned char *image;    // the images of all ranks, img bytes apart
     ClLevel<M> L[kMaxCL];
 };
 
@@ -95,8 +99,9 @@ __device__ __forceinline__ void cl_store(unsigned a, double v) {
 }
 
 // slab of rank r on a level: global columns [cl_start(r), cl_start(r + 1))
-template <typename M> __device__ __forceinline__ int cl_start(const ClLevels<M> &P, const ClLevel<M> &L, int r) {
-    return min(((r * P.cols) >> P.lnc) << L.sh, L.nx);
+template <typename M> __host__ __device__ __forceinline__ int cl_start(const ClLevels<M> &P, const ClLevel<M> &L, int r) {
+    const int s = ((r * P.cols) >> P.lnc) << L.sh;
+    return s < L.nx ? s : L.nx;
 }
 // local columns [q0, q1) of the slab with d columns beyond it on each side, inside the domain
 struct ClRange { int s, w, q0, q1; };
@@ -109,52 +114,63 @@ __device__ __forceinline__ ClRange cl_range(const ClLevels<M> &P, const ClLevel<
     r.q1 = min(L.G + r.w + min(d, L.G), L.G + L.nx - r.s);
     return r;
 }
+// columns beyond its slab on which a CTA works the coarsest level's solution
+// itself: in FP64, bound by FP64 issue, none (the values are sent instead)
+template <typename M> __host__ __device__ __forceinline__ int cl_exact_depth(const ClLevels<M> &P) {
+    return sizeof(M) == sizeof(float) ? P.L[P.n - 1].E : 0;
+}
 
 // store v into field f (a shared-memory array in the level's layout) at global
 // column i, position m of the column, in every other CTA whose ghosts of depth
 // d cover it
 template <typename M>
-__device__ __forceinline__ void cl_push(const ClLevels<M> &P, const ClLevel<M> &L, M *f, int i, int m, int d, int rank, M v) {
+__device__ __forceinline__ void cl_push(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, M *f, int i, int m,
+                                        int d, int rank, M v) {
+    const short *st = (const short *)(sm + L.os);
     for (int r = rank - 1; r >= 0; --r) {
-        if (i >= cl_start(P, L, r + 1) + d) break;
-        cl_store(cl_addr(f + (i - cl_start(P, L, r) + L.G) * L.ps + m, r), v);
+        if (i >= st[r + 1] + d) break;
+        cl_store(cl_addr(f + (i - st[r] + L.G) * L.ps + m, r), v);
     }
     for (int r = rank + 1; r < P.nc; ++r) {
-        const int s = cl_start(P, L, r);
+        const int s = st[r];
         if (i < s - d) break;
         cl_store(cl_addr(f + (i - s + L.G) * L.ps + m, r), v);
     }
 }
 
-// Coefficients and lists of every level into shared memory; x and b cleared.
-// Ends without a barrier.
+// idx / n and the remainder, without integer division (rn = 1 / n; exact below 2^22)
+__device__ __forceinline__ int div_rem(int idx, int n, float rn, int &rem) {
+    int q = (int)(((float)idx + 0.5f) * rn);
+    rem = idx - q * n;
+    if (rem < 0) { --q; rem += n; } else if (rem >= n) { ++q; rem -= n; }
+    return q;
+}
+
+// The image of the cluster's levels, one per CTA of the cluster: coefficients
+// and lists in the local layout, once per set of coefficients, so that every
+// V-cycle (or solve) starts from one contiguous copy. Block (rank, slice).
+constexpr int kPackSlices = 8, kPackThreads = 256;
 template <int DIM, typename M>
-__device__ __forceinline__ void cl_load(const ClLevels<M> &P, unsigned char *sm, int rank) {
-    const int t = threadIdx.x, nt = blockDim.x;
+__global__ void __launch_bounds__(kPackThreads) k_cl_pack(ClLevels<M> P, int *__restrict__ ctl) {
+    griddep_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ctl[C_PACK] += 1;   // set-ups of this step call
+    const int rank = blockIdx.x, t = blockIdx.y * kPackThreads + threadIdx.x, nt = kPackSlices * kPackThreads;
+    unsigned char *im = P.image + (size_t)rank * P.img;
     for (int l = 0; l < P.n; ++l) {
         const ClLevel<M> &L = P.L[l];
         const int s = cl_start(P, L, rank);
-        M *x = (M *)(sm + L.ox), *b = (M *)(sm + L.ob), *id = (M *)(sm + L.oi);
-        M *c0 = (M *)(sm + L.oc[0]), *c1 = (M *)(sm + L.oc[1]), *c2 = (M *)(sm + L.oc[2]);
-        for (int c = t; c < L.nloc; c += nt) { x[c] = M(0); b[c] = M(0); }
-        const int pc = L.ps - L.ny * L.nz;   // unused cells at the end of a column
-        for (int c = t; c < L.ncol * pc; c += nt) {
-            const int q = c / pc, o = q * L.ps + L.ny * L.nz + c - q * pc;
-            id[o] = c0[o] = c1[o] = M(0);
-            if (DIM == 3) c2[o] = M(0);
-        }
-        for (int c = t; c < L.ncol * L.ny * L.nz; c += nt) {   // x fastest: rows of the global arrays
-            int q, j, k;
-            split3(c, L.ncol, L.rncol, L.ny, L.rny, q, j, k);
-            const int i = s - L.G + q, o = q * L.ps + j + L.ny * k;
+        M *id = (M *)(im + L.oi), *c0 = (M *)(im + L.oc[0]), *c1 = (M *)(im + L.oc[1]), *c2 = (M *)(im + L.oc[2]);
+        for (int o = t; o < L.nloc; o += nt) {
+            const int q = o / L.ps, m = o - q * L.ps, k = m / L.ny, j = m - k * L.ny, i = s - L.G + q;
+            const bool in = i >= 0 && k < L.nz;
             M v0 = M(0), v1 = M(0), v2 = M(0), vi = M(0);
-            if (i >= 0 && i < L.nx) {
+            if (in && i < L.nx) {
                 const int gc = i + L.nx * (j + L.ny * k);
                 v1 = L.c[1][i + L.nx * (j + (L.ny + 1) * k)];
                 if (DIM == 3) v2 = L.c[2][gc];
                 vi = L.idiag[gc];
             }
-            if (i >= 0 && i <= L.nx) v0 = L.c[0][i + (L.nx + 1) * (j + L.ny * k)];   // i = nx: the outlet, x = 0 beyond it
+            if (in && i <= L.nx) v0 = L.c[0][i + (L.nx + 1) * (j + L.ny * k)];   // i = nx: the outlet, x = 0 beyond it
             id[o] = vi;
             c0[o] = v0;
             c1[o] = v1;
@@ -167,54 +183,96 @@ __device__ __forceinline__ void cl_load(const ClLevels<M> &P, unsigned char *sm,
         const ClLevel<M> &C = P.L[last ? l : l + 1];
         const int cs = cl_start(P, C, rank);
         for (int h = t; h < L.ncol * L.ce; h += nt) {
-            int tj, k, q;
-            split3(h, hj, L.rhj, L.nz, 1.0f / (float)L.nz, tj, k, q);
+            const int q = h / L.ce, m = h - q * L.ce, k = m / hj, tj = m - k * hj;
             const int i = s - L.G + q;
 #pragma unroll
             for (int colour = 0; colour < 2; ++colour) {
                 const int j = 2 * tj + ((i + k + colour) & 1);
                 const bool in = i >= 0 && i < L.nx && j < L.ny;
-                ((unsigned short *)(sm + L.ol[colour]))[h] = in ? (unsigned short)(q * L.ps + j + L.ny * k) : kClNone;
+                ((unsigned short *)(im + L.ol[colour]))[h] = in ? (unsigned short)(q * L.ps + j + L.ny * k) : kClNone;
                 if (colour == 0 && !last) {
                     const int qc = (i >> (L.rx >> 1)) - cs + C.G;
-                    ((unsigned short *)(sm + L.op))[h] =
+                    ((unsigned short *)(im + L.op))[h] =
                         in && qc >= 0 && qc < C.ncol ? (unsigned short)(qc * C.ps + (j >> (L.ry >> 1)) + C.ny * (k >> (L.rz >> 1)))
                                                      : (unsigned short)0;
                 }
             }
         }
+        for (int r = t; r <= P.nc; r += nt) ((short *)(im + L.os))[r] = (short)cl_start(P, L, r);
     }
-}
-
-// rows of the coarsest level's inverse on which x is needed, in local cell
-// order without the columns' padding; written by an earlier kernel
-template <typename M>
-__device__ __forceinline__ void cl_load_inverse(const ClLevels<M> &P, unsigned char *sm, int rank) {
+    // rows of the coarsest level's inverse
     const ClLevel<M> &L = P.L[P.n - 1];
-    const ClRange R = cl_range(P, L, rank, L.E);
-    const int ne = L.nx * L.ny * L.nz, pl = L.ny * L.nz;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    M *inv = (M *)(sm + P.oinv);
-    for (int row = warp; row < (R.q1 - R.q0) * pl; row += nw) {
+    const ClRange R = cl_range(P, L, rank, cl_exact_depth(P));
+    const int ne = L.nx * L.ny * L.nz, pl = L.ny * L.nz, nr = (R.q1 - R.q0) * pl;
+    M *inv = (M *)(im + P.oinv);
+    for (int o = t; o < nr * ne; o += nt) {
+        const int row = o / ne, q = row / pl, m = row - q * pl;
+        inv[o] = P.inv[(size_t)(R.s - L.G + R.q0 + q + L.nx * m) * ne + o - row * ne];
+    }
+    for (int row = t; row < nr; row += nt) {
         const int q = row / pl, m = row - q * pl;
-        const M *src = P.inv + (size_t)(R.s - L.G + R.q0 + q + L.nx * m) * ne;
-        for (int v = lane; v < ne; v += 32) inv[row * ne + v] = src[v];
+        ((unsigned short *)(im + P.orow))[row] = (unsigned short)((R.q0 + q) * L.ps + m);
     }
 }
 
-// sum of the neighbour terms of one row: one after the other (the order of
-// mg_row_off), or the two of a direction first on the smallest levels
-template <int DIM, typename M>
-__device__ __forceinline__ M cl_off(const M *w, const M *x, int c, int ps, int ny, bool paired) {
-    const M a0 = w[0] * x[c - ps], a1 = w[1] * x[c + ps];
-    const M b0 = w[2] * x[c - 1], b1 = w[3] * x[c + 1];
-    M off = a0 + a1;
+// start the copy of the CTA's image into shared memory; x and b cleared
+// meanwhile. cp_async_wait_all and a barrier complete it.
+template <typename M>
+__device__ __forceinline__ void cl_load(const ClLevels<M> &P, unsigned char *sm, int rank) {
+    const unsigned char *im = P.image + (size_t)rank * P.img;
+    for (int q = threadIdx.x * 16; q < P.img; q += blockDim.x * 16) {
+        const unsigned d = (unsigned)__cvta_generic_to_shared(sm + q);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(im + q) : "memory");
+    }
+    for (int l = 0; l < P.n; ++l) {
+        const ClLevel<M> &L = P.L[l];
+        M *x = (M *)(sm + L.ox), *b = (M *)(sm + L.ob);
+        for (int c = threadIdx.x; c < L.nloc; c += blockDim.x) { x[c] = M(0); b[c] = M(0); }
+    }
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// b + the sum of the neighbour terms of one row. FP32: one term after the
+// other (the order of mg_row_off), or the two of a direction first on the
+// smallest levels, as the per-level kernels and the former coarse kernel
+// formed them. FP64 is bound by FP64 issue: fused multiply-adds.
+template <int DIM>
+__device__ __forceinline__ float cl_row_sum(const float *w, const float *x, int c, int ps, int ny, bool paired, float b) {
+    const float a0 = w[0] * x[c - ps], a1 = w[1] * x[c + ps];
+    const float b0 = w[2] * x[c - 1], b1 = w[3] * x[c + 1];
+    float off = a0 + a1;
     off = paired ? off + (b0 + b1) : (off + b0) + b1;
     if (DIM == 3) {
-        const M d0 = w[4] * x[c - ny], d1 = w[5] * x[c + ny];
+        const float d0 = w[4] * x[c - ny], d1 = w[5] * x[c + ny];
         off = paired ? off + (d0 + d1) : (off + d0) + d1;
     }
-    return off;
+    return b + off;
+}
+template <int DIM>
+__device__ __forceinline__ double cl_row_sum(const double *w, const double *x, int c, int ps, int ny, bool, double b) {
+    double t = fma(w[0], x[c - ps], b);
+    t = fma(w[1], x[c + ps], t);
+    t = fma(w[2], x[c - 1], t);
+    t = fma(w[3], x[c + 1], t);
+    if (DIM == 3) {
+        t = fma(w[4], x[c - ny], t);
+        t = fma(w[5], x[c + ny], t);
+    }
+    return t;
+}
+template <int DIM>
+__device__ __forceinline__ float cl_residual(const float *w, const float *x, int c, int ps, int ny, bool paired, float b) {
+    float dg = 0.f;   // the diagonal as it was formed
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) dg += w[2 * a] + w[2 * a + 1];
+    return b - (dg * x[c] - cl_row_sum<DIM>(w, x, c, ps, ny, paired, 0.f));
+}
+template <int DIM>
+__device__ __forceinline__ double cl_residual(const double *w, const double *x, int c, int ps, int ny, bool paired, double b) {
+    double dg = 0.0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) dg += w[2 * a] + w[2 * a + 1];
+    return fma(-dg, x[c], cl_row_sum<DIM>(w, x, c, ps, ny, paired, b));
 }
 // the coefficients of a row, from the low faces of the cell and its high neighbours
 template <int DIM, typename M>
@@ -230,171 +288,273 @@ __device__ __forceinline__ void cl_row(const ClLevel<M> &L, unsigned char *sm, i
     }
 }
 
-// one colour of a red-black sweep on the slab and d columns beyond it (no barrier)
-template <int DIM, typename M>
-__device__ __forceinline__ void cl_sweep(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, int colour, int d,
-                                         int rank) {
+// A thread's cells of a level, K list entries of each colour with their rows
+// in registers: loaded once for the half sweeps of a smoothing step, which
+// then read only x from shared memory. K = 0: any number of entries, the rows
+// read again in every half sweep.
+template <int DIM, typename M, int K> struct ClCells {
+    int c[2][K], dist[2][K];   // local cell; columns outside the slab (a large number: no cell)
+    M w[2][K][2 * DIM], id[2][K], b[2][K];
+    __device__ __forceinline__ void load(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, int rank) {
+        const ClRange R = cl_range(P, L, rank, L.D);
+        const M *bs = (const M *)(sm + L.ob), *ids = (const M *)(sm + L.oi);
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            const int h = R.q0 * L.ce + threadIdx.x + u * blockDim.x;
+            const bool in = h < R.q1 * L.ce;
+            int rem;
+            const int q = div_rem(h, L.ce, L.rce, rem), d = max(max(L.G - q, q - (L.G + R.w - 1)), 0);
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int cell = in ? ((const unsigned short *)(sm + L.ol[a]))[h] : kClNone;
+                const bool ok = cell != kClNone;
+                c[a][u] = ok ? cell : L.ps;   // a cell whose neighbours exist
+                dist[a][u] = ok ? d : 1 << 20;
+                cl_row<DIM, M>(L, sm, c[a][u], w[a][u]);
+                id[a][u] = ids[c[a][u]];
+                b[a][u] = bs[c[a][u]];
+            }
+        }
+    }
+    __device__ __forceinline__ void first(const ClLevel<M> &L, M *x) {
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (dist[0][u] <= L.D) x[c[0][u]] = b[0][u] * id[0][u];
+    }
+    template <int A> __device__ __forceinline__ void sweep(const ClLevel<M> &L, M *x, int d) {
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (dist[A][u] <= d)
+                x[c[A][u]] = cl_row_sum<DIM>(w[A][u], x, c[A][u], L.ps, L.ny, L.paired, b[A][u]) * id[A][u];
+    }
+    __device__ __forceinline__ void residual(const ClLevel<M> &L, const M *x, M *rs) {
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int u = 0; u < K; ++u)
+                if (dist[a][u] == 0)
+                    rs[c[a][u] - L.G * L.ps] = cl_residual<DIM>(w[a][u], x, c[a][u], L.ps, L.ny, L.paired, b[a][u]);
+    }
+    __device__ __forceinline__ void prolong(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, int rank, M *x,
+                                            const M *xc, int d) {
+        const int q0 = cl_range(P, L, rank, L.D).q0;
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+            if (dist[0][u] <= d)
+                x[c[0][u]] += xc[((const unsigned short *)(sm + L.op))[q0 * L.ce + threadIdx.x + u * blockDim.x]];
+    }
+};
+template <int DIM, typename M> struct ClCells<DIM, M, 0> {
+    const ClLevels<M> *P;
+    unsigned char *sm;
+    int rank;
+    __device__ __forceinline__ void load(const ClLevels<M> &P_, const ClLevel<M> &, unsigned char *sm_, int rank_) {
+        P = &P_;
+        sm = sm_;
+        rank = rank_;
+    }
+    template <typename F> __device__ __forceinline__ void each(const ClLevel<M> &L, int colour, int d, F f) {
+        const unsigned short *lst = (const unsigned short *)(sm + L.ol[colour]);
+        const ClRange R = cl_range(*P, L, rank, d);
+        for (int h = R.q0 * L.ce + threadIdx.x; h < R.q1 * L.ce; h += blockDim.x) {
+            const int c = lst[h];
+            if (c != kClNone) f(c, h);
+        }
+    }
+    __device__ __forceinline__ void first(const ClLevel<M> &L, M *x) {
+        const M *b = (const M *)(sm + L.ob), *id = (const M *)(sm + L.oi);
+        each(L, 0, L.D, [&](int c, int) { x[c] = b[c] * id[c]; });
+    }
+    template <int A> __device__ __forceinline__ void sweep(const ClLevel<M> &L, M *x, int d) {
+        const M *b = (const M *)(sm + L.ob), *id = (const M *)(sm + L.oi);
+        each(L, A, d, [&](int c, int) {
+            M w[2 * DIM];
+            cl_row<DIM, M>(L, sm, c, w);
+            x[c] = cl_row_sum<DIM>(w, x, c, L.ps, L.ny, L.paired, b[c]) * id[c];
+        });
+    }
+    __device__ __forceinline__ void residual(const ClLevel<M> &L, const M *x, M *rs) {
+        const M *b = (const M *)(sm + L.ob);
+        for (int a = 0; a < 2; ++a)
+            each(L, a, 0, [&](int c, int) {
+                M w[2 * DIM];
+                cl_row<DIM, M>(L, sm, c, w);
+                rs[c - L.G * L.ps] = cl_residual<DIM>(w, x, c, L.ps, L.ny, L.paired, b[c]);
+            });
+    }
+    __device__ __forceinline__ void prolong(const ClLevels<M> &, const ClLevel<M> &L, unsigned char *, int, M *x, const M *xc,
+                                            int d) {
+        const unsigned short *par = (const unsigned short *)(sm + L.op);
+        each(L, 0, d, [&](int c, int h) { x[c] += xc[par[h]]; });
+    }
+};
+
+// pre-smoothing from x = 0 and the residual of the slab's cells; no barrier after it
+template <int DIM, typename M, int K>
+__device__ __forceinline__ void cl_pre(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, int rank) {
     M *x = (M *)(sm + L.ox);
-    const M *b = (const M *)(sm + L.ob), *id = (const M *)(sm + L.oi);
-    const unsigned short *lst = (const unsigned short *)(sm + L.ol[colour]);
-    const ClRange R = cl_range(P, L, rank, d);
-    for (int h = R.q0 * L.ce + threadIdx.x; h < R.q1 * L.ce; h += blockDim.x) {
-        const int c = lst[h];
-        if (c == kClNone) continue;
-        M w[2 * DIM];
-        cl_row<DIM, M>(L, sm, c, w);
-        x[c] = (b[c] + cl_off<DIM, M>(w, x, c, L.ps, L.ny, L.paired)) * id[c];
+    ClCells<DIM, M, K> cells;
+    cells.load(P, L, sm, rank);
+    cells.first(L, x);
+    __syncthreads();
+    for (int s = 0; s < L.nu; ++s) {
+        if (s > 0) {
+            cells.template sweep<0>(L, x, L.D - 2 * s);
+            __syncthreads();
+        }
+        cells.template sweep<1>(L, x, s == L.nu - 1 ? 1 : L.D - 2 * s - 1);   // the last one is read by the residual only
+        __syncthreads();
+    }
+    cells.residual(L, x, (M *)(sm + P.ors));
+}
+// prolongation to the colour-0 cells and post-smoothing; no barrier after it
+template <int DIM, typename M, int K>
+__device__ __forceinline__ void cl_post(const ClLevels<M> &P, int l, unsigned char *sm, int rank) {
+    const ClLevel<M> &L = P.L[l];
+    M *x = (M *)(sm + L.ox);
+    ClCells<DIM, M, K> cells;
+    cells.load(P, L, sm, rank);
+    cells.prolong(P, L, sm, rank, x, (const M *)(sm + P.L[l + 1].ox), L.E + 2 * L.nu);
+    for (int s = 0; s < L.nu; ++s) {
+        __syncthreads();
+        cells.template sweep<1>(L, x, L.E + 2 * (L.nu - s) - 1);
+        __syncthreads();
+        cells.template sweep<0>(L, x, L.E + 2 * (L.nu - s) - 2);
     }
 }
-// the first colour-0 half sweep from x = 0, on every column that holds b
-template <typename M>
-__device__ __forceinline__ void cl_first_sweep(const ClLevels<M> &P, const ClLevel<M> &L, unsigned char *sm, int rank) {
-    M *x = (M *)(sm + L.ox);
-    const M *b = (const M *)(sm + L.ob), *id = (const M *)(sm + L.oi);
-    const unsigned short *lst = (const unsigned short *)(sm + L.ol[0]);
-    const ClRange R = cl_range(P, L, rank, L.G);
-    for (int h = R.q0 * L.ce + threadIdx.x; h < R.q1 * L.ce; h += blockDim.x) {
-        const int c = lst[h];
-        if (c != kClNone) x[c] = b[c] * id[c];
-    }
+// entries of a colour that a thread of the CTA takes
+template <typename M> __device__ __forceinline__ int cl_per_thread(const ClLevels<M> &P, const ClLevel<M> &L, int rank) {
+    const ClRange R = cl_range(P, L, rank, L.D);
+    return ((R.q1 - R.q0) * L.ce + (int)blockDim.x - 1) / (int)blockDim.x;
 }
 
-// residual of the slab's cells, then b of the next level = the sum over the
-// children (x fastest), stored into every CTA whose ghosts cover it (on the
-// coarsest level, into every CTA's gathered copy)
+// b of the next level = the sum over the children's residuals (x fastest),
+// stored into every CTA whose ghosts cover it (on the coarsest level, into
+// every CTA's gathered copy)
 template <int DIM, typename M>
 __device__ __forceinline__ void cl_restrict(const ClLevels<M> &P, int l, unsigned char *sm, int rank) {
     const ClLevel<M> &L = P.L[l], &C = P.L[l + 1];
-    M *rs = (M *)(sm + P.ors);
-    const ClRange F = cl_range(P, L, rank, 0);
-    {
-        const M *x = (const M *)(sm + L.ox), *b = (const M *)(sm + L.ob);
-        const unsigned short *l0 = (const unsigned short *)(sm + L.ol[0]), *l1 = (const unsigned short *)(sm + L.ol[1]);
-        const int n = F.w * L.ce;
-        for (int h = threadIdx.x; h < 2 * n; h += blockDim.x) {
-            const int c = h < n ? l0[F.q0 * L.ce + h] : l1[F.q0 * L.ce + h - n];
-            if (c == kClNone) continue;
-            M w[2 * DIM], dg = M(0);
-            cl_row<DIM, M>(L, sm, c, w);
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) dg += w[2 * a] + w[2 * a + 1];   // the diagonal as it was formed
-            rs[c - F.q0 * L.ps] = b[c] - (dg * x[c] - cl_off<DIM, M>(w, x, c, L.ps, L.ny, L.paired));
-        }
-    }
-    __syncthreads();
+    const M *rs = (const M *)(sm + P.ors);
+    const int fw = cl_range(P, L, rank, 0).w;
     const ClRange S = cl_range(P, C, rank, 0);
     const bool last = l + 1 == P.n - 1;
     M *bc = (M *)(sm + C.ob), *bx = (M *)(sm + P.obx);
-    const float rw = 1.0f / (float)S.w;
-    for (int q = threadIdx.x; q < S.w * C.ny * C.nz; q += blockDim.x) {
-        int p, J, K;
-        split3(q, S.w, rw, C.ny, C.rny, p, J, K);
+    const int pl = C.ny * C.nz;
+    const float rpl = 1.0f / (float)pl;
+    for (int q = threadIdx.x; q < S.w * pl; q += blockDim.x) {
+        int m, J;
+        const int p = div_rem(q, pl, rpl, m), K = DIM == 3 ? div_rem(m, C.ny, C.rny, J) : (J = m, 0);
+        const int base = p * L.rx * L.ps + J * L.ry + L.ny * (K * L.rz);
         M acc = M(0);
-        for (int kk = K * L.rz; kk < min((K + 1) * L.rz, L.nz); ++kk)
-            for (int jj = J * L.ry; jj < min((J + 1) * L.ry, L.ny); ++jj)
-                for (int pp = p * L.rx; pp < min((p + 1) * L.rx, F.w); ++pp) acc += rs[pp * L.ps + jj + L.ny * kk];
+#pragma unroll
+        for (int kk = 0; kk < (DIM == 3 ? 2 : 1); ++kk)
+#pragma unroll
+            for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp)
+                    if (kk < L.rz && jj < L.ry && pp < L.rx && K * L.rz + kk < L.nz && J * L.ry + jj < L.ny &&
+                        p * L.rx + pp < fw)
+                        acc += rs[base + pp * L.ps + jj + L.ny * kk];
         const int i = S.s + p;
         if (last) {
-            const int gc = i + C.nx * (J + C.ny * K);
+            const int gc = i + C.nx * m;
             for (int r = 0; r < P.nc; ++r) cl_store(cl_addr(bx + gc, r), acc);
         } else {
-            const int m = J + C.ny * K;
             bc[(p + C.G) * C.ps + m] = acc;
-            cl_push(P, C, bc, i, m, C.G, rank, acc);
+            cl_push(P, C, sm, bc, i, m, C.G, rank, acc);
         }
     }
 }
 
-// x = inverse * b on the coarsest level, on the columns that need it: a warp
-// per row, lanes over the columns of the inverse, four rows at a time
+// x = inverse * b on the coarsest level: a warp per row, lanes over the
+// columns of the inverse, two rows at a time (a CTA meets every phase once per
+// iteration with few warps, so that code size costs instruction fetches:
+// eight rows at a time took 3950 cycles for 5 rows per warp)
 template <typename M> __device__ __forceinline__ void cl_exact(const ClLevels<M> &P, unsigned char *sm, int rank) {
+    constexpr int U = 2;
     const ClLevel<M> &L = P.L[P.n - 1];
-    const ClRange R = cl_range(P, L, rank, L.E);
+    const ClRange R = cl_range(P, L, rank, cl_exact_depth(P));
     const int ne = L.nx * L.ny * L.nz, pl = L.ny * L.nz, nr = (R.q1 - R.q0) * pl;
     const M *inv = (const M *)(sm + P.oinv), *bx = (const M *)(sm + P.obx);
     M *x = (M *)(sm + L.ox);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int r0 = warp; r0 < nr; r0 += 4 * nw) {
-        M acc[4] = {M(0), M(0), M(0), M(0)};
+#pragma unroll 1
+    for (int r0 = warp; r0 < nr; r0 += U * nw) {
+        M acc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) acc[u] = M(0);
         for (int m = lane; m < ne; m += 32) {
             const M v = bx[m];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (r0 + u * nw < nr) acc[u] += inv[(r0 + u * nw) * ne + m] * v;
+            for (int u = 0; u < U; ++u)
+                if (r0 + u * nw < nr) {
+                    const M a = inv[(r0 + u * nw) * ne + m];
+                    acc[u] = sizeof(M) == sizeof(double) ? (M)fma((double)a, (double)v, (double)acc[u]) : acc[u] + a * v;
+                }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u)
                 if (r0 + u * nw < nr) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int row = r0 + u * nw, q = row / pl;
-            if (lane == 0 && row < nr) x[(R.q0 + q) * L.ps + row - q * pl] = acc[u];
+        for (int u = 0; u < U; ++u) {
+            const int row = r0 + u * nw;
+            if (lane == 0 && row < nr) {
+                const int c = ((const unsigned short *)(sm + P.orow))[row];
+                x[c] = acc[u];
+                if (cl_exact_depth(P) < L.E) {
+                    const int q = c / L.ps;
+                    cl_push(P, L, sm, x, R.s - L.G + q, c - q * L.ps, L.E, rank, acc[u]);
+                }
+            }
         }
     }
-}
-
-// x of the colour-0 cells += the coarser level's x
-template <typename M> __device__ __forceinline__ void cl_prolong(const ClLevels<M> &P, int l, unsigned char *sm, int rank) {
-    const ClLevel<M> &L = P.L[l];
-    M *x = (M *)(sm + L.ox);
-    const M *xc = (const M *)(sm + P.L[l + 1].ox);
-    const unsigned short *lst = (const unsigned short *)(sm + L.ol[0]), *par = (const unsigned short *)(sm + L.op);
-    const ClRange R = cl_range(P, L, rank, L.E + 2 * L.nu);
-    for (int h = R.q0 * L.ce + threadIdx.x; h < R.q1 * L.ce; h += blockDim.x) {
-        const int c = lst[h];
-        if (c != kClNone) x[c] += xc[par[h]];
-    }
+    if (cl_exact_depth(P) < L.E) cl_sync(P.nc);
+    else __syncthreads();
 }
 
 // The V-cycle over the cluster's levels. On entry the first level's b (with
 // its ghosts; the gathered b when it is the coarsest) is in place and a
 // cluster barrier has been passed since. On return x of the first level is
 // valid on E columns beyond the slab; no barrier has been passed since its
-// last half sweep (the solution, when it is the coarsest level).
+// last half sweep.
 template <int DIM, typename M>
 __device__ __forceinline__ void cl_vcycle(const ClLevels<M> &P, unsigned char *sm, int rank) {
+    constexpr bool F32 = sizeof(M) == sizeof(float);
     for (int l = 0; l < P.n - 1; ++l) {
         const ClLevel<M> &L = P.L[l];
-        cl_first_sweep<M>(P, L, sm, rank);
+        const int per = cl_per_thread(P, L, rank);
+        if (per <= 1) cl_pre<DIM, M, 1>(P, L, sm, rank);
+        else if (per <= 2) cl_pre<DIM, M, 2>(P, L, sm, rank);
+        else if (F32 && per <= 4) cl_pre<DIM, M, F32 ? 4 : 0>(P, L, sm, rank);
+        else cl_pre<DIM, M, 0>(P, L, sm, rank);
         __syncthreads();
-        for (int s = 0; s < L.nu; ++s) {
-            if (s > 0) {
-                cl_sweep<DIM, M>(P, L, sm, 0, L.D - 2 * s, rank);
-                __syncthreads();
-            }
-            // the last one is read by the residual only
-            cl_sweep<DIM, M>(P, L, sm, 1, s == L.nu - 1 ? 1 : L.D - 2 * s - 1, rank);
-            __syncthreads();
-        }
         cl_restrict<DIM, M>(P, l, sm, rank);
         cl_sync(P.nc);
     }
     cl_exact<M>(P, sm, rank);
     for (int l = P.n - 2; l >= 0; --l) {
         const ClLevel<M> &L = P.L[l];
-        __syncthreads();
-        cl_prolong<M>(P, l, sm, rank);
-        for (int s = 0; s < L.nu; ++s) {
-            __syncthreads();
-            cl_sweep<DIM, M>(P, L, sm, 1, L.E + 2 * (L.nu - s) - 1, rank);
-            __syncthreads();
-            cl_sweep<DIM, M>(P, L, sm, 0, L.E + 2 * (L.nu - s) - 2, rank);
-        }
+        const int per = cl_per_thread(P, L, rank);
+        if (l < P.n - 2) __syncthreads();
+        if (per <= 1) cl_post<DIM, M, 1>(P, l, sm, rank);
+        else if (per <= 2) cl_post<DIM, M, 2>(P, l, sm, rank);
+        else if (F32 && per <= 4) cl_post<DIM, M, F32 ? 4 : 0>(P, l, sm, rank);
+        else cl_post<DIM, M, 0>(P, l, sm, rank);
     }
 }
 
 // The V-cycle below the per-level kernels: b of the first level from b_top,
-// its x to x_top. Coefficients (fixed during a solve) are loaded before the
+// its x to x_top. The image (fixed during a solve) is copied in before the
 // grid-dependency wait.
 template <int DIM, typename M>
 __global__ void __launch_bounds__(512, 1) k_mg_cluster(ClLevels<M> P, const M *__restrict__ b_top, M *__restrict__ x_top) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int rank = cl_rank();
     const ClLevel<M> &L = P.L[0];
-    cl_load<DIM, M>(P, sm, rank);
-    cl_load_inverse<M>(P, sm, rank);
+    cl_load<M>(P, sm, rank);
+    cp_async_wait_all();
     __syncthreads();
     griddep_wait();
     M *b = (M *)(sm + L.ob), *bx = (M *)(sm + P.obx);
@@ -451,66 +611,83 @@ struct ClSolve {
 };
 struct ClControl {        // one per CTA, written by its thread 0 from totals all CTAs share
     double target, itarget, rz0, rz1;
+    double test2;         // square of the norm the iteration stops at
+    double rrz;           // 1 / rz1
     double alpha, beta;
     float alpha_f, beta_f;
     int more;
 };
 
-// totals over the cluster of nv FP64 values per thread, valid in warp 0 of
-// every CTA (same order everywhere: same result). Two buffers, alternating: a
-// CTA may store for the next reduction while another still reads this one.
-template <typename M>
-__device__ __forceinline__ void cl_sum(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, double *v, int nv) {
-    double *sh = (double *)(sm + P.ored), *slot = sh + 512 + buf * 4 * kMaxCluster;
-    const int t = threadIdx.x, nt = blockDim.x;
-    for (int q = 0; q < nv; ++q) {
-        __syncthreads();
-        sh[t] = v[q];
-        __syncthreads();
-        if (t < 32) {
-            double s = sh[t];
-            for (int m = t + 32; m < nt; m += 32) s += sh[m];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (t < P.nc) cl_store(cl_addr(slot + q * kMaxCluster + rank, t), s);
-        }
-    }
+// totals over the cluster of nv FP64 values per thread (at most four; a warp
+// sums each), valid in warp 0 of every CTA (same order everywhere: same
+// result). Two buffers, alternating: a CTA may store for the next reduction
+// while another still reads this one. aside() is called by a warp that does
+// not sum.
+struct ClNothing { __device__ __forceinline__ void operator()() const {} };
+template <typename M, typename F = ClNothing>
+__device__ __forceinline__ void cl_sum(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, double *v, int nv,
+                                       F aside = F()) {
+    const int t = threadIdx.x, nt = blockDim.x, warp = t >> 5, lane = t & 31;
+    double *sh = (double *)(sm + P.ored), *slot = sh + 4 * nt + buf * 4 * kMaxCluster;
+    for (int q = 0; q < nv; ++q) sh[q * nt + t] = v[q];
+    __syncthreads();
+    if (warp < nv) {
+        const double *a = sh + warp * nt;
+        double s = 0.0;   // blocks of 128 k threads
+        for (int m = lane; m < nt; m += 128) s += (a[m] + a[m + 32]) + (a[m + 64] + a[m + 96]);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane < P.nc) cl_store(cl_addr(slot + warp * kMaxCluster + rank, lane), s);
+    } else if (warp == 4) aside();
     cl_sync(P.nc);
-    if (t < 32)
+    if (warp == 0)
         for (int q = 0; q < nv; ++q) {
-            double s = t < P.nc ? slot[q * kMaxCluster + t] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            double s = lane < P.nc ? slot[q * kMaxCluster + lane] : 0.0;
+            for (int o = P.nc >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             v[q] = s;
         }
     buf ^= 1;
 }
 // the same for one value of the vectors' type: FP64 as above, FP32 in
 // compensated pairs; the total is valid in thread 0
-template <typename M>
-__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc64 a) {
-    cl_sum(P, sm, rank, buf, &a.s, 1);
+template <typename M, typename F = ClNothing>
+__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc64 a, F aside = F()) {
+    cl_sum(P, sm, rank, buf, &a.s, 1, aside);
     return a.s;
 }
-template <typename M>
-__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc32 a) {
-    float2 *slot = (float2 *)((double *)(sm + P.ored) + 512 + buf * 4 * kMaxCluster);
-    const int t = threadIdx.x;
+template <typename M, typename F = ClNothing>
+__device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm, int rank, int &buf, DotAcc32 a, F aside = F()) {
+    const int t = threadIdx.x, nw = blockDim.x >> 5, warp = t >> 5, lane = t & 31;
+    float2 *sh = (float2 *)(sm + P.ored), *slot = (float2 *)((double *)(sm + P.ored) + 4 * blockDim.x + buf * 4 * kMaxCluster);
+    auto tree = [](float &s, float &e, int from) {
+#pragma unroll 1
+        for (int o = from; o > 0; o >>= 1) {
+            const float so = __shfl_xor_sync(0xffffffffu, s, o), eo = __shfl_xor_sync(0xffffffffu, e, o);
+            float sn, se;
+            two_sum(s, so, sn, se);
+            s = sn;
+            e += eo + se;
+        }
+    };
     float s = a.s, e = a.e;
-    block_pair_f(s, e);
-    if (t < 32) {
-        s = __shfl_sync(0xffffffffu, s, 0);
-        e = __shfl_sync(0xffffffffu, e, 0);
-        if (t < P.nc) {
-            const unsigned d = cl_addr(slot + rank, t);
+    tree(s, e, 16);
+    if (lane == 0) sh[warp] = make_float2(s, e);
+    __syncthreads();
+    if (warp == 0) {
+        s = lane < nw ? sh[lane].x : 0.f;
+        e = lane < nw ? sh[lane].y : 0.f;
+        tree(s, e, 16);
+        if (lane < P.nc) {
+            const unsigned d = cl_addr(slot + rank, lane);
             cl_store(d, s);
             cl_store(d + 4, e);
         }
-    }
+    } else if (warp == 4) aside();
     cl_sync(P.nc);
     double tot = 0.0;
-    if (t < 32) {
-        s = t < P.nc ? slot[t].x : 0.f;
-        e = t < P.nc ? slot[t].y : 0.f;
-        warp_sum_pair(s, e);
+    if (warp == 0) {
+        s = lane < P.nc ? slot[lane].x : 0.f;
+        e = lane < P.nc ? slot[lane].y : 0.f;
+        tree(s, e, P.nc >> 1);
         if (t == 0) tot = (double)s + (double)e;
     }
     buf ^= 1;
@@ -521,13 +698,27 @@ __device__ __forceinline__ double cl_dot(const ClLevels<M> &P, unsigned char *sm
 #define CL_OWN_CELLS()                                                                                        \
     for (int g_ = t, pc, j, k_; g_ < S.w * L.ny && (split3(g_, S.w, rw, L.ny, L.rny, pc, j, k_), true); g_ += blockDim.x)
 
-// groups of own cells that one thread of the launched CG kernels sums
-// (launch_rpt): own column pc, rows j0 + u by for u < rpt
-#define CL_ROW_GROUPS(rpt)                                                                               \
-    for (int g_ = t, nb_ = (L.ny + A.by * (rpt) - 1) / (A.by * (rpt)), pc, ty_, blk_; g_ < S.w * A.by * nb_; \
-         g_ += blockDim.x)                                                                               \
-        if (split3(g_, A.by, rby, nb_, 1.0f / (float)nb_, ty_, blk_, pc); true)                          \
-            if (const int j0 = blk_ * A.by * (rpt) + ty_; j0 < L.ny)
+// own cells of level 0, a column after the other: position o = pc ps + j in the
+// slab's columns, local cell o + G ps
+#define CL_COLUMN_CELLS()                                                                                     \
+    for (int g_ = t, pc, j, o; g_ < S.w * L.ny && (pc = div_rem(g_, L.ny, L.rny, j), o = pc * ps + j, true); g_ += blockDim.x)
+
+// sums of the groups of own cells that one thread of the launched CG kernels
+// takes (launch_groups): products f of own column pc, rows j0 + u by for u < rpt
+template <typename T>
+__device__ __forceinline__ typename DotAcc<T>::type cl_group_sums(const T *f, int w, int ny, int ps, int by, int rpt) {
+    typename DotAcc<T>::type acc;
+    const int nb = (ny + by * rpt - 1) / (by * rpt), ng = by * nb;
+    const float rng = 1.0f / (float)ng, rby = 1.0f / (float)by;
+    for (int g = threadIdx.x; g < w * ng; g += blockDim.x) {
+        int m, ty;
+        const int pc = div_rem(g, ng, rng, m), blk = div_rem(m, by, rby, ty);
+        T a = T(0);
+        for (int u = 0, j = blk * by * rpt + ty; u < rpt && j < ny; ++u, j += by) a += f[pc * ps + j];
+        acc.add(a);
+    }
+    return acc;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve A) {
@@ -538,13 +729,14 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
     const ClLevel<T> &L = P.L[0];
     const int ps = L.ps;
     const ClRange S = cl_range(P, L, rank, 0);
-    cl_load<2, T>(P, sm, rank);
-    cl_load_inverse<T>(P, sm, rank);
+    cl_load<T>(P, sm, rank);
     T *x = (T *)(sm + L.ox), *r = (T *)(sm + L.ob), *bx = (T *)(sm + P.obx);
     T *p = (T *)(sm + A.op) - (L.G - 1) * ps, *Ap = (T *)(sm + A.oap) - (L.G - 1) * ps, *e = (T *)(sm + A.oe) - (L.G - 1) * ps;
     for (int c = t + (L.G - 1) * ps; c < (L.G + S.w + 1) * ps; c += blockDim.x) { p[c] = T(0); Ap[c] = T(0); }
-    const float rw = 1.0f / (float)S.w, rby = 1.0f / (float)A.by;
+    T *prod = (T *)(sm + P.ors);   // products of a dot, by own cell
+    const float rw = 1.0f / (float)S.w;
     int buf = 0, its = 0, outer = 0, nan_seen = 0, notconv = 0;
+    cp_async_wait_all();
     cl_sync(P.nc);   // every CTA's shared memory is ready for remote stores
     griddep_wait();
 
@@ -555,7 +747,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
         if (P.n == 1)
             for (int m = 0; m < P.nc; ++m) cl_store(cl_addr(bx + S.s + pc + L.nx * j, m), rc);
         else
-            cl_push(P, L, r, S.s + pc, j, L.G, rank, rc);
+            cl_push(P, L, sm, r, S.s + pc, j, L.G, rank, rc);
     };
 
     double qbar = 0.0, qsum[1] = {0.0};
@@ -592,6 +784,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
         const bool bad = !(isfinite(bn) && isfinite(rn));
         K.target = A.rtol * (bn > 0.0 ? bn : rn);
         K.itarget = fmax(kInnerRtol * rn, kTripMargin * K.target);
+        K.test2 = MIXED ? K.itarget * K.itarget : K.target * K.target;
         K.rz0 = 0.0;
         K.more = !bad && rn > K.target;
         nan_seen |= bad;
@@ -615,7 +808,8 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             __syncthreads();
             typename DotAcc<T>::type dz;   // r.z: a colour-0 cell with its row partner (level 0 on its own: cell by cell)
             for (int g = t; g < ((S.w + 1) >> 1) * L.ny; g += blockDim.x) {
-                const int tp = g / L.ny, j = g - tp * L.ny, lo = (2 * tp + L.G) * ps + j, odd = (S.s + j) & 1;
+                int j;
+                const int tp = div_rem(g, L.ny, L.rny, j), lo = (2 * tp + L.G) * ps + j, odd = (S.s + j) & 1;
                 const bool two = 2 * tp + 1 < S.w;
                 const int ca = odd ? lo + ps : lo, cb = odd ? lo : lo + ps;   // colour 0, colour 1
                 T a = T(0);
@@ -627,7 +821,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             const double rz = cl_dot(P, sm, rank, buf, dz);
             if (t == 0) {
                 K.rz1 = rz;
-                K.beta = K.rz0 != 0.0 ? rz / K.rz0 : 0.0;
+                K.beta = K.rz0 != 0.0 ? rz * K.rrz : 0.0;
                 K.beta_f = (float)K.beta;
             }
             __syncthreads();
@@ -636,32 +830,27 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             if constexpr (MIXED) {   // p = z + beta p, Ap = M z + beta Ap, p.Ap
                 const T be = K.beta_f;
                 const bool fresh = be == T(0);
-                CL_ROW_GROUPS(kApplyRows) {
-                    T a = T(0);
-#pragma unroll
-                    for (int u = 0; u < kApplyRows; ++u) {
-                        const int j = j0 + u * A.by;
-                        if (j >= L.ny) break;
-                        const int c = (pc + L.G) * ps + j;
-                        const T zc = x[c];
-                        const T pn = fresh ? zc : zc + be * p[c];
-                        T y = c0[c] * (zc - x[c - ps]);
-                        y += c0[c + ps] * (zc - x[c + ps]);
-                        y += c1[c] * (zc - x[c - 1]);
-                        y += c1[c + 1] * (zc - x[c + 1]);
-                        const T an = fresh ? y : y + be * Ap[c];
-                        p[c] = pn;
-                        Ap[c] = an;
-                        a += pn * an;
-                    }
-                    dp.add(a);
+                CL_COLUMN_CELLS() {
+                    const int c = o + L.G * ps;
+                    const T zc = x[c];
+                    const T pn = fresh ? zc : zc + be * p[c];
+                    T y = c0[c] * (zc - x[c - ps]);
+                    y += c0[c + ps] * (zc - x[c + ps]);
+                    y += c1[c] * (zc - x[c - 1]);
+                    y += c1[c + 1] * (zc - x[c + 1]);
+                    const T an = fresh ? y : y + be * Ap[c];
+                    p[c] = pn;
+                    Ap[c] = an;
+                    prod[o] = pn * an;
                 }
+                __syncthreads();
+                dp = cl_group_sums<T>(prod, S.w, L.ny, ps, A.by, kApplyRows);
             } else {   // p = z + beta p (one ghost column as well), Ap = M p, p.Ap
                 const T be = K.beta;
                 for (int c = t + (L.G - 1) * ps; c < (L.G + S.w + 1) * ps; c += blockDim.x) p[c] = x[c] + be * p[c];
                 __syncthreads();
-                CL_ROW_GROUPS(1) {
-                    const int c = (pc + L.G) * ps + j0;
+                CL_COLUMN_CELLS() {
+                    const int c = o + L.G * ps;
                     const T pv = p[c];
                     T y = c0[c] * (pv - p[c - ps]);
                     y += c0[c + ps] * (pv - p[c + ps]);
@@ -679,30 +868,27 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             __syncthreads();
             const T al = MIXED ? (T)K.alpha_f : (T)K.alpha;
             typename DotAcc<T>::type dr;
-            CL_ROW_GROUPS(kUpdateRows) {   // x += alpha p, r -= alpha Ap, r.r
-                T a = T(0);
-#pragma unroll
-                for (int u = 0; u < kUpdateRows; ++u) {
-                    const int j = j0 + u * A.by;
-                    if (j >= L.ny) break;
-                    const int c = (pc + L.G) * ps + j;
-                    if constexpr (MIXED) e[c] = it == 0 ? al * p[c] : e[c] + al * p[c];
-                    else A.q[S.s + pc + L.nx * j] += al * p[c];
-                    const T rc = r[c] - al * Ap[c];
-                    put_r(pc, j, rc);
-                    a += rc * rc;
-                }
-                dr.add(a);
+            CL_COLUMN_CELLS() {   // x += alpha p, r -= alpha Ap, r.r
+                const int c = o + L.G * ps;
+                if constexpr (MIXED) e[c] = it == 0 ? al * p[c] : e[c] + al * p[c];
+                else A.q[S.s + pc + L.nx * j] += al * p[c];
+                const T rc = r[c] - al * Ap[c];
+                put_r(pc, j, rc);
+                if constexpr (MIXED) prod[o] = rc * rc;
+                else dr.add(rc * rc);
             }
-            const double rr = cl_dot(P, sm, rank, buf, dr);
+            if constexpr (MIXED) {
+                __syncthreads();
+                dr = cl_group_sums<T>(prod, S.w, L.ny, ps, A.by, kUpdateRows);
+            }
+            const double rr = cl_dot(P, sm, rank, buf, dr, [&] { if (t == 128) K.rrz = 1.0 / K.rz1; });
             ++it;
             ++its;
             if (t == 0) {
                 K.rz0 = K.rz1;
-                const double rn = sqrt(rr);
-                const bool bad = !isfinite(rn);
+                const bool bad = !isfinite(rr);
                 nan_seen |= bad;
-                bool more = !bad && rn > (MIXED ? K.itarget : K.target);
+                bool more = !bad && rr > K.test2;
                 if (more && it >= A.maxit) { notconv = 1; more = false; }
                 K.more = more;
                 if (rank == 0) A.scal[S_RR] = rr;
@@ -715,7 +901,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
             CL_OWN_CELLS() {
                 const int c = (pc + L.G) * ps + j;
                 x[c] = e[c];
-                cl_push(P, L, x, S.s + pc, j, 1, rank, e[c]);
+                cl_push(P, L, sm, x, S.s + pc, j, 1, rank, e[c]);
             }
             cl_sync(P.nc);
             const T *c0 = (const T *)(sm + L.oc[0]), *c1 = (const T *)(sm + L.oc[1]);
@@ -751,6 +937,7 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
                 bool more = !bad && rn > K.target;
                 if (more && outer >= kMaxOuter) { notconv = 1; more = false; }
                 K.itarget = fmax(kInnerRtol * rn, kTripMargin * K.target);
+                K.test2 = K.itarget * K.itarget;
                 K.rz0 = 0.0;
                 K.more = more;
                 if (rank == 0) A.scal[S_RR] = rr[0];
@@ -774,28 +961,10 @@ __global__ void __launch_bounds__(512, 1) k_solve_cluster(ClLevels<T> P, ClSolve
 // the coarsest level's explicit inverse
 // ---------------------------------------------------------------------------
 // Formed on the first PISO set-up of a step call and every refresh-th one
-// after it (ctl[C_PACK] counts them); in between the stored inverse is kept (a
-// preconditioner component: a stale one changes iterations, not the solution).
-__device__ __forceinline__ bool inverse_due(int *ctl, int refresh) {
-    __shared__ int due_s;
-    if (threadIdx.x == 0) {
-        due_s = ctl[C_PACK] % refresh == 0;
-        ctl[C_PACK] += 1;
-    }
-    __syncthreads();
-    return due_s;
-}
+// after it (ctl[C_PACK], advanced by k_cl_pack, counts them); in between the
+// stored inverse is kept (a preconditioner component: a stale one changes
+// iterations, not the solution).
 
-// FP32: Gauss-Jordan elimination without pivoting, in place (the matrix is
-// symmetric positive definite: the fluid is connected to the Dirichlet
-// outlet). Rows of cells that are solid or have no coefficients decouple; a
-// pivot that vanishes (a pocket cut off from the outlet) drops its row and
-// column. Each thread keeps an 8x8 tile in registers; per pivot its row and
-// column pass through double-buffered shared memory, one block barrier per
-// pivot (128 pivots, against two barriers and 48 shared-memory accesses per
-// thread and pivot for a matrix in shared memory). Every entry sees the same
-// operations in the same order whatever the layout.
-constexpr int kGjThreads = 256, kGjTile = 8;
 // f(0), ..., f(N - 1) with the index a constant from the start, so that an
 // array it indexes is a set of registers (choices between elements of a loop
 // unrolled later are made by address, which puts the array in local memory)
@@ -808,17 +977,34 @@ template <typename F, int... I> __device__ __forceinline__ void static_for(F f, 
 template <int N, typename F> __device__ __forceinline__ void static_for(F f) {
     static_for(f, std::make_integer_sequence<int, N>{});
 }
+
+// FP32: Gauss-Jordan elimination without pivoting, in place (the matrix is
+// symmetric positive definite: the fluid is connected to the Dirichlet
+// outlet). Rows of cells that are solid or have no coefficients decouple; a
+// pivot that vanishes (a pocket cut off from the outlet) drops its row and
+// column. One CTA; each thread keeps an 8x8 tile of the matrix in registers,
+// and the pivots go eight at a time: the 8x8 pivot tile (one warp), then its
+// rows and columns (a thread per column and per row), then the eight rank-one
+// updates of every other tile, four block barriers per eight pivots: 84 us at
+// 128 cells. (Pivot by pivot, one barrier each: 143 us; with the matrix in
+// shared memory: 240 us.) Every entry sees
+// the same operations in the same order whatever the grouping.
+constexpr int kGjThreads = 256, kGjTile = 8;
 template <int DIM>
 __global__ void __launch_bounds__(kGjThreads) k_mg_inverse_dense(GridD g, MG3<float> cc, const float *__restrict__ diag,
                                                                  const uint8_t *__restrict__ fluid,
                                                                  float *__restrict__ inv, int refresh,
-                                                                 int *__restrict__ ctl) {
+                                                                 const int *__restrict__ ctl) {
     static_assert(kGjThreads * kGjTile * kGjTile == kExactCells * kExactCells, "tiles cover the matrix");
     constexpr int B = kGjTile, TC = kExactCells / B;
     griddep_wait();
-    if (!inverse_due(ctl, refresh)) return;
-    __shared__ __align__(16) float rowb[2][kExactCells], colb[2][kExactCells];
-    const int t = threadIdx.x, n = g.ncell, i0 = (t / TC) * B, j0 = (t % TC) * B;
+    if (ctl[C_PACK] % refresh != 0) return;
+    // panels of the pivot tile's rows and columns; per pivot: the multipliers
+    // of every row and the normalised pivot row
+    __shared__ __align__(16) float ak[B][kExactCells], nk[B][kExactCells], rowp[B][kExactCells];
+    __shared__ float colp[kExactCells][B + 1];
+    __shared__ float pa[B][B], pn[B][B], pinv_s[B];   // the same inside the pivot tile, and the reciprocal pivots
+    const int t = threadIdx.x, n = g.ncell, ti = t / TC, tj = t % TC, i0 = ti * B, j0 = tj * B;
     // the (at most 2 DIM + 1) entries of every row, one thread per row
     __shared__ int ecol[kExactCells][2 * DIM + 1];
     __shared__ float eval[kExactCells][2 * DIM + 1];
@@ -850,66 +1036,131 @@ __global__ void __launch_bounds__(kGjThreads) k_mg_inverse_dense(GridD g, MG3<fl
             static_for<B>([&](auto v) { A[u * B + v] = c == v ? w : A[u * B + v]; });
         });
     });
-    // publish row and column k of the current matrix
-    auto publish = [&](int k) {
-        float *rb = rowb[k & 1], *cb = colb[k & 1];
-        const int ku = k - i0, kv = k - j0;
-        if (ku >= 0 && ku < B)
-            static_for<B>([&](auto v) {
-                float a = 0.f;
-                static_for<B>([&](auto u) { a = ku == u ? A[u * B + v] : a; });
-                rb[j0 + v] = a;
-            });
-        if (kv >= 0 && kv < B)
-            static_for<B>([&](auto u) {
-                float a = 0.f;
-                static_for<B>([&](auto v) { a = kv == v ? A[u * B + v] : a; });
-                cb[i0 + u] = a;
-            });
-    };
-    publish(0);
-    for (int k = 0; k < n; ++k) {
+#pragma unroll 1
+    for (int kb = 0; kb * B < n; ++kb) {
+        if (ti == kb) static_for<B * B>([&](auto q) { rowp[q / B][j0 + q % B] = A[q]; });
+        if (tj == kb) static_for<B * B>([&](auto q) { colp[i0 + q / B][q % B] = A[q]; });
         __syncthreads();
-        const float *rb = rowb[k & 1], *cb = colb[k & 1];
-        const float pv = rb[k];
-        const bool skip = !(pv > 0.f);
-        const float pinv = skip ? 0.f : 1.f / pv;
-        float nk[B], ai[B];
-        static_for<B>([&](auto v) {
-            nk[v] = rb[j0 + v] * pinv;   // the normalised pivot row
-            ai[v] = cb[i0 + v];
-        });
-        const int ku = k - i0, kv = k - j0;
-        if (!skip) static_for<B * B>([&](auto q) { A[q] = fmaf(-ai[q / B], nk[q % B], A[q]); });
-        if (kv >= 0 && kv < B)
-            static_for<B * B>([&](auto q) { A[q] = q % B == kv ? (skip ? 0.f : -ai[q / B] * pinv) : A[q]; });
-        if (ku >= 0 && ku < B)
-            static_for<B * B>([&](auto q) {
-                A[q] = q / B == ku ? (skip ? 0.f : (q % B == kv ? pinv : nk[q % B])) : A[q];
+        if (t < 32) {   // the pivot tile: lane v < 8 holds its column v
+            const int v = t & (B - 1);
+            float p[B];
+            static_for<B>([&](auto u) { p[u] = rowp[u][kb * B + v]; });
+            static_for<B>([&](auto k) {
+                const float pv = __shfl_sync(0xffffffffu, p[k], k);
+                const float pinv = pv > 0.f ? 1.f / pv : 0.f;   // a vanished pivot zeroes its row and column
+                const float nv = p[k] * pinv;
+                static_for<B>([&](auto u) {
+                    const float a = __shfl_sync(0xffffffffu, p[u], k);
+                    if (t == 0) pa[k][u] = a;
+                    p[u] = v == k ? -a * pinv : fmaf(-a, nv, p[u]);
+                });
+                p[k] = v == k ? pinv : nv;
+                if (t < B) pn[k][v] = nv;
+                if (t == 0) pinv_s[k] = pinv;
             });
-        if (k + 1 < n) publish(k + 1);
+            if (t < B) static_for<B>([&](auto u) { rowp[u][kb * B + v] = p[u]; });
+        }
+        __syncthreads();
+        if (t < kExactCells) {   // column t of the pivot rows
+            const int j = t;
+            if (j / B == kb) {
+                static_for<B>([&](auto k) { nk[k][j] = pn[k][j - kb * B]; });
+            } else {
+                float r[B];
+                static_for<B>([&](auto u) { r[u] = rowp[u][j]; });
+                static_for<B>([&](auto k) {
+                    const float v = r[k] * pinv_s[k];
+                    nk[k][j] = v;
+                    static_for<B>([&](auto u) { r[u] = u == k ? v : fmaf(-pa[k][u], v, r[u]); });
+                });
+                static_for<B>([&](auto u) { rowp[u][j] = r[u]; });
+            }
+        } else {                 // row i of the pivot columns
+            const int i = t - kExactCells;
+            if (i / B != kb) {
+                float c[B];
+                static_for<B>([&](auto v) { c[v] = colp[i][v]; });
+                static_for<B>([&](auto k) {
+                    const float a = c[k];
+                    ak[k][i] = a;
+                    static_for<B>([&](auto v) { c[v] = v == k ? -a * pinv_s[k] : fmaf(-a, pn[k][v], c[v]); });
+                });
+                static_for<B>([&](auto v) { colp[i][v] = c[v]; });
+            }
+        }
+        __syncthreads();
+        if (ti == kb) {
+            static_for<B * B>([&](auto q) { A[q] = rowp[q / B][j0 + q % B]; });
+        } else if (tj == kb) {
+            static_for<B * B>([&](auto q) { A[q] = colp[i0 + q / B][q % B]; });
+        } else {
+#pragma unroll 2
+            for (int k = 0; k < B; ++k) {
+                const float4 a0 = *(const float4 *)&ak[k][i0], a1 = *(const float4 *)&ak[k][i0 + 4];
+                const float4 v0 = *(const float4 *)&nk[k][j0], v1 = *(const float4 *)&nk[k][j0 + 4];
+                const float a[B] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                const float v[B] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+                static_for<B * B>([&](auto q) { A[q] = fmaf(-a[q / B], v[q % B], A[q]); });
+            }
+        }
+        __syncthreads();
     }
     static_for<B * B>([&](auto q) {
         if (i0 + q / B < n && j0 + q % B < n) inv[(i0 + q / B) * n + j0 + q % B] = A[q];
     });
 }
 
-// FP64: LDL^T without pivoting in band form (the matrix is symmetric positive
-// definite: the fluid is connected to the Dirichlet outlet), cells ordered
-// with the shortest axis fastest, so that the band is the product of the two
-// shortest extents (4 to about 25 for at most 128 cells), then one thread per
-// column of the inverse solves L D L^T x = e_j: n^2 (2 bw + 1) operations
-// instead of the n^3 of a dense elimination. Rows of cells that are solid or
-// have no coefficients, and of pivots that vanish (a pocket cut off from the
-// outlet), give a zero row and column. (A dense elimination is bound by the
-// SM's two FP64 FMAs per clock: 1.1 ms at 128 cells.)
+// FP64: LDL^T without pivoting in band form, cells ordered with the shortest
+// axis fastest, so that the band is the product of the two shortest extents (4
+// to about 25 for at most 128 cells), then L D L^T x = e_j for every column j
+// of the inverse: n^2 (2 bw + 1) operations instead of the n^3 of a dense
+// elimination, which the SM's two FP64 FMAs per clock take 1.1 ms for at 128
+// cells. What is left is a serial chain along the cells: one warp factorises,
+// and a thread solves one column with the last bw values in registers, the
+// newest one's term added last, so that the chain is one FMA per cell. Blocks
+// of one warp (the factorisation repeated in each) share the columns, since
+// four warps on one SM would be bound by its FP64 rate. Rows of cells that are
+// solid or have no coefficients, and of pivots that vanish, give a zero row
+// and column.
+template <typename M, int W>
+__device__ __forceinline__ void band_solve(const M *B, const M *rD, M *Y, int n, int bw, int col, bool live) {
+    // B[i (bw + 1) + d] = L(i, i - d); Y[i 32 + lane]
+    M win[W];
+    const int lane = threadIdx.x & 31, st = bw + 1;
+#pragma unroll
+    for (int d = 0; d < W; ++d) win[d] = M(0);
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {   // L y = e_col
+        M a = i == col && live ? M(1) : M(0);
+#pragma unroll
+        for (int d = W; d >= 1; --d)
+            if (d <= bw) a = fma(-B[i * st + d], win[d - 1], a);   // entries before the first cell are 0
+#pragma unroll
+        for (int d = W - 1; d > 0; --d) win[d] = win[d - 1];
+        win[0] = a;
+        Y[i * 32 + lane] = a;
+    }
+#pragma unroll
+    for (int d = 0; d < W; ++d) win[d] = M(0);
+#pragma unroll 1
+    for (int i = n - 1; i >= 0; --i) {   // L^T x = D^-1 y
+        M a = Y[i * 32 + lane] * rD[i];
+#pragma unroll
+        for (int d = W; d >= 1; --d)
+            if (d <= bw && i + d < n) a = fma(-B[(i + d) * st + d], win[d - 1], a);
+#pragma unroll
+        for (int d = W - 1; d > 0; --d) win[d] = win[d - 1];
+        win[0] = a;
+        Y[i * 32 + lane] = a;
+    }
+}
 template <int DIM, typename M>
-__global__ void __launch_bounds__(128) k_mg_inverse_band(GridD g, MG3<M> cc, const M *__restrict__ diag,
-                                                    const uint8_t *__restrict__ fluid, M *__restrict__ inv, int refresh,
-                                                    int *__restrict__ ctl) {
+__global__ void __launch_bounds__(32) k_mg_inverse_band(GridD g, MG3<M> cc, const M *__restrict__ diag,
+                                                        const uint8_t *__restrict__ fluid, M *__restrict__ inv, int refresh,
+                                                        const int *__restrict__ ctl) {
     extern __shared__ __align__(16) unsigned char sm[];
     griddep_wait();
-    if (!inverse_due(ctl, refresh)) return;
+    if (ctl[C_PACK] % refresh != 0) return;
     const int t = threadIdx.x, n = g.ncell;
     // axes by extent, shortest first
     int ax[3] = {0, 1, 2};
@@ -925,11 +1176,12 @@ __global__ void __launch_bounds__(128) k_mg_inverse_band(GridD g, MG3<M> cc, con
     st[ax[2]] = e[ax[0]] * e[ax[1]];
     const int bw = st[ax[2]], W = bw + 1;
     M *B = (M *)sm;                       // B[r W + d] = A(r, r - d), then L (d > 0) and D (d = 0)
-    M *Y = B + (size_t)kExactCells * W;   // Y[i n + j]: column j of the inverse, band order
+    M *rD = B + (size_t)kExactCells * W;
+    M *Y = rD + kExactCells;              // Y[i 32 + lane]: this block's columns of the inverse, band order
     __shared__ int cell_s[kExactCells];   // cell of a band index
-    for (int q = t; q < n * W; q += blockDim.x) B[q] = M(0);
-    __syncthreads();
-    for (int c = t; c < n; c += blockDim.x) {
+    for (int q = t; q < n * W; q += 32) B[q] = M(0);
+    __syncwarp();
+    for (int c = t; c < n; c += 32) {
         const int i = c % g.nx, j = (c / g.nx) % g.ny, k = c / (g.nx * g.ny);
         const int r = i * st[0] + j * st[1] + k * st[2];
         cell_s[r] = c;
@@ -942,61 +1194,34 @@ __global__ void __launch_bounds__(128) k_mg_inverse_band(GridD g, MG3<M> cc, con
         for (int a = 0; a < DIM; ++a)   // the low neighbours are those of smaller band index
             if (ijk[a] > 0) B[r * W + st[a]] = -cc.a[a][flo(g, a, i, j, k)];
     }
-    // right-looking factorisation: after step k the columns beyond k hold the Schur complement
+    __syncwarp();
+    // right-looking factorisation: after step k the columns beyond k hold the
+    // Schur complement and column k the entries of L
     for (int k = 0; k < n; ++k) {
-        __syncthreads();
         const M d = B[k * W];
-        const bool ok = d > M(0);
-        const M rd = ok ? M(1) / d : M(0);
+        const M rd = d > M(0) ? M(1) / d : M(0);
         const int m = min(bw, n - 1 - k);
-        for (int q = t; q < m * m; q += blockDim.x) {   // A(k+1+u, k+1+v) -= A(k+1+u, k) A(k+1+v, k) / d, v <= u
+        for (int q = t; q < m * m; q += 32) {   // A(k+1+u, k+1+v) -= A(k+1+u, k) A(k+1+v, k) / d, v <= u
             const int u = q / m, v = q - u * m;
-            if (v > u) continue;
-            B[(k + 1 + u) * W + (u - v)] -= B[(k + 1 + u) * W + u + 1] * rd * B[(k + 1 + v) * W + v + 1];
-        }
-    }
-    __syncthreads();
-    // column k of L: A(r, k) / D(k); a vanished pivot drops its row and column
-    for (int q = t; q < n * bw; q += blockDim.x) {
-        const int r = q / bw, d = q - r * bw + 1;
-        if (r < d) continue;
-        const M p = B[(r - d) * W];
-        B[r * W + d] = p > M(0) ? B[r * W + d] / p : M(0);
-    }
-    __syncthreads();
-    if (t < n) {
-        const M dt = B[t * W];
-        for (int i = 0; i < t; ++i) Y[i * n + t] = M(0);
-        for (int i = t; i < n; ++i) {   // L y = e_t
-            M a0 = i == t ? M(1) : M(0), a1 = M(0);
-            const int m = min(bw, i - t);
-            int d = 1;
-            for (; d + 1 <= m; d += 2) {
-                a0 = fma(-B[i * W + d], Y[(i - d) * n + t], a0);
-                a1 = fma(-B[i * W + d + 1], Y[(i - d - 1) * n + t], a1);
+            if (v <= u) {
+                M *a = B + (k + 1 + u) * W + (u - v);
+                *a = fma(-(B[(k + 1 + u) * W + u + 1] * rd), B[(k + 1 + v) * W + v + 1], *a);
             }
-            if (d <= m) a0 = fma(-B[i * W + d], Y[(i - d) * n + t], a0);
-            Y[i * n + t] = a0 + a1;
         }
-        for (int i = n - 1; i >= 0; --i) {   // L^T x = D^-1 y
-            const M di = B[i * W];
-            M a0 = di > M(0) ? Y[i * n + t] / di : M(0), a1 = M(0);
-            const int m = min(bw, n - 1 - i);
-            int d = 1;
-            for (; d + 1 <= m; d += 2) {
-                a0 = fma(-B[(i + d) * W + d], Y[(i + d) * n + t], a0);
-                a1 = fma(-B[(i + d + 1) * W + d + 1], Y[(i + d + 1) * n + t], a1);
-            }
-            if (d <= m) a0 = fma(-B[(i + d) * W + d], Y[(i + d) * n + t], a0);
-            const bool live = di > M(0) && dt > M(0);
-            Y[i * n + t] = live ? a0 + a1 : M(0);
-        }
+        __syncwarp();
+        for (int u = t; u < m; u += 32) B[(k + 1 + u) * W + u + 1] *= rd;
+        if (t == 0) rD[k] = rd;
+        __syncwarp();
     }
-    __syncthreads();
-    for (int q = t; q < n * n; q += blockDim.x) {
-        const int r = q / n, j = q - r * n;
-        inv[cell_s[r] * n + cell_s[j]] = Y[q];
-    }
+    const int col = blockIdx.x * 32 + t;
+    const bool live = col < n && rD[col] > M(0);
+    if (bw <= 4) band_solve<M, 4>(B, rD, Y, n, bw, col, live);
+    else if (bw <= 8) band_solve<M, 8>(B, rD, Y, n, bw, col, live);
+    else if (bw <= 12) band_solve<M, 12>(B, rD, Y, n, bw, col, live);
+    else band_solve<M, 26>(B, rD, Y, n, bw, col, live);
+    __syncwarp();
+    if (col < n)
+        for (int r = 0; r < n; ++r) inv[cell_s[r] * n + cell_s[col]] = Y[r * 32 + t];
 }
 
 }  // namespace oscar

@@ -14,6 +14,7 @@ constexpr int kMaxLevels = 24;
 constexpr int kRedBlocks = 1216;      // 152 SMs x 8: fixed grid of every reduction (deterministic order)
 constexpr int kRedSlots = 16;         // partial-sum slots
 constexpr double kSyncTimeoutSec = 600.0;
+constexpr size_t kClImageBytes = 16 * 220 * 1024;              // one image per CTA of a cluster, at most its shared memory
 constexpr size_t kClInvBytes = 128 * 128 * sizeof(double);   // explicit inverse of a level of at most 128 cells
 
 // Scalar slots in the device scalar array (double).
@@ -131,6 +132,7 @@ struct Instance {
     int solve_nc;          // CTAs of the whole-solve cluster, 0 when solves run as launches
     size_t solve_smem;
     void *cl_inv;          // explicit inverse of the coarsest level (kClInvBytes)
+    void *cl_image;        // shared-memory images of the cluster's CTAs (kClImageBytes)
     cudaStream_t aux;      // branch of the operator set-up
     cudaEvent_t ev_fork, ev_join;
     int pending;           // kind (0 drag, 1 relax, 2 standard) of a launched step not yet waited for, or -1

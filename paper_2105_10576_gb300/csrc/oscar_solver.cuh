@@ -172,7 +172,11 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // is still bound by its latency; in FP64 they are bound by FP64 issue above
 // 1024 cells). A 2D grid of at most solve_cells is solved whole in one cluster
 // when its vectors fit the shared memory.
-constexpr int kVcycleCtas = 16, kVcycleThreads = 512, kSolveCtas = 16, kSolveThreads = 256;
+constexpr int kVcycleCtas = 16, kVcycleThreads = 512, kSolveCtas = 16;
+// fewer threads make the block and cluster barriers shorter, more take larger
+// slabs with fewer entries per thread (128x16 FP64: 256 threads 8.03 ms per
+// pass, 512 8.53; 512x64 mixed: 4.25 and 3.64)
+inline int solve_threads(int ncell) { return ncell <= 8192 ? 256 : 512; }
 template <typename T> struct ClRule;
 template <> struct ClRule<float> {
     static constexpr long long vcycle_cells = 8, solve_cells = 65536;
@@ -270,10 +274,18 @@ template <typename T> struct Impl {
         const Level &E = I.lev[exact_level(I, top_level(I))];
         if constexpr (sizeof(M) == sizeof(float))
             launchk(k_mg_inverse_dense<DIM>, 1, kGjThreads, 0, st, to_dev(E.g), mg3(E), (const M *)E.diag,
-                    (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, I.ctl), ++I.nlaunch;
+                    (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, (const int *)I.ctl), ++I.nlaunch;
         else
-            launchk(k_mg_inverse_band<DIM, M>, 1, 128, inverse_smem(E.g), st, to_dev(E.g), mg3(E), (const M *)E.diag,
-                    (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, I.ctl), ++I.nlaunch;
+            launchk(k_mg_inverse_band<DIM, M>, (E.g.ncell + 31) / 32, 32, inverse_smem(E.g), st, to_dev(E.g), mg3(E),
+                    (const M *)E.diag, (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, (const int *)I.ctl),
+                ++I.nlaunch;
+        {   // the images of the levels the solves work in a cluster
+            ClLevels<M> P;
+            ClSolve A;
+            if (I.solve_nc) cl_fill(I, P, 0, I.solve_nc, &A);
+            else cl_fill(I, P, top_level(I), I.cl_nc);
+            launchk(k_cl_pack<DIM, M>, dim3(P.nc, kPackSlices), kPackThreads, 0, st, P, I.ctl), ++I.nlaunch;
+        }
         OSCAR_LAUNCH_CHECK();
         return 0;
     }
@@ -290,8 +302,7 @@ template <typename T> struct Impl {
     static size_t inverse_smem(const GridH &g) {
         int e[3] = {g.nx, g.ny, g.nz};
         std::sort(e, e + 3);
-        const size_t n = g.ncell;
-        return (kExactCells * (size_t)(e[0] * e[1] + 1) + n * n) * sizeof(M);
+        return (kExactCells * (size_t)(e[0] * e[1] + 2) + 32 * (size_t)g.ncell) * sizeof(M);
     }
 
     // Levels l0 .. of a cluster of at most nc_max CTAs and their shared-memory
@@ -343,26 +354,35 @@ template <typename T> struct Impl {
             C.ce = ((C.ny + 1) / 2) * C.nz;
             C.rncol = 1.0f / (float)C.ncol;
             C.rny = 1.0f / (float)C.ny;
-            C.rhj = 1.0f / (float)((C.ny + 1) / 2);
+            C.rce = 1.0f / (float)C.ce;
             for (int a = 0; a < 3; ++a) C.c[a] = (const M *)L.c[a];
             C.idiag = (const M *)L.idiag;
-            C.ox = take(n * sizeof(M));
-            C.ob = take(n * sizeof(M));
             C.oi = take(n * sizeof(M));
             for (int a = 0; a < L.g.dim; ++a) C.oc[a] = take(n * sizeof(M));
             const size_t nh = (size_t)C.ncol * C.ce * sizeof(unsigned short);
             C.ol[0] = take(nh);
             C.ol[1] = take(nh);
             if (!last) C.op = take(nh);
+            C.os = take((P.nc + 1) * sizeof(short));
+            if (C.nx > 32767) return (size_t)-1;   // slab starts are 16-bit numbers
             if (!last) rs = std::max(rs, (size_t)w[q] * C.ps);
         }
         const ClLevel<M> &Lc = P.L[P.n - 1];
         const size_t ne = I.lev[le].g.ncell;
+        const size_t nrow = std::min((size_t)(w[P.n - 1] + 2 * cl_exact_depth(P)) * Lc.ny * Lc.nz, ne);
+        P.oinv = take(nrow * ne * sizeof(M));
+        P.orow = take(nrow * sizeof(unsigned short));
+        P.img = (int)off;
+        P.image = (unsigned char *)I.cl_image;
+        for (int q = 0; q < P.n; ++q) {
+            P.L[q].ox = take((size_t)P.L[q].nloc * sizeof(M));
+            P.L[q].ob = take((size_t)P.L[q].nloc * sizeof(M));
+        }
+        if (A) rs = std::max(rs, (size_t)w[0] * P.L[0].ps);   // the products of a dot
         P.ors = take(rs * sizeof(M));
         P.obx = take(ne * sizeof(M));
-        P.oinv = take(std::min((size_t)Lc.ncol * Lc.ny * Lc.nz, ne) * ne * sizeof(M));
         if (A) {
-            P.ored = take((512 + 2 * 4 * kMaxCluster) * sizeof(double));
+            P.ored = take((4 * solve_threads(I.g.ncell) + 2 * 4 * kMaxCluster) * sizeof(double));
             const size_t n = (size_t)(w[0] + 2) * P.L[0].ps;
             A->op = take(n * sizeof(M));
             A->oap = take(n * sizeof(M));
@@ -534,7 +554,7 @@ template <typename T> struct Impl {
             A.inv_nf = with_E ? 1.0 / (double)I.n_fluid : 0.0;
             A.maxit = I.P.cg_maxit;
             A.by = (int)launch3(I.g).block.y;
-            launchx(!with_E, P.nc, k_solve_cluster<T>, P.nc, kSolveThreads, I.solve_smem, I.stream, P, A), ++I.nlaunch;
+            launchx(!with_E, P.nc, k_solve_cluster<T>, P.nc, solve_threads(I.g.ncell), I.solve_smem, I.stream, P, A), ++I.nlaunch;
             OSCAR_LAUNCH_CHECK();
             return 0;
         }
