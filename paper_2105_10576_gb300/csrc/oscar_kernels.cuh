@@ -77,6 +77,48 @@ template <> struct GA<float> {
     __device__ static __forceinline__ float V(const GridD &g) { return g.Vf; }
 };
 
+// Divisions by grid constants and the time step. An FP64 division is about ten
+// FP64 instructions on a GPU that issues two FP64 FMAs per clock and SM: in
+// FP64 they are multiplications by the reciprocal (GR<double>: 128x32x32 FP64
+// momentum prediction 200 -> 110 us); in FP32, where they are not what bounds a
+// kernel, divisions, and GR is empty.
+template <typename T> struct GR {};
+template <> struct GR<double> {
+    double rh[3], Sh[3], rV, rS, rdt;   // 1 / h, S / h, 1 / V, 1 / (2 sum S), 1 / dt
+};
+template <typename T> inline GR<T> to_gr(const GridH &g, double dt) {
+    GR<T> r;
+    if constexpr (sizeof(T) == sizeof(double)) {
+        for (int a = 0; a < 3; ++a) {
+            r.rh[a] = 1.0 / g.h[a];
+            r.Sh[a] = g.S[a] / g.h[a];
+        }
+        r.rV = 1.0 / g.V;
+        r.rS = 1.0 / (2.0 * (g.S[0] + g.S[1] + g.S[2]));
+        r.rdt = 1.0 / dt;
+    }
+    return r;
+}
+__device__ __forceinline__ float div_h(const GridD &g, const GR<float> &, int a, float x) { return x / g.hf[a]; }
+__device__ __forceinline__ double div_h(const GridD &, const GR<double> &r, int a, double x) { return x * r.rh[a]; }
+__device__ __forceinline__ double div_half_h(const GridD &, const GR<double> &r, int a, double x) { return x * (2.0 * r.rh[a]); }
+__device__ __forceinline__ float mul_S_div_h(const GridD &g, const GR<float> &, int a, float x) { return x * g.Sf[a] / g.hf[a]; }
+__device__ __forceinline__ double mul_S_div_h(const GridD &, const GR<double> &r, int a, double x) { return x * r.Sh[a]; }
+__device__ __forceinline__ float mul_S_div_half_h(const GridD &g, const GR<float> &, int a, float x) {
+    return x * g.Sf[a] / (0.5f * g.hf[a]);
+}
+__device__ __forceinline__ double mul_S_div_half_h(const GridD &, const GR<double> &r, int a, double x) {
+    return x * (2.0 * r.Sh[a]);
+}
+__device__ __forceinline__ float div_V(const GridD &g, const GR<float> &, float x) { return x / g.Vf; }
+__device__ __forceinline__ double div_V(const GridD &, const GR<double> &r, double x) { return x * r.rV; }
+__device__ __forceinline__ float div_dt(const GR<float> &, float x, float dt) { return x / dt; }
+__device__ __forceinline__ double div_dt(const GR<double> &r, double x, double) { return x * r.rdt; }
+__device__ __forceinline__ float div_2S(const GR<float> &, float x, float den) { return x / den; }
+__device__ __forceinline__ double div_2S(const GR<double> &r, double x, double) { return x * r.rS; }
+__device__ __forceinline__ float div_by(float x, float d, float) { return x / d; }
+__device__ __forceinline__ double div_by(double x, double, double rd) { return x * rd; }
+
 template <typename T> struct P3 { T *a[3]; };
 template <typename T> struct C3 { const T *a[3]; };
 
@@ -108,6 +150,16 @@ inline L3 launch_rows(const GridH &g, int target) {
     int want = target / gx > 0 ? target / gx : 1;
     int m = (gy + want - 1) / want;
     l.grid = dim3(gx, (gy + m - 1) / m, 1);
+    l.nblocks = (int)(l.grid.x * l.grid.y);
+    return l;
+}
+
+// at most two blocks of 1024 threads per SM over (x, rows), rows looped
+inline L3 launch_sms(const GridH &g) {
+    L3 l = launch3(g.nx, g.ny * g.nz, 1);
+    const int bx = (int)l.block.x, by = 1024 / bx, gx = (int)l.grid.x, gy = (g.ny * g.nz + by - 1) / by;
+    l.block = dim3(bx, by, 1);
+    l.grid = dim3(gx, std::max(1, std::min(gy, 304 / gx)), 1);
     l.nblocks = (int)(l.grid.x * l.grid.y);
     return l;
 }
@@ -560,7 +612,7 @@ __global__ void k_transport_low(GridD g, const uint32_t *__restrict__ info, cons
 template <int DIM, typename T>
 __global__ void k_transport_ratio(GridD g, const uint32_t *__restrict__ info, const T *__restrict__ alpha,
                                   const T *__restrict__ aL, const T *__restrict__ Pp, const T *__restrict__ Pm, T rV,
-                                  T *__restrict__ Rp, T *__restrict__ Rm) {
+                                  T rrV, T *__restrict__ Rp, T *__restrict__ Rm) {
     griddep_wait();
     CELL_IJK(g);
     if (!inside) return;
@@ -585,8 +637,8 @@ __global__ void k_transport_ratio(GridD g, const uint32_t *__restrict__ info, co
     }
     if (amax > T(1)) amax = T(1);
     if (amin < T(0)) amin = T(0);
-    T Qp = (amax - l0) / rV;
-    T Qm = (l0 - amin) / rV;
+    T Qp = div_by(amax - l0, rV, rrV);
+    T Qm = div_by(l0 - amin, rV, rrV);
     if (Qp < T(0)) Qp = T(0);
     if (Qm < T(0)) Qm = T(0);
     T pp = Pp[c], pm = Pm[c];
@@ -630,7 +682,7 @@ __global__ void k_transport_update(GridD g, const uint32_t *__restrict__ info, c
 // (Section 2.1; wall condition of Eqs. VOFd / VOFc)
 // ---------------------------------------------------------------------------
 template <int DIM, typename T>
-__global__ void k_smooth(GridD g, const uint32_t *__restrict__ info, const T *__restrict__ src, T *__restrict__ dst) {
+__global__ void k_smooth(GridD g, GR<T> gr, const uint32_t *__restrict__ info, const T *__restrict__ src, T *__restrict__ dst) {
     griddep_wait();
     CELL_IJK(g);
     if (!inside) return;
@@ -649,22 +701,22 @@ __global__ void k_smooth(GridD g, const uint32_t *__restrict__ info, const T *__
             den += Sa;
         }
     }
-    dst[c] = num / den;
+    dst[c] = div_2S(gr, num, den);
 }
 
 template <int DIM, typename T>
-__device__ __forceinline__ T gauss_grad(const GridD &g, const uint32_t *__restrict__ info, const T *__restrict__ x, int c,
+__device__ __forceinline__ T gauss_grad(const GridD &g, const GR<T> &gr, const uint32_t *__restrict__ info, const T *__restrict__ x, int c,
                                         int b) {
     uint32_t inf = info[c];
     int off = noff(g, b);
     T xc = x[c];
     T f0 = ftype(inf, b, 0) == FT_INTERIOR ? T(0.5) * (xc + x[c - off]) : xc;
     T f1 = ftype(inf, b, 1) == FT_INTERIOR ? T(0.5) * (xc + x[c + off]) : xc;
-    return (f1 - f0) / GA<T>::h(g, b);
+    return div_h(g, gr, b, f1 - f0);
 }
 
 template <int DIM, int A, typename T>
-__global__ void k_normals(GridD g, const uint32_t *__restrict__ info, const T *__restrict__ as, T ct, T deltaN,
+__global__ void k_normals(GridD g, GR<T> gr, const uint32_t *__restrict__ info, const T *__restrict__ as, T ct, T deltaN,
                           T *__restrict__ nfA) {
     griddep_wait();
     FACE_IJK(g, A);
@@ -673,11 +725,11 @@ __global__ void k_normals(GridD g, const uint32_t *__restrict__ info, const T *_
     T n = T(0);
     if (t == FT_INTERIOR) {
         T gv[3] = {T(0), T(0), T(0)};
-        gv[A] = (as[H] - as[L]) / GA<T>::h(g, A);
+        gv[A] = div_h(g, gr, A, as[H] - as[L]);
 #pragma unroll
         for (int b = 0; b < DIM; ++b) {
             if (b == A) continue;
-            gv[b] = T(0.5) * (gauss_grad<DIM, T>(g, info, as, L, b) + gauss_grad<DIM, T>(g, info, as, H, b));
+            gv[b] = T(0.5) * (gauss_grad<DIM, T>(g, gr, info, as, L, b) + gauss_grad<DIM, T>(g, gr, info, as, H, b));
         }
         T mag = T(0);
 #pragma unroll
@@ -691,14 +743,14 @@ __global__ void k_normals(GridD g, const uint32_t *__restrict__ info, const T *_
 }
 
 template <int DIM, typename T>
-__global__ void k_curvature(GridD g, const uint32_t *__restrict__ info, C3<T> nf, T *__restrict__ kappa) {
+__global__ void k_curvature(GridD g, GR<T> gr, const uint32_t *__restrict__ info, C3<T> nf, T *__restrict__ kappa) {
     griddep_wait();
     CELL_IJK(g);
     if (!inside) return;
     if (!(info[c] & INFO_FLUID)) { kappa[c] = T(0); return; }
     T acc = T(0);
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) acc += (nf.a[a][fhi(g, a, i, j, k)] - nf.a[a][flo(g, a, i, j, k)]) / GA<T>::h(g, a);
+    for (int a = 0; a < DIM; ++a) acc += div_h(g, gr, a, nf.a[a][fhi(g, a, i, j, k)] - nf.a[a][flo(g, a, i, j, k)]);
     kappa[c] = -acc;
 }
 
@@ -716,7 +768,7 @@ template <typename T> __device__ __forceinline__ T mix(T al, T p1, T p2) { retur
 // OSCAR_CONV_AREA mode exits when this energy changes by less than the
 // tolerance (relative) over a sub-step.
 template <int DIM, typename T>
-__global__ void k_relax_energy(int n, GridD g, const uint32_t *__restrict__ info, const T *__restrict__ alpha,
+__global__ void k_relax_energy(int n, GridD g, GR<T> gr, const uint32_t *__restrict__ info, const T *__restrict__ alpha,
                                C3<T> u, Fluid<T> fl, double sigma, double *__restrict__ part, int stride,
                                unsigned *__restrict__ ticket, double *__restrict__ scal, int slot) {
     griddep_wait();
@@ -726,7 +778,7 @@ __global__ void k_relax_energy(int n, GridD g, const uint32_t *__restrict__ info
         T m2 = T(0), u2 = T(0);
 #pragma unroll
         for (int b = 0; b < DIM; ++b) {
-            const T gb = gauss_grad<DIM, T>(g, info, alpha, c, b);
+            const T gb = gauss_grad<DIM, T>(g, gr, info, alpha, c, b);
             m2 += gb * gb;
             const T ub = u.a[b][c];
             u2 += ub * ub;
@@ -740,7 +792,7 @@ __global__ void k_relax_energy(int n, GridD g, const uint32_t *__restrict__ info
 
 // rA = 1/A, A = rho/dt + (viscous diagonal + rho * inflow flux)/V
 template <int DIM, typename T>
-__global__ void k_rA(GridD g, const uint32_t *__restrict__ info, const T *__restrict__ alpha, C3<T> phic, Fluid<T> fl,
+__global__ void k_rA(GridD g, GR<T> gr, const uint32_t *__restrict__ info, const T *__restrict__ alpha, C3<T> phic, Fluid<T> fl,
                      T dt, T *__restrict__ rA) {
     griddep_wait();
     CELL_IJK(g);
@@ -753,15 +805,14 @@ __global__ void k_rA(GridD g, const uint32_t *__restrict__ info, const T *__rest
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         int off = noff(g, a);
-        T Sa = GA<T>::S(g, a), ha = GA<T>::h(g, a);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             int t = ftype(inf, a, s);
             if (t == FT_INTERIOR) {
                 T mun = mix(alpha[s ? c + off : c - off], fl.mu1, fl.mu2);
-                acc += T(0.5) * (mu + mun) * Sa / ha;
+                acc += mul_S_div_h(g, gr, a, T(0.5) * (mu + mun));
             } else if (t == FT_WALL || t == FT_INLET) {
-                acc += mu * Sa / (T(0.5) * ha);
+                acc += mul_S_div_half_h(g, gr, a, mu);
             }
             if (t == FT_INTERIOR || t == FT_INLET) {
                 T fo = (s ? T(1) : T(-1)) * phic.a[a][s ? fhi(g, a, i, j, k) : flo(g, a, i, j, k)];
@@ -769,25 +820,24 @@ __global__ void k_rA(GridD g, const uint32_t *__restrict__ info, const T *__rest
             }
         }
     }
-    rA[c] = T(1) / (rho / dt + (acc + rho * cin) / GA<T>::V(g));
+    rA[c] = T(1) / (div_dt(gr, rho, dt) + div_V(g, gr, acc + rho * cin));
 }
 
 // pressure-operator coefficients c_f (multigrid level 0) and CSF face forces
 template <int A, typename T>
-__global__ void k_face_coeffs(GridD g, const uint32_t *__restrict__ info, const T *__restrict__ rA,
+__global__ void k_face_coeffs(GridD g, GR<T> gr, const uint32_t *__restrict__ info, const T *__restrict__ rA,
                               const T *__restrict__ kappa, const T *__restrict__ alpha, T sigma, int has_st,
                               T *__restrict__ cf, T *__restrict__ fst, double *__restrict__ cf64) {
     griddep_wait();
     FACE_IJK(g, A);
     int L, H;
     int t = decode_face<A>(g, info, i, j, k, L, H);
-    T Sa = GA<T>::S(g, A), ha = GA<T>::h(g, A);
     T cc = T(0), fs = T(0);
     if (t == FT_INTERIOR) {
-        cc = T(0.5) * (rA[L] + rA[H]) * Sa / ha;
-        if (has_st) fs = sigma * T(0.5) * (kappa[L] + kappa[H]) * (alpha[H] - alpha[L]) / ha;
+        cc = mul_S_div_h(g, gr, A, T(0.5) * (rA[L] + rA[H]));
+        if (has_st) fs = div_h(g, gr, A, sigma * T(0.5) * (kappa[L] + kappa[H]) * (alpha[H] - alpha[L]));
     } else if (t == FT_OUTLET) {
-        cc = rA[L] * Sa / (T(0.5) * ha);
+        cc = mul_S_div_half_h(g, gr, A, rA[L]);
     }
     cf[f] = cc;
     fst[f] = fs;
@@ -796,7 +846,7 @@ __global__ void k_face_coeffs(GridD g, const uint32_t *__restrict__ info, const 
 
 // Gauss gradients of the velocity iterate: G[comp*3 + dir]
 template <int DIM, typename T>
-__global__ void k_vel_grad(GridD g, const uint32_t *__restrict__ info, C3<T> v, T vin0, P3<T> G0, P3<T> G1, P3<T> G2) {
+__global__ void k_vel_grad(GridD g, GR<T> gr, const uint32_t *__restrict__ info, C3<T> v, T vin0, P3<T> G0, P3<T> G1, P3<T> G2) {
     griddep_wait();
     CELL_IJK(g);
     if (!inside) return;
@@ -819,7 +869,7 @@ __global__ void k_vel_grad(GridD g, const uint32_t *__restrict__ info, C3<T> v, 
                 else if (t == FT_OUTLET) fv[s] = vc;
                 else fv[s] = T(0);
             }
-            Gr[comp][dir][c] = (fv[1] - fv[0]) / GA<T>::h(g, dir);
+            Gr[comp][dir][c] = div_h(g, gr, dir, fv[1] - fv[0]);
         }
     }
 }
@@ -829,7 +879,7 @@ __global__ void k_vel_grad(GridD g, const uint32_t *__restrict__ info, C3<T> v, 
 // transpose viscous term. A latency-bound gather: the register cap (6 blocks
 // of 256 threads per SM instead of 4) keeps more loads in flight.
 template <int DIM, typename T>
-__global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, const uint32_t *__restrict__ info, C3<T> v, C3<T> vold, C3<T> phic,
+__global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, GR<T> gr, const uint32_t *__restrict__ info, C3<T> v, C3<T> vold, C3<T> phic,
                              const T *__restrict__ alpha, const T *__restrict__ rA, Fluid<T> fl, T vin0, T dt,
                              C3<T> G0, C3<T> G1, C3<T> G2, P3<T> hbya) {
     griddep_wait();
@@ -845,7 +895,6 @@ __global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, const uint32_t *
     T al = alpha[c];
     T rho = mix(al, fl.rho1, fl.rho2), mu = mix(al, fl.mu1, fl.mu2);
     T rAc = rA[c];
-    const T Vc = GA<T>::V(g);
     T lap[3] = {T(0), T(0), T(0)}, conv[3] = {T(0), T(0), T(0)}, tr[3] = {T(0), T(0), T(0)},
       inflow[3] = {T(0), T(0), T(0)};
     T vc[3];
@@ -866,7 +915,7 @@ __global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, const uint32_t *
                 const int nb = s ? c + off : c - off;
                 const T mun = mix(alpha[nb], fl.mu1, fl.mu2);
                 const T muf = T(0.5) * (mu + mun);
-                const T lapc = muf * Sa / ha;
+                const T lapc = mul_S_div_h(g, gr, a, muf);
                 const T pc = phic.a[a][f];
                 const bool fromL = pc >= T(0);
                 const int up = fromL ? (s ? c : nb) : (s ? nb : c);
@@ -891,7 +940,7 @@ __global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, const uint32_t *
 #pragma unroll
                 for (int comp = 0; comp < DIM; ++comp) {
                     const T vin = comp == 0 ? vin0 : T(0);
-                    lap[comp] += mu * Sa / (T(0.5) * ha) * vin;
+                    lap[comp] += mul_S_div_half_h(g, gr, a, mu) * vin;
                     if (fo < T(0)) inflow[comp] += -fo * vin;
                     else conv[comp] += fo * (vin - vc[comp]);
                     tr[comp] += sg * mu * Sa * Gr[a][comp][c];
@@ -901,8 +950,8 @@ __global__ void __launch_bounds__(256, 6) k_momentum_H(GridD g, const uint32_t *
     }
 #pragma unroll
     for (int comp = 0; comp < DIM; ++comp) {
-        T Hc = rho * vold.a[comp][c] / dt;
-        Hc += (lap[comp] + rho * (inflow[comp] - conv[comp]) + tr[comp]) / Vc;
+        T Hc = div_dt(gr, rho * vold.a[comp][c], dt);
+        Hc += div_V(g, gr, lap[comp] + rho * (inflow[comp] - conv[comp]) + tr[comp]);
         hbya.a[comp][c] = rAc * Hc;
     }
 }
@@ -995,7 +1044,7 @@ __device__ __forceinline__ void correct_pair(const GridD &g, const uint32_t *__r
 // extents being multiples of 32), the other high faces formed again. FP64
 // instructions are scarce on this GPU, and this halves them.
 template <int DIM, typename T>
-__global__ void k_correct(GridD g, const uint32_t *__restrict__ info, C3<T> phis, C3<T> cf, const double *__restrict__ q,
+__global__ void k_correct(GridD g, GR<T> gr, const uint32_t *__restrict__ info, C3<T> phis, C3<T> cf, const double *__restrict__ q,
                           P3<T> phi, C3<T> hbya, const T *__restrict__ rA, C3<T> fst, P3<T> v) {
     griddep_wait();
     CELL_IJK(g);
@@ -1020,7 +1069,6 @@ __global__ void k_correct(GridD g, const uint32_t *__restrict__ info, C3<T> phis
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         const int off = noff(g, a);
-        const T ha = GA<T>::h(g, a);
         T gs = T(0);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
@@ -1031,15 +1079,19 @@ __global__ void k_correct(GridD g, const uint32_t *__restrict__ info, C3<T> phis
                 if (s == 0) dq = dlo[a];
                 else if (a == 0 && next_in_warp) dq = dnext;
                 else dq = (T)(q[c + off] - qc);
-                gs += fst.a[a][f] - dq / ha;
+                gs += fst.a[a][f] - div_h(g, gr, a, dq);
             } else if (t == FT_OUTLET) {
-                gs += -(T)(0.0 - qc) / (T(0.5) * ha);
+                if constexpr (sizeof(T) == sizeof(double)) gs += div_half_h(g, gr, a, qc);
+                else gs += -(T)(0.0 - qc) / (T(0.5) * GA<T>::h(g, a));
             }
         }
         v.a[a][c] = hbya.a[a][c] + rA[c] * T(0.5) * gs;
     }
 }
 
+// acc + w x: a product and a sum in FP32, fused in FP64 (half the FP64 instructions)
+__device__ __forceinline__ float mg_madd(float w, float x, float acc) { return acc + w * x; }
+__device__ __forceinline__ double mg_madd(double w, double x, double acc) { return fma(w, x, acc); }
 // (M x)_P = sum_f c_f (x_P - x_N) + sum_outlet c_f x_P, evaluated in type V
 template <int DIM, typename T, typename V>
 __device__ __forceinline__ V poisson_row(const GridD &g, uint32_t inf, int c, int i, int j, int k, C3<T> cf,
@@ -1054,9 +1106,9 @@ __device__ __forceinline__ V poisson_row(const GridD &g, uint32_t inf, int c, in
             int t = ftype(inf, a, s);
             if (t == FT_INTERIOR) {
                 int f = s ? fhi(g, a, i, j, k) : flo(g, a, i, j, k);
-                acc += (V)cf.a[a][f] * (xc - x[s ? c + off : c - off]);
+                acc = mg_madd((V)cf.a[a][f], xc - x[s ? c + off : c - off], acc);
             } else if (t == FT_OUTLET) {
-                acc += (V)cf.a[a][fhi(g, a, i, j, k)] * xc;
+                acc = mg_madd((V)cf.a[a][fhi(g, a, i, j, k)], xc, acc);
             }
         }
     }
@@ -1578,17 +1630,32 @@ __device__ __forceinline__ void mg_row_coeffs(const GridD &g, MG3<M> cc, int i, 
         w[2 * a + 1] = ijk[a] < n[a] - 1 ? cc.a[a][fhi(g, a, i, j, k)] : M(0);
     }
 }
-template <int DIM, typename M>
-__device__ __forceinline__ M mg_row_off(const GridD &g, const M *w, const M *x, int cell, int i, int j, int k) {
+// b + the sum of the neighbour terms of a row
+template <int DIM, typename M, typename F>
+__device__ __forceinline__ M mg_row_sum(const GridD &g, const M *w, M b, int i, int j, int k, F x) {
     const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
-    M acc = M(0);
+    M acc = sizeof(M) == sizeof(double) ? b : M(0);
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        const int off = noff(g, a);
-        if (ijk[a] > 0) acc += w[2 * a] * x[cell - off];
-        if (ijk[a] < n[a] - 1) acc += w[2 * a + 1] * x[cell + off];
+        if (ijk[a] > 0) acc = mg_madd(w[2 * a], x(a, 0), acc);
+        if (ijk[a] < n[a] - 1) acc = mg_madd(w[2 * a + 1], x(a, 1), acc);
     }
-    return acc;
+    return sizeof(M) == sizeof(double) ? acc : b + acc;
+}
+template <int DIM, typename M>
+__device__ __forceinline__ M mg_row_sum(const GridD &g, const M *w, M b, const M *x, int cell, int i, int j, int k) {
+    return mg_row_sum<DIM, M>(g, w, b, i, j, k, [&](int a, int s) { return x[s ? cell + noff(g, a) : cell - noff(g, a)]; });
+}
+// b - M x of a row with diagonal dg
+template <int DIM>
+__device__ __forceinline__ float mg_residual(const GridD &g, const float *w, float dg, float b, const float *x, int cell, int i,
+                                             int j, int k) {
+    return b - (dg * x[cell] - mg_row_sum<DIM, float>(g, w, 0.f, x, cell, i, j, k));
+}
+template <int DIM>
+__device__ __forceinline__ double mg_residual(const GridD &g, const double *w, double dg, double b, const double *x, int cell,
+                                              int i, int j, int k) {
+    return fma(-dg, x[cell], mg_row_sum<DIM, double>(g, w, b, x, cell, i, j, k));
 }
 
 // one colour of a red-black Gauss-Seidel sweep; thread ti handles the cell
@@ -1617,28 +1684,19 @@ __global__ void k_mg_rbgs(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__
     }
     griddep_wait();
     if (!ok) return;
-    M off;
+    const M bc = b[cell];
+    M t;
     if constexpr (PRO) {
-        const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz}, sh[3] = {s0, s1, s2};
-        const int pc[3] = {i >> s0, j >> s1, k >> s2};
-        off = M(0);
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            const int o = noff(g, a);
-#pragma unroll
-            for (int sd = 0; sd < 2; ++sd) {
-                const bool in = sd ? ijk[a] < n[a] - 1 : ijk[a] > 0;
-                if (!in) continue;
-                int pp[3] = {pc[0], pc[1], pc[2]};
-                pp[a] = (ijk[a] + (sd ? 1 : -1)) >> sh[a];
-                const M v = x[sd ? cell + o : cell - o] + xc[pp[0] + gc.nx * (pp[1] + gc.ny * pp[2])];
-                off += w[2 * a + sd] * v;
-            }
-        }
+        const int sh[3] = {s0, s1, s2}, ijk[3] = {i, j, k};
+        t = mg_row_sum<DIM, M>(g, w, bc, i, j, k, [&](int a, int s) {
+            int pp[3] = {i >> s0, j >> s1, k >> s2};
+            pp[a] = (ijk[a] + (s ? 1 : -1)) >> sh[a];
+            return x[s ? cell + noff(g, a) : cell - noff(g, a)] + xc[pp[0] + gc.nx * (pp[1] + gc.ny * pp[2])];
+        });
     } else {
-        off = mg_row_off<DIM, M>(g, w, x, cell, i, j, k);
+        t = mg_row_sum<DIM, M>(g, w, bc, x, cell, i, j, k);
     }
-    x[cell] = (b[cell] + off) * id;
+    x[cell] = t * id;
 }
 
 // The last half sweep of the finest level (colour 0) fused with r.z: the
@@ -1673,7 +1731,7 @@ __global__ void __launch_bounds__(256) k_mg_rbgs_dot(GridD g, MG3<M> cc, const M
         M acc = M(0);
         if (ok) {
             const M bc = b[cell];
-            const M xn = (bc + mg_row_off<DIM, M>(g, w, x, cell, i, j, k)) * id;
+            const M xn = mg_row_sum<DIM, M>(g, w, bc, x, cell, i, j, k) * id;
             x[cell] = xn;
             acc = bc * xn;
         }
@@ -1730,7 +1788,7 @@ __global__ void __launch_bounds__(256) k_mg_resid_restrict(GridD gf, GridD gc, c
     griddep_wait();
     M rv = M(0);
     if (in) {
-        rv = b[cell] - (dg * x[cell] - mg_row_off<DIM, M>(gf, w, x, cell, i, j, k));
+        rv = mg_residual<DIM>(gf, w, dg, b[cell], x, cell, i, j, k);
         rv = fl ? rv : M(0);
     }
     res[t] = rv;

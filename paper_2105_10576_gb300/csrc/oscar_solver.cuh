@@ -213,7 +213,7 @@ template <typename T> struct Impl {
                                                                   (T)I.P.c_alpha, (T)I.P.alpha_inlet, rV, tp(I.aL),
                                                                   tp(I.Pp), tp(I.Pm)), ++I.nlaunch;
         launchk(k_transport_ratio<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, tp(I.alpha), tp(I.aL), tp(I.Pp),
-                                                                    tp(I.Pm), rV, tp(I.Rp), tp(I.Rm)), ++I.nlaunch;
+                                                                    tp(I.Pm), rV, (T)(I.g.V / dt), tp(I.Rp), tp(I.Rm)), ++I.nlaunch;
         launchk(k_transport_update<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, tp(I.alpha), c3(phi), c3(I.nf),
                                                                      (T)I.P.c_alpha, tp(I.aL), tp(I.Rp), tp(I.Rm), rV,
                                                                      tp(I.alpha_new)), ++I.nlaunch;
@@ -229,20 +229,21 @@ template <typename T> struct Impl {
     static int interface_d(Instance &I, void *alpha) {
         GridD g = to_dev(I.g);
         L3 L = launch3(I.g);
+        const GR<T> gr = to_gr<T>(I.g, 1.0);
         void *src = alpha;
         for (int pass = 0; pass < I.P.n_smooth; ++pass) {
             void *dst = (pass % 2 == 0) ? I.alpha_s : I.alpha_tmp;
-            launchk(k_smooth<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, tp(src), tp(dst)), ++I.nlaunch;
+            launchk(k_smooth<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, tp(src), tp(dst)), ++I.nlaunch;
             src = dst;
         }
         const T *as = tp(src);
         T ct = (T)I.cos_theta, dn = (T)I.deltaN;
         L3 F0 = launch3_faces(I.g, 0), F1 = launch3_faces(I.g, 1), F2 = launch3_faces(I.g, 2);
-        launchk(k_normals<DIM, 0, T>, F0.grid, F0.block, 0, I.stream, g, I.info, as, ct, dn, tp(I.nf[0])), ++I.nlaunch;
-        launchk(k_normals<DIM, 1, T>, F1.grid, F1.block, 0, I.stream, g, I.info, as, ct, dn, tp(I.nf[1])), ++I.nlaunch;
+        launchk(k_normals<DIM, 0, T>, F0.grid, F0.block, 0, I.stream, g, gr, I.info, as, ct, dn, tp(I.nf[0])), ++I.nlaunch;
+        launchk(k_normals<DIM, 1, T>, F1.grid, F1.block, 0, I.stream, g, gr, I.info, as, ct, dn, tp(I.nf[1])), ++I.nlaunch;
         if (DIM == 3)
-            launchk(k_normals<DIM, 2, T>, F2.grid, F2.block, 0, I.stream, g, I.info, as, ct, dn, tp(I.nf[2])), ++I.nlaunch;
-        launchk(k_curvature<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.nf), tp(I.kappa)), ++I.nlaunch;
+            launchk(k_normals<DIM, 2, T>, F2.grid, F2.block, 0, I.stream, g, gr, I.info, as, ct, dn, tp(I.nf[2])), ++I.nlaunch;
+        launchk(k_curvature<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, c3(I.nf), tp(I.kappa)), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
         return 0;
     }
@@ -570,7 +571,7 @@ template <typename T> struct Impl {
             int nrr = 0;
             OSCAR_TRY(pcg_body<DIM>(I, mixed ? (V *)I.cg_e : (V *)q, mixed ? 1 : 0, &nrr));
             if constexpr (mixed) {
-                const L3 L = launch_rows(I.g, kRedBlocks);
+                const L3 L = launch_sms(I.g);
                 launchk(k_cg_refine<DIM>, L.grid, L.block, 0, I.stream, to_dev(I.g), I.info, c3(I.lev[0].c),
                         (const float *)I.cg_e, q, I.cg_r64, (float *)I.cg_r, (const float *)I.lev[0].idiag,
                         (float *)I.cg_z, part(I, kPartRr), nrr, part(I, kPartRefine), I.red_stride, I.ticket, L.nblocks,
@@ -594,18 +595,19 @@ template <typename T> struct Impl {
         GridD g = to_dev(I.g);
         L3 L = launch3(I.g);
         L3 F[3] = {launch3_faces(I.g, 0), launch3_faces(I.g, 1), launch3_faces(I.g, 2)};
+        const GR<T> gr = to_gr<T>(I.g, dt);
         Fluid<T> fl{(T)I.P.rho1, (T)I.P.rho2, (T)I.P.mu1, (T)I.P.mu2};
         const T *al = tp(I.alpha_new);
-        launchk(k_rA<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, al, c3(I.phic), fl, (T)dt, tp(I.rA)), ++I.nlaunch;
+        launchk(k_rA<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, al, c3(I.phic), fl, (T)dt, tp(I.rA)), ++I.nlaunch;
         void **cf = I.lev[0].c;
         T sig = (T)I.P.sigma;
         int st = has_st ? 1 : 0;
-        launchk(k_face_coeffs<0, T>, F[0].grid, F[0].block, 0, I.stream, g, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
+        launchk(k_face_coeffs<0, T>, F[0].grid, F[0].block, 0, I.stream, g, gr, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
                                                                     tp(cf[0]), tp(I.fst[0]), cf64_out(I, 0)), ++I.nlaunch;
-        launchk(k_face_coeffs<1, T>, F[1].grid, F[1].block, 0, I.stream, g, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
+        launchk(k_face_coeffs<1, T>, F[1].grid, F[1].block, 0, I.stream, g, gr, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
                                                                     tp(cf[1]), tp(I.fst[1]), cf64_out(I, 1)), ++I.nlaunch;
         if (DIM == 3)
-            launchk(k_face_coeffs<2, T>, F[2].grid, F[2].block, 0, I.stream, g, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
+            launchk(k_face_coeffs<2, T>, F[2].grid, F[2].block, 0, I.stream, g, gr, I.info, tp(I.rA), tp(I.kappa), al, sig, st,
                                                                         tp(cf[2]), tp(I.fst[2]), cf64_out(I, 2)), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
         // the multigrid operators are first needed by the solve: they are built
@@ -617,8 +619,8 @@ template <typename T> struct Impl {
         P3<T> Gp0 = p3(&I.G[0]), Gp1 = p3(&I.G[3]), Gp2 = p3(&I.G[6]);
         C3<T> Gc0 = c3(&I.G[0]), Gc1 = c3(&I.G[3]), Gc2 = c3(&I.G[6]);
         for (int corr = 0; corr < I.P.n_piso; ++corr) {
-            launchk(k_vel_grad<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(v), (T)vin0, Gp0, Gp1, Gp2), ++I.nlaunch;
-            launchk(k_momentum_H<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(v), c3(I.vold), c3(I.phic), al,
+            launchk(k_vel_grad<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, c3(v), (T)vin0, Gp0, Gp1, Gp2), ++I.nlaunch;
+            launchk(k_momentum_H<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, c3(v), c3(I.vold), c3(I.phic), al,
                                                                    tp(I.rA), fl, (T)vin0, (T)dt, Gc0, Gc1, Gc2,
                                                                    p3(I.hbya)), ++I.nlaunch;
             launchk(k_phistar_rhs<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.hbya), tp(I.rA), c3(I.fst),
@@ -633,7 +635,7 @@ template <typename T> struct Impl {
             }
             OSCAR_LAUNCH_CHECK();
             OSCAR_TRY(pcg_d<DIM>(I, q, I.cg_b, corr == 0));
-            launchk(k_correct<DIM, T>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.phis), c3(cf), q, p3(phi),
+            launchk(k_correct<DIM, T>, L.grid, L.block, 0, I.stream, g, gr, I.info, c3(I.phis), c3(cf), q, p3(phi),
                     c3(I.hbya), tp(I.rA), c3(I.fst), p3(v)), ++I.nlaunch;
             OSCAR_LAUNCH_CHECK();
         }
@@ -662,10 +664,10 @@ template <typename T> struct Impl {
         GridD g = to_dev(I.g);
         Fluid<T> fl{(T)I.P.rho1, (T)I.P.rho2, (T)I.P.mu1, (T)I.P.mu2};
         if (I.g.dim == 3)
-            launchk(k_relax_energy<3, T>, kRedBlocks, BS, 0, I.stream, I.g.ncell, g, I.info, (const T *)I.alpha,
+            launchk(k_relax_energy<3, T>, kRedBlocks, BS, 0, I.stream, I.g.ncell, g, to_gr<T>(I.g, 1.0), I.info, (const T *)I.alpha,
                     c3(I.u_cr), fl, I.P.sigma, I.partials, I.red_stride, I.ticket, I.scal, slot), ++I.nlaunch;
         else
-            launchk(k_relax_energy<2, T>, kRedBlocks, BS, 0, I.stream, I.g.ncell, g, I.info, (const T *)I.alpha,
+            launchk(k_relax_energy<2, T>, kRedBlocks, BS, 0, I.stream, I.g.ncell, g, to_gr<T>(I.g, 1.0), I.info, (const T *)I.alpha,
                     c3(I.u_cr), fl, I.P.sigma, I.partials, I.red_stride, I.ticket, I.scal, slot), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
         return 0;
