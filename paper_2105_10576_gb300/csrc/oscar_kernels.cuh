@@ -35,6 +35,7 @@ constexpr int BS = 256;
 constexpr int kCtaCells = 1024;      // largest cta_cells of a schedule
 constexpr int kApplyRows = 2;    // rows per thread of k_cg_pz_apply
 constexpr int kUpdateRows = 4;   // rows per thread of k_cg_update
+template <typename M> constexpr int kDotRows = sizeof(M) == sizeof(float) ? 2 : 1;   // rows per thread of k_mg_rbgs_dot
 
 // Programmatic dependent launch: wait until the preceding kernel has
 // completed and its writes are visible, then let the next kernel's CTAs be
@@ -1311,58 +1312,63 @@ __global__ void k_cg_apply_dot(GridD g, const uint32_t *__restrict__ info, C3<T>
 // Mixed path: p = z + beta p and Ap = M z + beta Ap (the search direction
 // update folded into the operator apply: M p = M z + beta M p_old, so every
 // thread writes only its own cell), then p.Ap; beta = 0 starts afresh. Each
-// thread takes RPT rows of a group (launch_groups), loaded together; the cell
-// flags and face coefficients, fixed during a solve, are loaded before the
-// grid dependency wait for its first group, the vectors after it.
+// thread takes RPT rows of a group (launch_groups), loaded together; the face
+// coefficients, fixed during a solve, are loaded before the grid dependency
+// wait for its first group, the vectors after it. Faces that do not belong to
+// the operator (walls, the inlet, faces of solid cells) have zero
+// coefficients and z is 0 beyond the outlet, so no face types are read: the
+// kernel was bound by instruction issue (55 % of its peak) with them.
 template <int DIM, typename T, typename V, int RPT>
-__global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, const uint32_t *__restrict__ info, C3<T> cf, const V *__restrict__ z,
+__global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, C3<T> cf, const V *__restrict__ z,
                               V *__restrict__ p, V *__restrict__ Ap, const double *__restrict__ rz_part, int nrz,
                               double *__restrict__ part, int groups, double *__restrict__ scal, int *__restrict__ ctl) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nrow = g.ny * g.nz;
-    uint32_t inf[RPT];
+    const int nrow = g.ny * g.nz, step = blockDim.y * RPT;
+    const int off[3] = {1, g.nx, g.nx * g.ny};
     T w[RPT][2 * DIM];
     V zc[RPT], zn[RPT][2 * DIM], po[RPT], ao[RPT];
+    int c[RPT], j[RPT], k[RPT];
+    bool in[RPT];
     auto load_fixed = [&](int row0) {
 #pragma unroll
         for (int u = 0; u < RPT; ++u) {
             const int row = row0 + u * blockDim.y;
-            inf[u] = 0;
-            if (i < g.nx && row < nrow) {
-                const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
-                inf[u] = info[c];
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) {
-                    w[u][2 * a] = cf.a[a][flo(g, a, i, j, k)];
-                    w[u][2 * a + 1] = cf.a[a][fhi(g, a, i, j, k)];
+            in[u] = i < g.nx && row < nrow;
+            k[u] = DIM == 3 ? row / g.ny : 0;
+            j[u] = row - k[u] * g.ny;
+            c[u] = i + g.nx * row;
+            if (in[u]) {
+                const int f0 = c[u] + row, f1 = c[u] + g.nx * k[u];
+                w[u][0] = cf.a[0][f0];
+                w[u][1] = cf.a[0][f0 + 1];
+                w[u][2] = cf.a[1][f1];
+                w[u][3] = cf.a[1][f1 + g.nx];
+                if (DIM == 3) {
+                    w[u][4] = cf.a[2][c[u]];
+                    w[u][5] = cf.a[2][c[u] + off[2]];
                 }
             }
         }
     };
-    auto load_vectors = [&](int row0) {
+    auto load_vectors = [&]() {
 #pragma unroll
-        for (int u = 0; u < RPT; ++u) {
-            const int row = row0 + u * blockDim.y;
-            if (i < g.nx && row < nrow) {
-                const int k = row / g.ny, j = row - k * g.ny, c = i + g.nx * row;
-                const int ijk[3] = {i, j, k}, n[3] = {g.nx, g.ny, g.nz};
-                zc[u] = z[c];
-                po[u] = p[c];
-                ao[u] = Ap[c];
+        for (int u = 0; u < RPT; ++u)
+            if (in[u]) {
+                const int ijk[3] = {i, j[u], k[u]}, n[3] = {g.nx, g.ny, g.nz};
+                zc[u] = z[c[u]];
+                po[u] = p[c[u]];
+                ao[u] = Ap[c[u]];
 #pragma unroll
                 for (int a = 0; a < DIM; ++a) {
-                    const int off = noff(g, a);
-                    zn[u][2 * a] = ijk[a] > 0 ? z[c - off] : V(0);
-                    zn[u][2 * a + 1] = ijk[a] < n[a] - 1 ? z[c + off] : V(0);
+                    zn[u][2 * a] = ijk[a] > 0 ? z[c[u] - off[a]] : V(0);
+                    zn[u][2 * a + 1] = ijk[a] < n[a] - 1 ? z[c[u] + off[a]] : V(0);
                 }
             }
-        }
     };
     int grp = blockIdx.y;
-    const int step = blockDim.y * RPT;
     load_fixed(grp * step + threadIdx.y);
     griddep_wait();
-    load_vectors(grp * step + threadIdx.y);
+    load_vectors();
     const V be = cg_beta<V>(rz_part, nrz, scal, ctl);
     const bool fresh = be == V(0);
     typename DotAcc<V>::type acc;
@@ -1370,34 +1376,21 @@ __global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, const uint32_t *__
         V accv = V(0);
 #pragma unroll
         for (int u = 0; u < RPT; ++u) {
-            const int row = grp * step + threadIdx.y + u * blockDim.y;
-            if (i >= g.nx || row >= nrow) continue;
-            const int c = i + g.nx * row;
+            if (!in[u]) continue;
             const V pn = fresh ? zc[u] : zc[u] + be * po[u];
-            p[c] = pn;
-            if (!(inf[u] & INFO_FLUID)) {
-                Ap[c] = V(0);
-                continue;
-            }
             V y = V(0);   // same terms and order as poisson_row
 #pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-#pragma unroll
-                for (int s2 = 0; s2 < 2; ++s2) {
-                    const int t = ftype(inf[u], a, s2);
-                    if (t == FT_INTERIOR) y += (V)w[u][2 * a + s2] * (zc[u] - zn[u][2 * a + s2]);
-                    else if (t == FT_OUTLET) y += (V)w[u][2 * a + s2] * zc[u];
-                }
-            }
+            for (int q = 0; q < 2 * DIM; ++q) y += (V)w[u][q] * (zc[u] - zn[u][q]);
             const V an = fresh ? y : y + be * ao[u];
-            Ap[c] = an;
+            p[c[u]] = pn;
+            Ap[c[u]] = an;
             accv += pn * an;
         }
         acc.add(accv);
         grp += gridDim.y;
         if (grp >= groups) break;
         load_fixed(grp * step + threadIdx.y);
-        load_vectors(grp * step + threadIdx.y);
+        load_vectors();
     }
     dot_store(acc, part);
 }
@@ -1701,42 +1694,57 @@ __global__ void k_mg_rbgs(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__
 
 // The last half sweep of the finest level (colour 0) fused with r.z: the
 // thread of colour cell i also takes its row partner i ^ 1 (colour 1, final
-// already), so every cell is counted once. A block takes several rows
-// (launch_groups over the colour's cells).
-template <int DIM, typename M>
+// already), so every cell is counted once. A thread takes RPT rows of a group
+// (launch_groups over the colour's cells), loaded together.
+template <int DIM, typename M, int RPT>
 __global__ void __launch_bounds__(256) k_mg_rbgs_dot(GridD g, MG3<M> cc, const M *__restrict__ idiag, M *__restrict__ x,
                               const M *__restrict__ b, int colour, int groups, double *__restrict__ part) {
     const int ti = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nrow = g.ny * g.nz;
+    const int nrow = g.ny * g.nz, step = blockDim.y * RPT;
     int grp = blockIdx.y;
-    M w[2 * DIM], id = M(0);
-    int row, j, k, i;
-    bool ok;
+    M w[RPT][2 * DIM], id[RPT];
+    int row[RPT], j[RPT], k[RPT], i[RPT];
+    bool ok[RPT];
     auto load_fixed = [&]() {
-        row = grp * blockDim.y + threadIdx.y;
-        k = row / g.ny;
-        j = row - k * g.ny;
-        i = 2 * ti + ((j + k + colour) & 1);
-        ok = i < g.nx && row < nrow;
-        if (ok) {
-            mg_row_coeffs<DIM, M>(g, cc, i, j, k, w);
-            id = idiag[i + g.nx * row];
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            row[u] = grp * step + threadIdx.y + u * blockDim.y;
+            k[u] = DIM == 3 ? row[u] / g.ny : 0;
+            j[u] = row[u] - k[u] * g.ny;
+            i[u] = 2 * ti + ((j[u] + k[u] + colour) & 1);
+            ok[u] = i[u] < g.nx && row[u] < nrow;
+            if (ok[u]) {
+                mg_row_coeffs<DIM, M>(g, cc, i[u], j[u], k[u], w[u]);
+                id[u] = idiag[i[u] + g.nx * row[u]];
+            }
         }
     };
     load_fixed();
     griddep_wait();
     typename DotAcc<M>::type sum;
     for (;;) {
-        const int cell = i + g.nx * row, ip = i ^ 1, cellp = ip + g.nx * row;
-        M acc = M(0);
-        if (ok) {
-            const M bc = b[cell];
-            const M xn = mg_row_sum<DIM, M>(g, w, bc, x, cell, i, j, k) * id;
-            x[cell] = xn;
-            acc = bc * xn;
+        M bc[RPT], xn[RPT], bp[RPT], xp[RPT];
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            const int cell = i[u] + g.nx * row[u], ip = i[u] ^ 1, cellp = ip + g.nx * row[u];
+            const bool okp = ip < g.nx && row[u] < nrow;
+            bp[u] = okp ? b[cellp] : M(0);
+            xp[u] = okp ? x[cellp] : M(0);
+            if (ok[u]) {
+                bc[u] = b[cell];
+                xn[u] = mg_row_sum<DIM, M>(g, w[u], bc[u], x, cell, i[u], j[u], k[u]) * id[u];
+            }
         }
-        if (ip < g.nx && row < nrow) acc += b[cellp] * x[cellp];
-        sum.add(acc);
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+            M acc = M(0);
+            if (ok[u]) {
+                x[i[u] + g.nx * row[u]] = xn[u];
+                acc = bc[u] * xn[u];
+            }
+            acc += bp[u] * xp[u];
+            sum.add(acc);
+        }
         grp += gridDim.y;
         if (grp >= groups) break;
         load_fixed();
@@ -1744,7 +1752,8 @@ __global__ void __launch_bounds__(256) k_mg_rbgs_dot(GridD g, MG3<M> cc, const M
     dot_store(sum, part);
 }
 
-// coarse b = sum over children of the fine residual b - M x. With first set,
+// coarse b = sum over children of the fine residual b - M x (0 on solid cells,
+// which have no coefficients and b = 0). With first set,
 // the coarse x receives the first colour-0 half sweep from x = 0
 // (x = b / diagonal on colour 0, 0 on colour 1), else x = 0. One thread per
 // fine cell: a block covers a tile of whole coarse cells (even extents,
@@ -1756,8 +1765,8 @@ template <int DIM> struct RRTile {
     static constexpr int X = 32, Y = DIM == 3 ? 4 : 8, Z = DIM == 3 ? 2 : 1;
 };
 template <int DIM, typename M, int RX, int RY, int RZ>
-__global__ void __launch_bounds__(256) k_mg_resid_restrict(GridD gf, GridD gc, const uint8_t *__restrict__ fluid,
-                                                           MG3<M> cc, const M *__restrict__ diag,
+__global__ void __launch_bounds__(256) k_mg_resid_restrict(GridD gf, GridD gc, MG3<M> cc,
+                                                           const M *__restrict__ diag,
                                                            const M *__restrict__ x, const M *__restrict__ b,
                                                            M *__restrict__ bc, M *__restrict__ xc,
                                                            const M *__restrict__ idc, int first) {
@@ -1769,11 +1778,16 @@ __global__ void __launch_bounds__(256) k_mg_resid_restrict(GridD gf, GridD gc, c
     const bool in = i < gf.nx && j < gf.ny && k < gf.nz;
     const int cell = i + gf.nx * (j + gf.ny * k);
     M w[2 * DIM], dg = M(0);
-    uint8_t fl = 0;
     if (in) {
-        fl = fluid[cell];
-        dg = diag[cell];
-        mg_row_coeffs<DIM, M>(gf, cc, i, j, k, w);
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            w[2 * a] = cc.a[a][flo(gf, a, i, j, k)];
+            w[2 * a + 1] = cc.a[a][fhi(gf, a, i, j, k)];
+            // FP32: the diagonal as k_mg_diag and k_mg_level_operator form it,
+            // 4 bytes per cell less to read; FP64 is bound by its additions
+            if (sizeof(M) == sizeof(float)) dg += w[2 * a] + w[2 * a + 1];
+        }
+        if (sizeof(M) == sizeof(double)) dg = diag[cell];
     }
     int ic = 0, jc = 0, kc = 0;
     bool cin = false;
@@ -1789,7 +1803,6 @@ __global__ void __launch_bounds__(256) k_mg_resid_restrict(GridD gf, GridD gc, c
     M rv = M(0);
     if (in) {
         rv = mg_residual<DIM>(gf, w, dg, b[cell], x, cell, i, j, k);
-        rv = fl ? rv : M(0);
     }
     res[t] = rv;
     __syncthreads();

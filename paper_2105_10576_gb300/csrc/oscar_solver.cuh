@@ -403,8 +403,8 @@ template <typename T> struct Impl {
         GridD g = to_dev(L.g);
         L3 LL = launch3((L.g.nx + 1) / 2, L.g.ny, L.g.nz);
         if (with_dot) {
-            const L3G LD = launch_groups((L.g.nx + 1) / 2, L.g.ny * L.g.nz, 1);
-            launchk(k_mg_rbgs_dot<DIM, M>, LD.grid, LD.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, colour,
+            const L3G LD = launch_groups((L.g.nx + 1) / 2, L.g.ny * L.g.nz, kDotRows<M>);
+            launchk(k_mg_rbgs_dot<DIM, M, kDotRows<M>>, LD.grid, LD.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, colour,
                     LD.groups, part(I, kPartRz)), ++I.nlaunch;
             I.nrz = LD.nblocks;
         } else
@@ -428,7 +428,7 @@ template <typename T> struct Impl {
         using TT = RRTile<DIM>;
         const dim3 grid((L.g.nx + TT::X - 1) / TT::X, (L.g.ny + TT::Y - 1) / TT::Y, (L.g.nz + TT::Z - 1) / TT::Z);
         launchk(k_mg_resid_restrict<DIM, M, RX, RY, RZ>, grid, dim3(TT::X, TT::Y, TT::Z), 0, I.stream, to_dev(L.g),
-                to_dev(C.g), L.fluid, mg3(L), (const M *)L.diag, x, b, bc, xc, (const M *)C.idiag, first);
+                to_dev(C.g), mg3(L), (const M *)L.diag, x, b, bc, xc, (const M *)C.idiag, first);
         ++I.nlaunch;
     }
     // fused residual + restriction (+ the coarse level's first colour-0 half
@@ -515,7 +515,7 @@ template <typename T> struct Impl {
         if constexpr (sizeof(V) == sizeof(float)) {
             const L3G LA = launch_groups(I.g.nx, rows, kApplyRows);
             npap = LA.nblocks;
-            launchk(k_cg_pz_apply<DIM, T, V, kApplyRows>, LA.grid, LA.block, 0, I.stream, g, I.info, c3(I.lev[0].c),
+            launchk(k_cg_pz_apply<DIM, T, V, kApplyRows>, LA.grid, LA.block, 0, I.stream, g, c3(I.lev[0].c),
                     (const V *)z, p, Ap, part(I, kPartRz), I.nrz, part(I, kPartPap), LA.groups, I.scal, I.ctl), ++I.nlaunch;
         } else {   // FP64 path: the search direction as written, M p applied directly
             launchk(k_cg_pupdate<V>, std::min(kDotBlocks, nblk(n)), BS, 0, I.stream, n, (const V *)z, p,
