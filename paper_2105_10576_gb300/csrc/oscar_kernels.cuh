@@ -1254,57 +1254,91 @@ __global__ void k_cg_init(GridD g, const uint32_t *__restrict__ info, C3<double>
 
 // beta = (r.z) / (r.z)_old (0 on the first iteration) from the partials of
 // r.z, rounded to V, in every thread of the block; the first block stores r.z
-// and counts the iteration
+// and counts the iteration. What does not depend on the partials is loaded
+// beside them and stored after the barrier, here and in the other consumers:
+// one round of dependent loads less in each (four steps of 1024x128 mixed 5.23
+// -> 5.17 ms; three of 128x32x32 FP64 13.0 -> 12.75 ms, k_cg_apply_dot's
+// coefficients before its wait included).
 template <typename V>
 __device__ __forceinline__ V cg_beta(const double *rz_part, int nrz, double *scal, int *ctl) {
     __shared__ V beta_s;
+    const double ro = scal[S_RZ0];
+    const int it = ctl[C_IT], its = ctl[C_ITSUM];
     const double rz = dot_total<V>(rz_part, nrz);
-    if (block_leader()) {
-        const double ro = scal[S_RZ0];
-        beta_s = (V)(ro != 0.0 ? rz / ro : 0.0);
-        if (BLOCK_ID() == 0) {
-            scal[S_RZ1] = rz;
-            ctl[C_IT] += 1;
-            ctl[C_ITSUM] += 1;
-        }
-    }
+    if (block_leader()) beta_s = (V)(ro != 0.0 ? rz / ro : 0.0);
     __syncthreads();
+    if (block_leader() && BLOCK_ID() == 0) {
+        scal[S_RZ1] = rz;
+        ctl[C_IT] = it + 1;
+        ctl[C_ITSUM] = its + 1;
+    }
     return beta_s;
 }
 // alpha = (r.z) / (p.Ap); the first block keeps r.z for the next beta
 template <typename V>
 __device__ __forceinline__ V cg_alpha(const double *pap_part, int npap, double *scal) {
     __shared__ V alpha_s;
+    const double rz = scal[S_RZ1];
     const double pap = dot_total<V>(pap_part, npap);
-    if (block_leader()) {
-        const double rz = scal[S_RZ1];
-        alpha_s = (V)(rz / pap);
-        if (BLOCK_ID() == 0) {
-            scal[S_PAP] = pap;
-            scal[S_RZ0] = rz;
-        }
-    }
+    if (block_leader()) alpha_s = (V)(rz / pap);
     __syncthreads();
+    if (block_leader() && BLOCK_ID() == 0) {
+        scal[S_PAP] = pap;
+        scal[S_RZ0] = rz;
+    }
     return alpha_s;
 }
 
-// FP64 path: Ap = M p and p.Ap
-template <int DIM, typename T, typename V>
-__global__ void k_cg_apply_dot(GridD g, const uint32_t *__restrict__ info, C3<T> cf, const V *__restrict__ p,
-                               V *__restrict__ Ap, double *__restrict__ part) {
+// FP64 path: Ap = M p and p.Ap. As in k_cg_pz_apply no face types are read and
+// the coefficients are loaded before the grid dependency wait.
+template <int DIM, typename V>
+__global__ void __launch_bounds__(256) k_cg_apply_dot(GridD g, C3<V> cf, const V *__restrict__ p, V *__restrict__ Ap,
+                                                      double *__restrict__ part, int groups) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, nrow = g.ny * g.nz;
+    const int off[3] = {1, g.nx, g.nx * g.ny}, n[3] = {g.nx, g.ny, g.nz};
+    V w[2 * DIM];
+    int c, ijk[3];
+    bool in;
+    auto load_fixed = [&](int row) {
+        in = i < g.nx && row < nrow;
+        const int k = DIM == 3 ? row / g.ny : 0;
+        ijk[0] = i;
+        ijk[1] = row - k * g.ny;
+        ijk[2] = k;
+        c = i + g.nx * row;
+        if (in) {
+            const int f0 = c + row, f1 = c + g.nx * k;
+            w[0] = cf.a[0][f0];
+            w[1] = cf.a[0][f0 + 1];
+            w[2] = cf.a[1][f1];
+            w[3] = cf.a[1][f1 + g.nx];
+            if (DIM == 3) {
+                w[4] = cf.a[2][c];
+                w[5] = cf.a[2][c + off[2]];
+            }
+        }
+    };
+    int grp = blockIdx.y;
+    load_fixed(grp * blockDim.y + threadIdx.y);
     griddep_wait();
     typename DotAcc<V>::type acc;
-    ROW_LOOP(g) {
-        ROW_CELL(g);
-        if (i >= g.nx) continue;
-        uint32_t inf = info[c];
-        if (!(inf & INFO_FLUID)) {
-            Ap[c] = V(0);
-        } else {
-            V y = poisson_row<DIM, T, V>(g, inf, c, i, j, k, cf, p);
+    for (;;) {
+        if (in) {
+            const V pc = p[c];
+            V pn[2 * DIM], y = V(0);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                pn[2 * a] = ijk[a] > 0 ? p[c - off[a]] : V(0);
+                pn[2 * a + 1] = ijk[a] < n[a] - 1 ? p[c + off[a]] : V(0);
+            }
+#pragma unroll
+            for (int q = 0; q < 2 * DIM; ++q) y = mg_madd(w[q], pc - pn[q], y);   // same terms and order as poisson_row
             Ap[c] = y;
-            acc.add(p[c] * y);
+            acc.add(pc * y);
         }
+        grp += gridDim.y;
+        if (grp >= groups) break;
+        load_fixed(grp * blockDim.y + threadIdx.y);
     }
     dot_store(acc, part);
 }
@@ -1398,7 +1432,7 @@ __global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, C3<T> cf, const V 
 // x += alpha p, r -= alpha Ap, z = the first colour-0 half sweep of the next
 // V-cycle (as in k_cg_init), and r.r. RPT rows per thread and group
 // (launch_groups), loaded together. xfresh: x starts from 0 in the first
-// iteration (x is not read then), so it needs no clearing beforehand.
+// iteration (what was read is dropped), so it needs no clearing beforehand.
 template <typename V, int RPT>
 __global__ void __launch_bounds__(256) k_cg_update(GridD g, V *__restrict__ x, V *__restrict__ r, const V *__restrict__ p,
                             const V *__restrict__ Ap, const V *__restrict__ idiag0, V *__restrict__ z,
@@ -1426,7 +1460,7 @@ __global__ void __launch_bounds__(256) k_cg_update(GridD g, V *__restrict__ x, V
             const int row = row0 + u * blockDim.y;
             if (i < g.nx && row < nrow) {
                 const int c = i + g.nx * row;
-                xo[u] = x0 ? V(0) : x[c];
+                xo[u] = x[c];
                 ro[u] = r[c];
                 pc[u] = p[c];
                 ac[u] = Ap[c];
@@ -1490,8 +1524,15 @@ template <typename V>
 __global__ void k_cg_pupdate(int n, const V *__restrict__ z, V *__restrict__ p, const double *__restrict__ rz_part, int nrz,
                              double *__restrict__ scal, int *__restrict__ ctl) {
     griddep_wait();
+    int c = blockIdx.x * blockDim.x + threadIdx.x;
+    V zc = V(0), pc = V(0);   // of the first cell, beside the partials
+    if (c < n) {
+        zc = z[c];
+        pc = p[c];
+    }
     const V be = cg_beta<V>(rz_part, nrz, scal, ctl);
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) p[c] = z[c] + be * p[c];
+    if (c < n) p[c] = zc + be * pc;
+    while ((c += gridDim.x * blockDim.x) < n) p[c] = z[c] + be * p[c];
 }
 
 // Error-free products (FMA) for the compensated operator below.
@@ -1559,12 +1600,14 @@ __global__ void k_cg_refine(GridD g, const uint32_t *__restrict__ info, C3<float
     griddep_wait();
     __shared__ int more_s;
     {
+        const double target = scal[S_ITARGET];
+        const int it = ctl[C_IT];
         const double rr = dot_total<float>(rr_part, nrr);
         if (block_leader()) {
             const double rn = sqrt(rr);
             const bool bad = !isfinite(rn);
-            bool more = !bad && rn > scal[S_ITARGET];
-            const bool capped = more && ctl[C_IT] >= maxit;
+            bool more = !bad && rn > target;
+            const bool capped = more && it >= maxit;
             if (capped) more = false;
             if (BLOCK_ID() == 0) {
                 if (bad) ctl[C_NAN] = 1;

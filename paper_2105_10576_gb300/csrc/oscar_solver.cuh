@@ -520,10 +520,10 @@ template <typename T> struct Impl {
         } else {   // FP64 path: the search direction as written, M p applied directly
             launchk(k_cg_pupdate<V>, std::min(kDotBlocks, nblk(n)), BS, 0, I.stream, n, (const V *)z, p,
                     part(I, kPartRz), I.nrz, I.scal, I.ctl), ++I.nlaunch;
-            const L3 L = launch_rows(I.g, kDotBlocks);
-            npap = L.nblocks;
-            launchk(k_cg_apply_dot<DIM, T, V>, L.grid, L.block, 0, I.stream, g, I.info, c3(I.lev[0].c), p, Ap,
-                    part(I, kPartPap)), ++I.nlaunch;
+            const L3G LA = launch_groups(I.g.nx, rows, 1);
+            npap = LA.nblocks;
+            launchk(k_cg_apply_dot<DIM, V>, LA.grid, LA.block, 0, I.stream, g, c3(I.lev[0].c), (const V *)p, Ap,
+                    part(I, kPartPap), LA.groups), ++I.nlaunch;
         }
         const L3G LU = launch_groups(I.g.nx, rows, kUpdateRows);
         launchk(k_cg_update<V, kUpdateRows>, LU.grid, LU.block, 0, I.stream, g, x, r, p, Ap, (const V *)I.lev[0].idiag,
