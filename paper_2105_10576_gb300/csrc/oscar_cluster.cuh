@@ -1112,47 +1112,131 @@ __global__ void __launch_bounds__(kGjThreads) k_mg_inverse_dense(GridD g, MG3<fl
 
 // FP64: LDL^T without pivoting in band form, cells ordered with the shortest
 // axis fastest, so that the band is the product of the two shortest extents (4
-// to about 25 for at most 128 cells), then L D L^T x = e_j for every column j
-// of the inverse: n^2 (2 bw + 1) operations instead of the n^3 of a dense
-// elimination, which the SM's two FP64 FMAs per clock take 1.1 ms for at 128
-// cells. What is left is a serial chain along the cells: one warp factorises,
-// and a thread solves one column with the last bw values in registers, the
-// newest one's term added last, so that the chain is one FMA per cell. Blocks
-// of one warp (the factorisation repeated in each) share the columns, since
-// four warps on one SM would be bound by its FP64 rate. Rows of cells that are
-// solid or have no coefficients, and of pivots that vanish, give a zero row
-// and column.
+// to 25 for at most 128 cells), then L D L^T x = e_j for every column j of the
+// inverse: n^2 (2 bw + 1) operations instead of the n^3 of a dense elimination,
+// which the SM's two FP64 FMAs per clock take 1.1 ms for at 128 cells. What is
+// left is a serial chain along the cells, halved by working from both ends: h
+// cells from the first and h from the last one on, by the two halves of a warp
+// in the same instructions, then the bw or bw + 1 cells between them. A column
+// of the factor costs a division and two FMAs in a row, a cell of a solve one
+// FMA (a thread keeps the last bw values of its column in registers, the
+// newest one's term added last; the next cell's factors are loaded before).
+// A block is one warp with 16 columns of the inverse, the factorisation
+// repeated in each: several warps on one SM would be bound by its FP64 rate.
+// 60 us for 32x4 cells, 98 for 16x8, 333 for 5x5x5 (from one end alone 130, 182
+// and 643 us).
+// Rows of cells that are solid or have no coefficients, and of pivots that
+// vanish (against the diagonal they came from), give a zero row and column.
+constexpr int kBandCols = 16;
+// the rows of the factor a half keeps, and the shared memory of the kernel
+struct BandShape { int n, bw, h, s, rows; };   // s cells in the middle; rows = h + s of either half
+__host__ __device__ inline BandShape band_shape(int n, int bw) {
+    BandShape b;
+    b.n = n;
+    b.bw = bw;
+    b.h = n > bw ? (n - bw) / 2 : 0;
+    b.s = n - 2 * b.h;
+    b.rows = b.h + b.s;
+    return b;
+}
+// per half: the matrix rows (bw + 1 each) and the factor (bw each) and pivots;
+// the columns of the inverse
+__host__ __device__ inline size_t band_words(const BandShape &b) {
+    return 2 * (size_t)b.rows * (2 * b.bw + 3) + (size_t)b.n * kBandCols;
+}
+// Substitution over count rows: row q takes start(q) less the products of
+// load(q, d) with the value d rows back (win[d - 1]), and goes to store(q). The
+// operands of a row are loaded while the row before is worked.
+template <typename M, int W, typename FL, typename FA, typename FS>
+__device__ __forceinline__ void band_rows(M (&win)[W], int bw, int count, FL load, FA start, FS store) {
+    M l[W], ln[W];
+#pragma unroll
+    for (int d = 0; d < W; ++d) l[d] = M(0);
+    if (count > 0) {
+#pragma unroll
+        for (int d = 0; d < W; ++d) if (d < bw) l[d] = load(0, d + 1);
+    }
+    M a = count > 0 ? start(0) : M(0);
+#pragma unroll 1
+    for (int q = 0; q < count; ++q) {
+        M an = M(0);
+#pragma unroll
+        for (int d = 0; d < W; ++d) ln[d] = M(0);
+        if (q + 1 < count) {
+#pragma unroll
+            for (int d = 0; d < W; ++d) if (d < bw) ln[d] = load(q + 1, d + 1);
+            an = start(q + 1);
+        }
+#pragma unroll
+        for (int d = W; d >= 1; --d) a = fma(-l[d - 1], win[d - 1], a);   // entries beyond the band are 0
+        store(q, a);
+#pragma unroll
+        for (int d = W - 1; d > 0; --d) win[d] = win[d - 1];
+        win[0] = a;
+#pragma unroll
+        for (int d = 0; d < W; ++d) l[d] = ln[d];
+        a = an;
+    }
+}
+// one column of the inverse per thread pair (t, t + 16): half 0 works the rows
+// from the first cell on, half 1 those from the last one on (its row q is band
+// row n - 1 - q), both the middle rows
 template <typename M, int W>
-__device__ __forceinline__ void band_solve(const M *B, const M *rD, M *Y, int n, int bw, int col, bool live) {
-    // B[i (bw + 1) + d] = L(i, i - d); Y[i 32 + lane]
+__device__ __forceinline__ void band_solve(const BandShape S, const M *L0, const M *L1, const M *D0, const M *D1, M *Y, int col, bool live) {
+    const int t = threadIdx.x, half = t / kBandCols, lane = t % kBandCols, bw = S.bw, h = S.h, s = S.s, n = S.n;
+    const M *L = half ? L1 : L0, *D = half ? D1 : D0;   // L[i bw + d - 1] = L(i, i - d)
+    const int mine = half ? n - 1 - col : col;          // the unit entry, in this half's row order
+    auto y = [&](int q) -> M & { return Y[(half ? n - 1 - q : q) * kBandCols + lane]; };
     M win[W];
-    const int lane = threadIdx.x & 31, st = bw + 1;
 #pragma unroll
     for (int d = 0; d < W; ++d) win[d] = M(0);
-#pragma unroll 1
-    for (int i = 0; i < n; ++i) {   // L y = e_col
-        M a = i == col && live ? M(1) : M(0);
+    // forward over this half's rows
+    band_rows<M, W>(win, bw, h, [&](int q, int d) { return L[q * bw + d - 1]; },
+                          [&](int q) { return live && q == mine ? M(1) : M(0); }, [&](int q, M a) { y(q) = a; });
+    // what they put into the middle rows: half 0 leaves it in Y, half 1 adds
+    M mid[W + 1];
 #pragma unroll
-        for (int d = W; d >= 1; --d)
-            if (d <= bw) a = fma(-B[i * st + d], win[d - 1], a);   // entries before the first cell are 0
+    for (int q = 0; q <= W; ++q) {
+        M a = M(0);
+        if (q < s) {
 #pragma unroll
-        for (int d = W - 1; d > 0; --d) win[d] = win[d - 1];
-        win[0] = a;
-        Y[i * 32 + lane] = a;
+            for (int d = W; d >= 1; --d)
+                if (d <= bw && d > q) a = fma(-L[(h + q) * bw + d - 1], win[d > q ? d - 1 - q : 0], a);
+        }
+        mid[q] = a;
     }
+    if (half == 0) {
 #pragma unroll
-    for (int d = 0; d < W; ++d) win[d] = M(0);
-#pragma unroll 1
-    for (int i = n - 1; i >= 0; --i) {   // L^T x = D^-1 y
-        M a = Y[i * 32 + lane] * rD[i];
-#pragma unroll
-        for (int d = W; d >= 1; --d)
-            if (d <= bw && i + d < n) a = fma(-B[(i + d) * st + d], win[d - 1], a);
-#pragma unroll
-        for (int d = W - 1; d > 0; --d) win[d] = win[d - 1];
-        win[0] = a;
-        Y[i * 32 + lane] = a;
+        for (int q = 0; q <= W; ++q)
+            if (q < s) Y[(h + q) * kBandCols + lane] = mid[q] + (live && h + q == col ? M(1) : M(0));
     }
+    __syncwarp();
+    if (half == 1) {
+#pragma unroll
+        for (int q = 0; q <= W; ++q)
+            if (q < s) Y[(h + s - 1 - q) * kBandCols + lane] += mid[q];
+    }
+    __syncwarp();
+    if (half == 0) {   // the middle rows: forward, then back
+#pragma unroll
+        for (int d = 0; d < W; ++d) win[d] = M(0);
+        band_rows<M, W>(win, bw, s, [&](int q, int d) { return q >= d ? L0[(h + q) * bw + d - 1] : M(0); },
+                              [&](int q) { return Y[(h + q) * kBandCols + lane]; },
+                              [&](int q, M a) { Y[(h + q) * kBandCols + lane] = a; });
+#pragma unroll
+        for (int d = 0; d < W; ++d) win[d] = M(0);
+        band_rows<M, W>(win, bw, s,
+                              [&](int q, int d) { return q >= d ? L0[(h + s - 1 - q + d) * bw + d - 1] : M(0); },
+                              [&](int q) { return Y[(h + s - 1 - q) * kBandCols + lane] * D0[h + s - 1 - q]; },
+                              [&](int q, M a) { Y[(h + s - 1 - q) * kBandCols + lane] = a; });
+    }
+    __syncwarp();
+    // back over this half's rows
+#pragma unroll
+    for (int d = 0; d < W; ++d) win[d] = d < s && d < bw ? y(h + d) : M(0);
+    band_rows<M, W>(win, bw, h, [&](int q, int d) { return L[(h - 1 - q + d) * bw + d - 1]; },
+                          [&](int q) { return y(h - 1 - q) * D[h - 1 - q]; }, [&](int q, M a) { y(h - 1 - q) = a; });
+    __syncwarp();
 }
 template <int DIM, typename M>
 __global__ void __launch_bounds__(32) k_mg_inverse_band(GridD g, MG3<M> cc, const M *__restrict__ diag,
@@ -1175,53 +1259,92 @@ __global__ void __launch_bounds__(32) k_mg_inverse_band(GridD g, MG3<M> cc, cons
     st[ax[1]] = e[ax[0]];
     st[ax[2]] = e[ax[0]] * e[ax[1]];
     const int bw = st[ax[2]], W = bw + 1;
-    M *B = (M *)sm;                       // B[r W + d] = A(r, r - d), then L (d > 0) and D (d = 0)
-    M *rD = B + (size_t)kExactCells * W;
-    M *Y = rD + kExactCells;              // Y[i 32 + lane]: this block's columns of the inverse, band order
+    const BandShape S = band_shape(n, bw);
+    // rows of a half: A[i W + d] = A(i, i - d), then the Schur complement;
+    // L[i bw + d - 1] = L(i, i - d); rD = reciprocal pivots. Half 1 counts rows
+    // and columns from the last cell back
+    const int half = t / kBandCols, lane = t % kBandCols;
+    M *A0 = (M *)sm, *A1 = A0 + S.rows * W, *L0 = A1 + S.rows * W, *L1 = L0 + S.rows * bw, *D0 = L1 + S.rows * bw;
+    M *D1 = D0 + S.rows, *T0 = D1 + S.rows, *T1 = T0 + S.rows, *Y = T1 + S.rows;   // T: pivots below it vanish
     __shared__ int cell_s[kExactCells];   // cell of a band index
-    for (int q = t; q < n * W; q += 32) B[q] = M(0);
+    __shared__ unsigned short tri_s[kExactCells * 4];   // (u, v), v <= u, of the entries of a column's update
+    const int total = 2 * S.rows * (2 * bw + 3);
+    for (int q = t; q < total; q += 32) A0[q] = M(0);
+    for (int u = t; u < bw; u += 32)
+        for (int v = 0; v <= u; ++v) tri_s[u * (u + 1) / 2 + v] = (unsigned short)(u << 8 | v);
     __syncwarp();
     for (int c = t; c < n; c += 32) {
         const int i = c % g.nx, j = (c / g.nx) % g.ny, k = c / (g.nx * g.ny);
-        const int r = i * st[0] + j * st[1] + k * st[2];
+        const int r = i * st[0] + j * st[1] + k * st[2], rr = n - 1 - r;
         cell_s[r] = c;
         const M d = diag[c];
         const bool live = fluid[c] && d > M(0);
         if (!live) continue;
-        B[r * W] = d;
+        const M tiny = d * M(1e-13);
+        if (r < S.rows) {
+            A0[r * W] = d;
+            T0[r] = tiny;
+        } else {
+            A1[rr * W] = d;
+            T1[rr] = tiny;
+        }
         const int ijk[3] = {i, j, k};
 #pragma unroll
-        for (int a = 0; a < DIM; ++a)   // the low neighbours are those of smaller band index
-            if (ijk[a] > 0) B[r * W + st[a]] = -cc.a[a][flo(g, a, i, j, k)];
-    }
-    __syncwarp();
-    // right-looking factorisation: after step k the columns beyond k hold the
-    // Schur complement and column k the entries of L
-    for (int k = 0; k < n; ++k) {
-        const M d = B[k * W];
-        const M rd = d > M(0) ? M(1) / d : M(0);
-        const int m = min(bw, n - 1 - k);
-        for (int q = t; q < m * m; q += 32) {   // A(k+1+u, k+1+v) -= A(k+1+u, k) A(k+1+v, k) / d, v <= u
-            const int u = q / m, v = q - u * m;
-            if (v <= u) {
-                M *a = B + (k + 1 + u) * W + (u - v);
-                *a = fma(-(B[(k + 1 + u) * W + u + 1] * rd), B[(k + 1 + v) * W + v + 1], *a);
-            }
+        for (int a = 0; a < DIM; ++a) {   // the low neighbour is the one of smaller band index
+            if (ijk[a] == 0) continue;
+            const M w = -cc.a[a][flo(g, a, i, j, k)];
+            if (r < S.rows) A0[r * W + st[a]] = w;
+            else A1[(n - 1 - (r - st[a])) * W + st[a]] = w;   // row r - st[a] of half 1: st[a] after r
         }
-        __syncwarp();
-        for (int u = t; u < m; u += 32) B[(k + 1 + u) * W + u + 1] *= rd;
-        if (t == 0) rD[k] = rd;
+    }
+    __syncwarp();
+    // right-looking: after step k the columns beyond k hold the Schur
+    // complement and column k of L the factor
+    const int np = bw * (bw + 1) / 2;
+    M *A = half ? A1 : A0, *L = half ? L1 : L0, *D = half ? D1 : D0, *T = half ? T1 : T0;
+#pragma unroll 1
+    for (int k = 0; k < S.h; ++k) {   // both halves
+        const M d = A[k * W];
+        const M rd = d > T[k] ? M(1) / d : M(0);
+        for (int q = lane; q < np; q += kBandCols) {   // A(k+1+u, k+1+v) -= A(k+1+u, k) A(k+1+v, k) / d
+            const int u = tri_s[q] >> 8, v = tri_s[q] & 255;
+            const M lu = A[(k + 1 + u) * W + u + 1] * rd;
+            M *x = A + (k + 1 + u) * W + (u - v);
+            *x = fma(-lu, A[(k + 1 + v) * W + v + 1], *x);
+            if (v == 0) L[(k + 1 + u) * bw + u] = lu;
+        }
+        if (lane == 0) D[k] = rd;
         __syncwarp();
     }
-    const int col = blockIdx.x * 32 + t;
-    const bool live = col < n && rD[col] > M(0);
-    if (bw <= 4) band_solve<M, 4>(B, rD, Y, n, bw, col, live);
-    else if (bw <= 8) band_solve<M, 8>(B, rD, Y, n, bw, col, live);
-    else if (bw <= 12) band_solve<M, 12>(B, rD, Y, n, bw, col, live);
-    else band_solve<M, 26>(B, rD, Y, n, bw, col, live);
+    // the middle rows: half 1's share of them to half 0's, then on with half 0
+    for (int q = t; q < S.s * W; q += 32) {
+        const int u = q / W, d = q - u * W, v = u - d;
+        if (v >= 0) A0[(S.h + u) * W + d] += A1[(S.h + S.s - 1 - v) * W + d];
+    }
     __syncwarp();
+#pragma unroll 1
+    for (int k = S.h; k < S.rows; ++k) {
+        const M d = A0[k * W];
+        const M rd = d > T0[k] ? M(1) / d : M(0);
+        const int m = S.rows - 1 - k < bw ? S.rows - 1 - k : bw, nm = m * (m + 1) / 2;
+        for (int q = t; q < nm; q += 32) {
+            const int u = tri_s[q] >> 8, v = tri_s[q] & 255;
+            const M lu = A0[(k + 1 + u) * W + u + 1] * rd;
+            M *x = A0 + (k + 1 + u) * W + (u - v);
+            *x = fma(-lu, A0[(k + 1 + v) * W + v + 1], *x);
+            if (v == 0) L0[(k + 1 + u) * bw + u] = lu;
+        }
+        if (t == 0) D0[k] = rd;
+        __syncwarp();
+    }
+    const int col = blockIdx.x * kBandCols + lane;
+    const bool live = col < n && (col < S.rows ? D0[col] : D1[n - 1 - col]) > M(0);
+    if (bw <= 4) band_solve<M, 4>(S, L0, L1, D0, D1, Y, col, live);
+    else if (bw <= 8) band_solve<M, 8>(S, L0, L1, D0, D1, Y, col, live);
+    else if (bw <= 12) band_solve<M, 12>(S, L0, L1, D0, D1, Y, col, live);
+    else band_solve<M, 25>(S, L0, L1, D0, D1, Y, col, live);
     if (col < n)
-        for (int r = 0; r < n; ++r) inv[cell_s[r] * n + cell_s[col]] = Y[r * 32 + t];
+        for (int r = half; r < n; r += 2) inv[cell_s[r] * n + cell_s[col]] = Y[r * kBandCols + lane];
 }
 
 }  // namespace oscar

@@ -277,7 +277,7 @@ template <typename T> struct Impl {
             launchk(k_mg_inverse_dense<DIM>, 1, kGjThreads, 0, st, to_dev(E.g), mg3(E), (const M *)E.diag,
                     (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, (const int *)I.ctl), ++I.nlaunch;
         else
-            launchk(k_mg_inverse_band<DIM, M>, (E.g.ncell + 31) / 32, 32, inverse_smem(E.g), st, to_dev(E.g), mg3(E),
+            launchk(k_mg_inverse_band<DIM, M>, (E.g.ncell + kBandCols - 1) / kBandCols, 32, inverse_smem(E.g), st, to_dev(E.g), mg3(E),
                     (const M *)E.diag, (const uint8_t *)E.fluid, (M *)I.cl_inv, I.coarse_refresh, (const int *)I.ctl),
                 ++I.nlaunch;
         {   // the images of the levels the solves work in a cluster
@@ -303,7 +303,7 @@ template <typename T> struct Impl {
     static size_t inverse_smem(const GridH &g) {
         int e[3] = {g.nx, g.ny, g.nz};
         std::sort(e, e + 3);
-        return (kExactCells * (size_t)(e[0] * e[1] + 2) + 32 * (size_t)g.ncell) * sizeof(M);
+        return band_words(band_shape(g.ncell, e[0] * e[1])) * sizeof(M);
     }
 
     // Levels l0 .. of a cluster of at most nc_max CTAs and their shared-memory
