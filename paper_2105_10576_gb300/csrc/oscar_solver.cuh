@@ -172,11 +172,15 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // is still bound by its latency; in FP64 they are bound by FP64 issue above
 // 1024 cells). A 2D grid of at most solve_cells is solved whole in one cluster
 // when its vectors fit the shared memory.
-constexpr int kVcycleCtas = 16, kVcycleThreads = 512, kSolveCtas = 16;
+constexpr int kVcycleCtas = 16, kVcycleThreads = 512;
 // fewer threads make the block and cluster barriers shorter, more take larger
 // slabs with fewer entries per thread (128x16 FP64: 256 threads 8.03 ms per
 // pass, 512 8.53; 512x64 mixed: 4.25 and 3.64)
 inline int solve_threads(int ncell) { return ncell <= 8192 ? 256 : 512; }
+// CTAs of the cluster: fewer exchange less, more have shorter slabs. FP32 at
+// 128x16 (six sub-steps): 8 CTAs 2.48 ms, 16 2.55; at 211x26 3.92 and 3.56.
+// FP64, bound by the SM's FP64 rate: 128x16 4.74 and 4.52.
+template <typename T> inline int solve_ctas(int ncell) { return sizeof(T) == sizeof(float) && ncell <= 2048 ? 8 : 16; }
 template <typename T> struct ClRule;
 template <> struct ClRule<float> {
     static constexpr long long vcycle_cells = 8, solve_cells = 65536;
@@ -883,7 +887,7 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     I.solve_nc = 0;
     if (I.cta_global && I.g.dim == 2 && I.g.ncell <= ClRule<T>::solve_cells) {
         ClSolve A;
-        I.solve_smem = Impl<T>::cl_fill(I, P, 0, kSolveCtas, &A);
+        I.solve_smem = Impl<T>::cl_fill(I, P, 0, solve_ctas<T>(I.g.ncell), &A);
         if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) I.solve_nc = P.nc;   // even slab starts
     }
     return 0;

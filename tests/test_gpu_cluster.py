@@ -1,0 +1,75 @@
+"""The thread-block-cluster kernels against the paths they stand in for.
+
+A pressure solve of a small 2D grid runs in one cluster, and the coarse levels
+of larger grids in another; with cta_global=0 the same levels are worked by
+per-level kernels and a cluster of one CTA. Mixed path: the same operations on
+the same operands, so the fields are bitwise equal. FP64 path: other orders of
+summation; with the solves converged to 1e-13 the fields agree to 1e-9 of
+their largest value.
+"""
+import numpy as np
+import pytest
+
+from paper_2105_10576_gb300 import inputs
+from paper_2105_10576_gb300 import oscar as ox
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _sim(shape, prec, rtol, seed, **sched):
+    nx, ny, nz = shape
+    c = inputs.random_small_case(seed, nx, ny, nz=nz, dim=3 if nz > 1 else 2)
+    p = dict(c.params, precision=prec, cg_rtol=rtol, conv_mode=inputs.CONV_PRES_RESID, conv_tol=0.0)
+    g = ox.Oscar(p, c.solid, c.alpha0)
+    g.set_schedule(sched)
+    dt_cfl, dt_b, dt_vd, N = ox.oscar_timesteps(p, 0.02)
+    return g, p, dt_vd, N
+
+
+# one, two and three slab columns per CTA, ragged slabs, the line between 8 and
+# 16 CTAs (2048 cells) and between 256 and 512 threads (8192), the largest grid
+# (65536 mixed, 16384 FP64) and the first beyond it; in 3D every coarsening
+# ratio and slabs that end inside the grid
+SHAPES = [(16, 8, 1), (37, 19, 1), (64, 32, 1), (129, 16, 1), (65, 33, 1), (256, 32, 1), (241, 35, 1), (257, 63, 1),
+          (512, 128, 1), (513, 128, 1), (33, 9, 21), (48, 40, 7), (50, 27, 26), (70, 12, 12)]
+
+
+@pytest.mark.parametrize("prec", [inputs.PREC_MIXED, inputs.PREC_FP64])
+@pytest.mark.parametrize("sweeps", [dict(), dict(mg_nu=1, mg_nu_mid=3, mg_nu_cta=1, cta_cells=256)])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_cluster_is_the_launched_path(shape, sweeps, prec):
+    mixed = prec == inputs.PREC_MIXED
+    out = []
+    for flag in (1, 0):
+        g, p, dt_vd, N = _sim(shape, prec, 1e-8 if mixed else 1e-13, 5 + shape[0], cta_global=flag, **sweeps)
+        g.drag_step(dt_vd)
+        g.relax(dt_vd / N, 2)
+        out.append([g.field(w) for w in (ox.FIELD_ALPHA, ox.FIELD_P, ox.FIELD_U, ox.FIELD_U + 1, ox.FIELD_PHI_VD)])
+        g.close()
+    for x, y in zip(*out):
+        if mixed:
+            assert np.array_equal(x, y)
+        else:
+            assert np.abs(x - y).max() <= 1e-9 * np.abs(y).max()
+
+
+# grids of one level: the V-cycle is the explicit inverse itself, so PCG needs
+# one iteration (FP64; one more for rounding), or with the FP32 inverse, off by
+# at most 1e-2 at the grids' density contrast, three per defect-correction trip
+# of 1e-4, three trips to 1e-9. Bands of 1 to 25, an even and an odd middle,
+# grids shorter than their band, the full 128 cells.
+@pytest.mark.parametrize("prec,most", [(inputs.PREC_FP64, 2), (inputs.PREC_MIXED, 9)])
+@pytest.mark.parametrize("shape", [(32, 4, 1), (16, 8, 1), (11, 11, 1), (19, 4, 1), (9, 3, 1), (4, 3, 1), (4, 32, 1),
+                                   (5, 5, 5), (4, 5, 6), (32, 2, 2), (2, 3, 21), (8, 4, 4), (3, 3, 3)])
+def test_coarsest_inverse(shape, prec, most):
+    g, p, dt_vd, N = _sim(shape, prec, 1e-9, 3, coarse_refresh=1)
+    g.drag_step(dt_vd)
+    assert g.stats()["cg_iters_total"] <= most * p["n_piso"]
+    assert np.isfinite(g.field(ox.FIELD_P)).all()
+    g.close()
