@@ -81,22 +81,25 @@ def grid_counts(c):
 def kernel_bytes(name: str, c, e: int):
     """Algorithmic bytes of one finest-level launch of kernel `name`
     ("k_x<args>"), or None for kernels without a streaming byte model (the
-    single-CTA coarse V-cycle, set-up and control kernels)."""
+    kernels that work in one thread-block cluster, set-up and control kernels)."""
     n, F, R, d = grid_counts(c)
     base = name.split("<")[0]
     if base == "k_mg_rbgs":          # x of every cell, b and 1/diag of one colour, half of x written, each face once
+        pro, dg = ([a.strip(" >") for a in name.split(",")] + ["", ""])[2:4]
         b = n * (e + e + e / 2) + F * e
-        return b + n / R * e if ", true>" in name else b   # + the coarse x of the folded prolongation
+        if dg == "true":             # 1/diag formed from the faces
+            b -= n * e / 2
+        return b + n / R * e if pro == "true" else b   # + the coarse x of the folded prolongation
     if base == "k_mg_rbgs_dot":      # + r and z of the other colour for r.z
         return n * (e + e + e / 2) + F * e + n * e
-    if base == "k_cg_pz_apply":      # z, p, Ap and info in; p, Ap out; each face once
-        return n * (5 * e + 4) + F * e
-    if base == "k_cg_apply_dot":     # FP64 path: p and info in, Ap out
-        return n * (2 * e + 4) + F * e
+    if base == "k_cg_pz_apply":      # z, p, Ap in; p, Ap out; each face once
+        return n * 5 * e + F * e
+    if base == "k_cg_apply_dot":     # FP64 path: p in, Ap out
+        return n * 2 * e + F * e
     if base == "k_cg_update":        # x, r, p, Ap, 1/diag in; x, r, z out
         return n * 8 * e
-    if base == "k_mg_resid_restrict":  # x, b, diag, fluid in; coarse b, x out; each face once
-        return n * (3 * e + 1) + n / R * 2 * e + F * e
+    if base == "k_mg_resid_restrict":  # x, b (FP64: and diag) in; coarse b, x out; each face once
+        return n * (3 if e == 8 else 2) * e + n / R * 2 * e + F * e
     if base == "k_momentum_H":       # v, vold, hbya (d each), alpha, rA, grad v (d*d), info; convecting faces once
         return n * (e * (3 * d + 2 + d * d) + 4) + F * e
     if base == "k_transport_low":

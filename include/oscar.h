@@ -223,7 +223,7 @@ int oscar_get_schedule(oscar_handle h, oscar_schedule *out);
 /* Replace the schedule (waits for the stream; the step graphs are rebuilt at
  * the next step call). OSCAR_E_INVALID_ARG for a value out of range, while an
  * asynchronous step is pending, or when the coarse levels chosen by cta_cells
- * do not fit the coarse CTA's shared memory; the schedule is then unchanged. */
+ * do not fit the cluster's shared memory; the schedule is then unchanged. */
 int oscar_set_schedule(oscar_handle h, const oscar_schedule *s);
 
 /* Release all device memory of the instance. */

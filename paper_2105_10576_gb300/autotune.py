@@ -1,8 +1,8 @@
 """Measuring autotuner of the pressure solver's schedule (oscar_schedule).
 
 The multigrid schedule (smoothing sweeps per level group, which levels go to
-the single coarse CTA, how often the coarsest level's inverse is refreshed)
-and the block shape of the cell kernels change how fast the pressure solves
+the coarse thread-block cluster, how often the coarsest level's inverse is
+refreshed) and the block shape of the cell kernels change how fast the pressure solves
 of an instance converge and run, not what they converge to. The best choice
 depends on the grid: on a small 2D grid every launch is latency-bound and
 fewer sweeps win, on a large 3D grid more sweeps pay for themselves through

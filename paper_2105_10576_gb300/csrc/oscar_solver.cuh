@@ -400,6 +400,15 @@ template <typename T> struct Impl {
     static M *lx(Instance &I, int l, V *z) { return l == 0 ? (M *)z : (M *)I.lev[l].x; }
     static M *lb(Instance &I, int l, V *r) { return l == 0 ? (M *)r : (M *)I.lev[l].b; }
 
+    // FP32 levels whose half sweeps stream from HBM (the coefficients, x, b and
+    // the inverse diagonal beyond what L2 keeps beside the other vectors) form
+    // the inverse diagonal instead of reading it. Whole steps without and with
+    // it: 256x128x128 (101 MB) 24.08 and 23.60 ms; 208x104x104 (54 MB) 14.78 and
+    // 15.11, 2048x1024 (42 MB) 21.73 and 22.00.
+    static constexpr double kStreamBytes = 80e6;
+    static bool diag_from_rows(const GridH &g) {
+        return sizeof(M) == sizeof(float) && (g.dim + 3.0) * g.ncell * sizeof(M) >= kStreamBytes;
+    }
     // one half sweep; with_dot (finest level only) also forms r.z and beta
     template <int DIM>
     static void smooth_level(Instance &I, int l, int colour, M *x, const M *b, bool with_dot = false) {
@@ -413,8 +422,9 @@ template <typename T> struct Impl {
             I.nrz = LD.nblocks;
         } else
             for (int rep = 0; rep < (l == 0 && I.repeat_fine ? 2 : 1); ++rep)   // a repeat is idempotent
-                launchk(k_mg_rbgs<DIM, M, false>, LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x,
-                        b, colour, g, 0, 0, 0, (const M *)nullptr), ++I.nlaunch;
+                launchk(diag_from_rows(L.g) ? k_mg_rbgs<DIM, M, false, sizeof(M) == sizeof(float)> : k_mg_rbgs<DIM, M, false, false>,
+                        LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, colour, g, 0, 0, 0,
+                        (const M *)nullptr), ++I.nlaunch;
     }
     // the first post-smoothing half sweep (colour 1) of level l with the
     // prolongation from level l + 1 (x of level l + 1 in xc) folded in
@@ -423,7 +433,7 @@ template <typename T> struct Impl {
         Level &L = I.lev[l], &C = I.lev[l + 1];
         GridD g = to_dev(L.g), gc = to_dev(C.g);
         L3 LL = launch3((L.g.nx + 1) / 2, L.g.ny, L.g.nz);
-        launchk(k_mg_rbgs<DIM, M, true>, LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, 1, gc,
+        launchk(diag_from_rows(L.g) ? k_mg_rbgs<DIM, M, true, sizeof(M) == sizeof(float)> : k_mg_rbgs<DIM, M, true, false>, LL.grid, LL.block, 0, I.stream, g, mg3(L), (const M *)L.idiag, x, b, 1, gc,
                 L.r[0] >> 1, L.r[1] >> 1, L.r[2] >> 1, xc), ++I.nlaunch;
     }
 

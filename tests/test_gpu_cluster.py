@@ -1,4 +1,4 @@
-"""The thread-block-cluster kernels against the paths they stand in for.
+"""The thread-block-cluster kernels, and other size-dependent forms, against the paths they stand in for.
 
 A pressure solve of a small 2D grid runs in one cluster, and the coarse levels
 of larger grids in another; with cta_global=0 the same levels are worked by
@@ -22,9 +22,9 @@ def built():
     __graft_entry__.build()
 
 
-def _sim(shape, prec, rtol, seed, **sched):
+def _sim(shape, prec, rtol, seed, solid_frac=0.15, **sched):
     nx, ny, nz = shape
-    c = inputs.random_small_case(seed, nx, ny, nz=nz, dim=3 if nz > 1 else 2)
+    c = inputs.random_small_case(seed, nx, ny, nz=nz, dim=3 if nz > 1 else 2, solid_frac=solid_frac)
     p = dict(c.params, precision=prec, cg_rtol=rtol, conv_mode=inputs.CONV_PRES_RESID, conv_tol=0.0)
     g = ox.Oscar(p, c.solid, c.alpha0)
     g.set_schedule(sched)
@@ -73,3 +73,20 @@ def test_coarsest_inverse(shape, prec, most):
     assert g.stats()["cg_iters_total"] <= most * p["n_piso"]
     assert np.isfinite(g.field(ox.FIELD_P)).all()
     g.close()
+
+
+# the smallest ragged grids whose finest half sweeps form the inverse diagonal
+# from the coefficients: a mixed step against the FP64 path, which reads it.
+# alpha as in the other mixed tests; a wrong diagonal would cost iterations
+# (the FP32 trips restart the iteration: at most twice the FP64 path's)
+@pytest.mark.parametrize("shape", [(255, 131, 101), (2051, 1951, 1)])
+def test_diagonal_from_coefficients(shape):
+    alpha, its = [], []
+    for prec in (inputs.PREC_MIXED, inputs.PREC_FP64):
+        g, p, dt_vd, N = _sim(shape, prec, 1e-8, 7, solid_frac=0.02)
+        g.drag_step(dt_vd)
+        alpha.append(g.field(ox.FIELD_ALPHA))
+        its.append(g.stats()["cg_iters_total"])
+        g.close()
+    assert np.abs(alpha[0] - alpha[1]).max() <= 1e-5
+    assert its[0] <= 2 * its[1]
