@@ -170,12 +170,23 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // cluster takes levels of at most vcycle_cells x cta_cells cells (default 8192
 // in FP32: 16 SMs then work about 512 cells each, where a launch per half sweep
 // is still bound by its latency; in FP64 they are bound by FP64 issue above
-// 1024 cells). A 2D grid of at most solve_cells is solved whole in one cluster
-// when its vectors fit the shared memory.
-constexpr int kVcycleCtas = 16, kVcycleThreads = 512;
+// 1024 cells). A 2D grid of at most kSolveCells is solved whole in one cluster
+// when its vectors fit the shared memory: beyond that a solve alone is still
+// shorter in the cluster (512x64 mixed 3.55 against 4.30 ms per five steps, 5.90
+// launched without any cluster), but it holds 16 SMs for work that the launches
+// spread thinner, and instances stepped together wait for each other (ten of
+// 1024x128 to 128x16: 12.4 against 10.2 ms; 64: 392 against 419 M
+// cell-updates/s).
+constexpr int kSolveCells = 16384;
+constexpr int kVcycleThreads = 512;
+// CTAs of the V-cycle's cluster. 16 make a V-cycle 1 to 2 us shorter, but a GPU
+// processing cluster holds only one such cluster, and instances stepped together
+// wait for it: 2D grids, which are stepped in batches, take 8 (1024x128 alone
+// 5.12 -> 5.24 ms; ten instances of 1024x128 to 128x16 10.2 -> 9.2 ms).
+inline int vcycle_ctas(int dim) { return dim == 2 ? 8 : 16; }
 // fewer threads make the block and cluster barriers shorter, more take larger
 // slabs with fewer entries per thread (128x16 FP64: 256 threads 8.03 ms per
-// pass, 512 8.53; 512x64 mixed: 4.25 and 3.64)
+// pass, 512 8.53; 512x64 mixed solved whole: 4.25 and 3.64)
 inline int solve_threads(int ncell) { return ncell <= 8192 ? 256 : 512; }
 // CTAs of the cluster: fewer exchange less, more have shorter slabs. FP32 at
 // 128x16 (six sub-steps): 8 CTAs 2.48 ms, 16 2.55; at 211x26 3.92 and 3.56.
@@ -183,10 +194,10 @@ inline int solve_threads(int ncell) { return ncell <= 8192 ? 256 : 512; }
 template <typename T> inline int solve_ctas(int ncell) { return sizeof(T) == sizeof(float) && ncell <= 2048 ? 8 : 16; }
 template <typename T> struct ClRule;
 template <> struct ClRule<float> {
-    static constexpr long long vcycle_cells = 8, solve_cells = 65536;
+    static constexpr long long vcycle_cells = 8;
 };
 template <> struct ClRule<double> {
-    static constexpr long long vcycle_cells = 1, solve_cells = 16384;
+    static constexpr long long vcycle_cells = 1;
 };
 
 template <typename T> struct Impl {
@@ -876,7 +887,7 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
-    const int nc = I.cta_global ? kVcycleCtas : 1;
+    const int nc = I.cta_global ? vcycle_ctas(I.g.dim) : 1;
     const int keep = I.lc0;
     auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
     int lc0 = I.nlev - 1;
@@ -895,7 +906,7 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     I.cl_smem = Impl<T>::cl_fill(I, P, lg, nc);
     I.cl_nc = P.nc;
     I.solve_nc = 0;
-    if (I.cta_global && I.g.dim == 2 && I.g.ncell <= ClRule<T>::solve_cells) {
+    if (I.cta_global && I.g.dim == 2 && I.g.ncell <= kSolveCells) {
         ClSolve A;
         I.solve_smem = Impl<T>::cl_fill(I, P, 0, solve_ctas<T>(I.g.ncell), &A);
         if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) I.solve_nc = P.nc;   // even slab starts

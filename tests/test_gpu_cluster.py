@@ -34,10 +34,10 @@ def _sim(shape, prec, rtol, seed, solid_frac=0.15, **sched):
 
 # one, two and three slab columns per CTA, ragged slabs, the line between 8 and
 # 16 CTAs (2048 cells) and between 256 and 512 threads (8192), the largest grid
-# (65536 mixed, 16384 FP64) and the first beyond it; in 3D every coarsening
-# ratio and slabs that end inside the grid
+# solved whole (16384) and the first beyond it, larger grids' levels in 8 CTAs;
+# in 3D every coarsening ratio and slabs that end inside the grid
 SHAPES = [(16, 8, 1), (37, 19, 1), (64, 32, 1), (129, 16, 1), (65, 33, 1), (256, 32, 1), (241, 35, 1), (257, 63, 1),
-          (512, 128, 1), (513, 128, 1), (33, 9, 21), (48, 40, 7), (50, 27, 26), (70, 12, 12)]
+          (256, 64, 1), (257, 64, 1), (512, 128, 1), (513, 128, 1), (33, 9, 21), (48, 40, 7), (50, 27, 26), (70, 12, 12)]
 
 
 @pytest.mark.parametrize("prec", [inputs.PREC_MIXED, inputs.PREC_FP64])
