@@ -191,7 +191,7 @@ static void carve(Instance &I, Carver &C) {
     }
     I.stage_dev = (double *)C.take(I.stage_len * sizeof(double));
     I.cl_inv = C.take(kClInvBytes);
-    I.cl_image = C.take(kClImageBytes);
+    I.cl_image = C.take(cl_image_bytes(I.g));
     I.partials = (double *)C.take((size_t)kRedSlots * I.red_stride * sizeof(double));
     I.scal = (double *)C.take(S_COUNT * sizeof(double));
     I.ctl = (int *)C.take(C_COUNT * sizeof(int));
@@ -356,7 +356,7 @@ int oscar_create(const oscar_params *p, const uint8_t *solid, const double *alph
     if (nf == 0) { delete H; return OSCAR_E_INVALID_ARG; }
     build_hierarchy(I);
     I.red_stride = reduction_stride(I.g);
-    I.lc0 = I.nlev - 1;   // refined by the solver set-up (shared-memory budget of the coarse CTA)
+    I.lc0 = I.nlev - 1;   // refined by the solver set-up (shared-memory budget of the cluster's CTAs)
     size_t stage = I.g.ncell;
     for (int a = 0; a < 3; ++a) if ((size_t)I.g.nf[a] > stage) stage = I.g.nf[a];
     I.stage_len = stage;

@@ -233,9 +233,10 @@ __device__ __forceinline__ void cl_load(const ClLevels<M> &P, unsigned char *sm,
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // b + the sum of the neighbour terms of one row. FP32: one term after the
-// other (the order of mg_row_off), or the two of a direction first on the
-// smallest levels, as the per-level kernels and the former coarse kernel
-// formed them. FP64 is bound by FP64 issue: fused multiply-adds.
+// other (the order of mg_row_sum), or the two of a direction first on the
+// levels of at most cta_cells cells (paired): FP32 rounding in the V-cycle is
+// amplified in the smoothest pressure mode, so a level's order is the same
+// whichever cluster works it. FP64 is bound by FP64 issue: fused multiply-adds.
 template <int DIM>
 __device__ __forceinline__ float cl_row_sum(const float *w, const float *x, int c, int ps, int ny, bool paired, float b) {
     const float a0 = w[0] * x[c - ps], a1 = w[1] * x[c + ps];

@@ -881,27 +881,33 @@ template <typename T> void Solver<T>::release_graphs(Instance &I) {
 
 // The cluster takes the levels of at most `cap` cells whose subtree fits its
 // shared memory; with cta_global it has several CTAs and takes the levels of
-// at most kVcycleCells * cap cells (never the finest one, whose x and b are the
+// at most vcycle_cells * cap cells (never the finest one, whose x and b are the
 // Krylov vectors), and a small 2D grid's whole solve runs in one cluster.
 template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
-    const int nc = I.cta_global ? vcycle_ctas(I.g.dim) : 1;
+    int nc = I.cta_global ? vcycle_ctas(I.g.dim) : 1;
     const int keep = I.lc0;
     auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
-    int lc0 = I.nlev - 1;
-    for (;;) {   // the layout depends on which levels take mg_nu_cta sweeps
-        I.lc0 = lc0;
-        if (!fits(lc0)) break;
-        if (lc0 == 0 || I.lev[lc0 - 1].g.ncell > cap) { --lc0; break; }
-        --lc0;
+    auto stored = [&]() { return (size_t)P.img * P.nc <= cl_image_bytes(I.g); };
+    int lc0;
+    for (;; nc /= 2) {   // fewer CTAs when the images of more have no room (never below 4)
+        lc0 = I.nlev - 1;
+        for (;;) {   // the layout depends on which levels take mg_nu_cta sweeps
+            I.lc0 = lc0;
+            if (!fits(lc0)) break;
+            if (lc0 == 0 || I.lev[lc0 - 1].g.ncell > cap) { --lc0; break; }
+            --lc0;
+        }
+        I.lc0 = ++lc0;   // the last one that fitted
+        if (lc0 == I.nlev) { I.lc0 = keep; return OSCAR_E_INVALID_ARG; }
+        Impl<T>::cl_fill(I, P, lc0, nc);
+        if (stored() || nc == 1) break;
     }
-    I.lc0 = ++lc0;   // the last one that fitted
-    if (lc0 == I.nlev) { I.lc0 = keep; return OSCAR_E_INVALID_ARG; }
     int lg = lc0;
     if (I.cta_global)
-        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1)) --lg;
+        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1) && stored()) --lg;
     I.lg = lg < lc0 ? lg : -1;
     I.cl_smem = Impl<T>::cl_fill(I, P, lg, nc);
     I.cl_nc = P.nc;
