@@ -168,9 +168,8 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 
 // Which levels and grids go to a cluster, and of how many CTAs. The V-cycle's
 // cluster takes levels of at most vcycle_cells x cta_cells cells (default 8192
-// in FP32: 16 SMs then work about 512 cells each, where a launch per half sweep
-// is still bound by its latency; in FP64 they are bound by FP64 issue above
-// 1024 cells). A 2D grid of at most kSolveCells is solved whole in one cluster
+// in FP32, where a launch per half sweep is still bound by its latency; in FP64
+// the cluster is bound by FP64 issue above 1024 cells). A 2D grid of at most kSolveCells is solved whole in one cluster
 // when its vectors fit the shared memory: beyond that a solve alone is still
 // shorter in the cluster (512x64 mixed 3.55 against 4.30 ms per five steps, 5.90
 // launched without any cluster), but it holds 16 SMs for work that the launches
@@ -179,11 +178,14 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // cell-updates/s).
 constexpr int kSolveCells = 16384;
 constexpr int kVcycleThreads = 512;
-// CTAs of the V-cycle's cluster. 16 make a V-cycle 1 to 2 us shorter, but a GPU
-// processing cluster holds only one such cluster, and instances stepped together
-// wait for it: 2D grids, which are stepped in batches, take 8 (1024x128 alone
-// 5.12 -> 5.24 ms; ten instances of 1024x128 to 128x16 10.2 -> 9.2 ms).
-inline int vcycle_ctas(int dim) { return dim == 2 ? 8 : 16; }
+// CTAs of the V-cycle's cluster: at most 8. 16 make a V-cycle 1 to 2 us
+// shorter, but all CTAs of a cluster need their SMs at the same time within one
+// GPU processing cluster, and instances stepped together wait for it. One alone
+// with 16 and 8: 1024x128 5.12 and 5.24 ms, 97x51x45 13.8 and 14.0, 256x64x64
+// 21.7 and 21.8; together: ten of 1024x128 to 128x16 10.2 and 9.2 ms, 24 of
+// 128x32x32 66.8 and 63.0 (before there were clusters 63.3), a mix of 36 in 2D
+// and 3D 88.9 and 83.2 (83.3).
+constexpr int kVcycleCtas = 8;
 // fewer threads make the block and cluster barriers shorter, more take larger
 // slabs with fewer entries per thread (128x16 FP64: 256 threads 8.03 ms per
 // pass, 512 8.53; 512x64 mixed solved whole: 4.25 and 3.64)
@@ -887,7 +889,7 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
-    int nc = I.cta_global ? vcycle_ctas(I.g.dim) : 1;
+    int nc = I.cta_global ? kVcycleCtas : 1;
     const int keep = I.lc0;
     auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
     auto stored = [&]() { return (size_t)P.img * P.nc <= cl_image_bytes(I.g); };

@@ -90,3 +90,24 @@ def test_diagonal_from_coefficients(shape):
         g.close()
     assert np.abs(alpha[0] - alpha[1]).max() <= 1e-5
     assert its[0] <= 2 * its[1]
+
+
+def _clusters(g, dt_vd):
+    """CTAs of every cluster kernel that a drag step launches, by kernel name."""
+    g.profile(True)
+    g.drag_step(dt_vd)
+    g.profile(False)
+    rows = [(name.split("<")[0].split(" ")[-1].split("::")[-1], grid) for name, grid, _, _ in g.profile_read()]
+    return {name: grid for name, grid in rows if "_cluster" in name}
+
+
+# the V-cycle's cluster: as many CTAs as the coarsest level has columns, at most
+# 8 (instances stepped together wait for wider ones)
+@pytest.mark.parametrize("shape,ctas", [((512, 128, 1), 8), ((256, 32, 32), 8), ((64, 64, 64), 4), ((24, 40, 40), 2)])
+@pytest.mark.parametrize("prec", [inputs.PREC_MIXED, inputs.PREC_FP64])
+def test_vcycle_cluster_width(shape, ctas, prec):
+    g, p, dt_vd, N = _sim(shape, prec, 1e-8, 11, solid_frac=0.05)
+    assert _clusters(g, dt_vd) == {"k_mg_cluster": ctas}
+    g.set_schedule(dict(cta_global=0))
+    assert _clusters(g, dt_vd) == {"k_mg_cluster": 1}
+    g.close()
