@@ -169,12 +169,13 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // Which levels and grids go to a cluster, and of how many CTAs. The V-cycle's
 // cluster takes levels of at most vcycle_cells x cta_cells cells (default 8192
 // in FP32, where a launch per half sweep is still bound by its latency; in FP64
-// the cluster is bound by FP64 issue above 1024 cells). A 2D grid of at most kSolveCells is solved whole in one cluster
-// when its vectors fit the shared memory: beyond that a solve alone is still
-// shorter in the cluster (512x64 mixed 3.55 against 4.30 ms per five steps, 5.90
-// launched without any cluster), but it holds 16 SMs for work that the launches
-// spread thinner, and instances stepped together wait for each other (ten of
-// 1024x128 to 128x16: 12.4 against 10.2 ms; 64: 392 against 419 M
+// the cluster is bound by FP64 issue above 1024 cells), of which a CTA works at
+// most kVcycleRows. A 2D grid of at most kSolveCells is solved whole in one
+// cluster when its vectors fit the shared memory: beyond that a solve alone is
+// still shorter in the cluster (512x64 mixed 3.55 against 4.30 ms per five steps,
+// 5.90 launched without any cluster), but it holds 16 SMs for work that the
+// launches spread thinner, and instances stepped together wait for each other
+// (ten of 1024x128 to 128x16: 12.4 against 10.2 ms; 64: 392 against 419 M
 // cell-updates/s).
 constexpr int kSolveCells = 16384;
 constexpr int kVcycleThreads = 512;
@@ -186,6 +187,16 @@ constexpr int kVcycleThreads = 512;
 // 128x32x32 66.8 and 63.0 (before there were clusters 63.3), a mix of 36 in 2D
 // and 3D 88.9 and 83.2 (83.3).
 constexpr int kVcycleCtas = 8;
+// Rows of the cluster's largest level that one CTA works, ghosts included: two
+// of each colour per thread. The CTAs are bounded by the columns of the
+// coarsest level, so on grids that are not long in x the level is worked by few
+// of them, or by each of them almost whole, and the launches are shorter. us per
+// PCG iteration with the level in the cluster and without: 4096 rows 16x1024
+// 55.1 and 51.1, 64x64x64 75.6 and 72.5, 32x32x32 53.2 and 50.4; 2000 to 3000
+// 120x48x48 76.3 and 74.9, 48x96x96 122.6 and 120.3, but 128x96x96 134.8 and
+// 135.9, 100x600 57.7 and 58.1; 2048 64x128x128 130.9 and 129.8, 64x512 55.1 and
+// 57.8; fewer 256x64x64 162.0 and 162.9, 1024x128 65.3 and 68.4.
+constexpr int kVcycleRows = 4 * kVcycleThreads;
 // fewer threads make the block and cluster barriers shorter, more take larger
 // slabs with fewer entries per thread (128x16 FP64: 256 threads 8.03 ms per
 // pass, 512 8.53; 512x64 mixed solved whole: 4.25 and 3.64)
@@ -407,6 +418,12 @@ template <typename T> struct Impl {
             A->oe = sizeof(M) == sizeof(float) ? take(n * sizeof(M)) : A->oap;
         }
         return off;
+    }
+
+    // rows of the first level that a CTA with the widest slab works
+    static long long cl_rows(const ClLevels<M> &P) {
+        const ClLevel<M> &L = P.L[0];
+        return (long long)std::min(L.nx, L.ncol - 2 * L.G + 2 * std::min(L.D, L.nx)) * L.ny * L.nz;
     }
 
     // x / b of level l (level 0 works in place on the Krylov vectors z / r)
@@ -883,8 +900,8 @@ template <typename T> void Solver<T>::release_graphs(Instance &I) {
 
 // The cluster takes the levels of at most `cap` cells whose subtree fits its
 // shared memory; with cta_global it has several CTAs and takes the levels of
-// at most vcycle_cells * cap cells (never the finest one, whose x and b are the
-// Krylov vectors), and a small 2D grid's whole solve runs in one cluster.
+// at most vcycle_cells * cap cells and kVcycleRows per CTA (never the finest one,
+// whose x and b are the Krylov vectors), and a small 2D grid's whole solve runs in one cluster.
 template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
@@ -909,7 +926,9 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     }
     int lg = lc0;
     if (I.cta_global)
-        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1) && stored()) --lg;
+        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1) && stored() &&
+               Impl<T>::cl_rows(P) <= kVcycleRows)
+            --lg;
     I.lg = lg < lc0 ? lg : -1;
     I.cl_smem = Impl<T>::cl_fill(I, P, lg, nc);
     I.cl_nc = P.nc;

@@ -111,3 +111,13 @@ def test_vcycle_cluster_width(shape, ctas, prec):
     g.set_schedule(dict(cta_global=0))
     assert _clusters(g, dt_vd) == {"k_mg_cluster": 1}
     g.close()
+
+
+# the levels above 1024 cells that the cluster takes: those of which a CTA works
+# at most 2048 rows (levels counted from the finest, 0; -1: none)
+@pytest.mark.parametrize("shape,level", [((512, 128, 1), 2), ((256, 32, 32), 2), ((64, 512, 1), 2), ((16, 1024, 1), -1),
+                                         ((64, 64, 64), -1), ((32, 32, 32), -1)])
+def test_vcycle_cluster_levels(shape, level):
+    g, p, dt_vd, N = _sim(shape, inputs.PREC_MIXED, 1e-8, 11, solid_frac=0.05)
+    assert g.stats()["mg_cta_global_level"] == level
+    g.close()
