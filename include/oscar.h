@@ -154,8 +154,9 @@ int oscar_standard_step(oscar_handle h, double dt);
 
 /* Device memory (bytes) that oscar_create would allocate for these parameters,
  * from the same layout computation and without allocating anything (for
- * admission control by memory footprint). Errors as oscar_create's parameter
- * validation. Not part of the paper's method. */
+ * admission control by memory footprint). A schedule other than the default one
+ * may add up to 2 MB (oscar_set_schedule). Errors as oscar_create's
+ * parameter validation. Not part of the paper's method. */
 int oscar_footprint(const oscar_params *p, size_t *bytes_out);
 
 /* Asynchronous forms of the three steps: each validates its arguments, launches
@@ -223,7 +224,9 @@ int oscar_get_schedule(oscar_handle h, oscar_schedule *out);
 /* Replace the schedule (waits for the stream; the step graphs are rebuilt at
  * the next step call). OSCAR_E_INVALID_ARG for a value out of range, while an
  * asynchronous step is pending, or when the coarse levels chosen by cta_cells
- * do not fit the cluster's shared memory; the schedule is then unchanged. */
+ * do not fit the cluster's shared memory; OSCAR_E_OOM when the images of the
+ * cluster's CTAs need more device memory than before and there is none. The
+ * schedule is then unchanged. */
 int oscar_set_schedule(oscar_handle h, const oscar_schedule *s);
 
 /* Release all device memory of the instance. */

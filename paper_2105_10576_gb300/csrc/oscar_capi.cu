@@ -191,7 +191,7 @@ static void carve(Instance &I, Carver &C) {
     }
     I.stage_dev = (double *)C.take(I.stage_len * sizeof(double));
     I.cl_inv = C.take(kClInvBytes);
-    I.cl_image = C.take(cl_image_bytes(I.g));
+    I.cl_image = C.take(I.cl_image_cap);
     I.partials = (double *)C.take((size_t)kRedSlots * I.red_stride * sizeof(double));
     I.scal = (double *)C.take(S_COUNT * sizeof(double));
     I.ctl = (int *)C.take(C_COUNT * sizeof(int));
@@ -281,12 +281,29 @@ const char *oscar_strerror(int code) {
     }
 }
 
-// grid, multigrid hierarchy and arena layout of an instance (no allocation)
+static int choose_cta(Instance &I, int cells) {
+    return I.prec == OSCAR_FP64 ? Solver<double>::choose_cta(I, cells) : Solver<float>::choose_cta(I, cells);
+}
+
+// grid, multigrid hierarchy, default schedule and arena layout of an instance
+// (no allocation)
 static void plan(Instance &I, const oscar_params *p) {
     I.P = *p;
     I.prec = p->precision;
     I.g = make_grid(p->dim, p->nx, p->ny, p->nz, p->hx, p->hy, p->hz);
+    I.mg_nu = 2;
+    I.mg_nu_c = 2;
+    I.mg_coarse_sweeps = 4;
+    I.mg_nu_cta = 2;
+    I.coarse_refresh = 8;
+    I.cta_cells = 1024;
+    I.block_x = 0;
+    I.cta_global = 1;
+    I.lg = -1;
     build_hierarchy(I);
+    I.lc0 = I.nlev - 1;
+    choose_cta(I, I.cta_cells);   // for the size of the images; the solver set-up reports what it returns
+    I.cl_image_cap = I.cl_image_need;
     I.red_stride = reduction_stride(I.g);
     size_t stage = I.g.ncell;
     for (int a = 0; a < 3; ++a) if ((size_t)I.g.nf[a] > stage) stage = I.g.nf[a];
@@ -294,6 +311,22 @@ static void plan(Instance &I, const oscar_params *p) {
     Carver dry{nullptr, 0, true};
     carve(I, dry);
     I.arena_bytes = dry.off + 256;
+}
+
+// Room for the images of the present schedule: kept when there is enough, else
+// allocated. The step graphs hold the address: the caller releases them, with
+// the stream idle.
+static int reserve_images(Instance &I) {
+    if (I.cl_image_need <= I.cl_image_cap) return 0;
+    void *p = nullptr;
+    if (cudaMalloc(&p, I.cl_image_need) != cudaSuccess) {
+        cudaGetLastError();
+        return OSCAR_E_OOM;
+    }
+    if (I.cl_image_own) cudaFree(I.cl_image_own);
+    I.cl_image = I.cl_image_own = p;
+    I.cl_image_cap = I.cl_image_need;
+    return 0;
 }
 
 int oscar_footprint(const oscar_params *p, size_t *bytes_out) {
@@ -320,8 +353,6 @@ int oscar_create(const oscar_params *p, const uint8_t *solid, const double *alph
     if (!H) return OSCAR_E_OOM;
     Instance &I = H->I;
     memset(&I, 0, sizeof(Instance));
-    I.P = *p;
-    I.prec = p->precision;
     I.stream = (cudaStream_t)stream;
     if (!I.stream) {   // graphs cannot be captured on the legacy default stream: use a private one
         if (cudaStreamCreateWithFlags(&I.stream, cudaStreamNonBlocking) != cudaSuccess) {
@@ -335,34 +366,17 @@ int oscar_create(const oscar_params *p, const uint8_t *solid, const double *alph
         const char *e = getenv("OSCAR_EAGER");
         I.eager = (e && e[0] == '1') ? 1 : 0;
     }
-    I.g = make_grid(p->dim, p->nx, p->ny, p->nz, p->hx, p->hy, p->hz);
+    plan(I, p);
     I.cos_theta = cos(p->theta_deg * M_PI / 180.0);
     I.deltaN = 1e-8 / pow(I.g.V, 1.0 / p->dim);
     I.last_N = 1;
     I.pending = -1;
-    I.mg_nu = 2;
-    I.mg_nu_c = 2;
-    I.mg_coarse_sweeps = 4;
-    I.mg_nu_cta = 2;
-    I.coarse_refresh = 8;
-    I.cta_cells = 1024;
-    I.block_x = 0;
-    I.cta_global = 1;
     I.repeat_fine = 0;
-    I.lg = -1;
     long long nf = 0;
     for (int c = 0; c < I.g.ncell; ++c) nf += solid[c] == 0;
     I.n_fluid = nf;
     if (nf == 0) { delete H; return OSCAR_E_INVALID_ARG; }
-    build_hierarchy(I);
-    I.red_stride = reduction_stride(I.g);
-    I.lc0 = I.nlev - 1;   // refined by the solver set-up (shared-memory budget of the cluster's CTAs)
-    size_t stage = I.g.ncell;
-    for (int a = 0; a < 3; ++a) if ((size_t)I.g.nf[a] > stage) stage = I.g.nf[a];
-    I.stage_len = stage;
-    Carver dry{nullptr, 0, true};
-    carve(I, dry);
-    I.arena_bytes = dry.off + 256;
+    const size_t stage = I.stage_len;
     if (cudaMalloc(&I.arena, I.arena_bytes) != cudaSuccess) {
         cudaGetLastError();
         delete H;
@@ -410,6 +424,7 @@ int oscar_destroy(oscar_handle h) {
         if (I.prec == OSCAR_FP64) Solver<double>::release_graphs(I);
         else Solver<float>::release_graphs(I);
         cudaFree(I.arena);
+        if (I.cl_image_own) cudaFree(I.cl_image_own);
     }
     for (int q = 0; q < 4; ++q)
         if (I.side[q]) cudaStreamDestroy(I.side[q]);
@@ -577,10 +592,10 @@ int oscar_set_schedule(oscar_handle h, const oscar_schedule *s) {
         I.coarse_refresh = v.coarse_refresh;
         I.block_x = v.block_x;
         I.cta_global = v.cta_global;
-        return I.prec == OSCAR_FP64 ? Solver<double>::choose_cta(I, v.cta_cells)
-                                    : Solver<float>::choose_cta(I, v.cta_cells);
+        return choose_cta(I, v.cta_cells);
     };
     rc = apply(*s);
+    if (!rc) rc = reserve_images(I);
     if (rc) {
         apply(old);
         return rc;
@@ -607,7 +622,7 @@ int oscar_stats(oscar_handle h, oscar_stats_t *out) {
     out->phase_volume = vol;
     out->n_fluid = I.n_fluid;
     out->cell_updates = I.cell_updates;
-    out->device_bytes = I.arena_bytes;
+    out->device_bytes = I.arena_bytes + (I.cl_image_own ? I.cl_image_cap : 0);
     out->kernel_launches = I.nexec;
     out->mg_first_cta_level = I.lc0;
     out->mg_cta_global_level = I.lg;

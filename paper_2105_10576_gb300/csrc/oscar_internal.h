@@ -14,7 +14,6 @@ constexpr int kMaxLevels = 24;
 constexpr int kRedBlocks = 1216;      // 152 SMs x 8: fixed grid of every reduction (deterministic order)
 constexpr int kRedSlots = 16;         // partial-sum slots
 constexpr double kSyncTimeoutSec = 600.0;
-constexpr size_t kClImageCta = 220 * 1024;   // image of one CTA of a cluster: at most its shared memory
 constexpr size_t kClInvBytes = 128 * 128 * sizeof(double);   // explicit inverse of a level of at most 128 cells
 
 // Scalar slots in the device scalar array (double).
@@ -41,10 +40,6 @@ struct GridH {
     int nf[3];
     double h[3], S[3], V;
 };
-
-// the images of a cluster's CTAs (16, or those of 4 on a small 3D grid, whose
-// other arrays would take less than the images of 16)
-inline size_t cl_image_bytes(const GridH &g) { return (g.dim == 3 && g.ncell < 32768 ? 4 : 16) * kClImageCta; }
 
 struct Level {
     GridH g;
@@ -136,7 +131,10 @@ struct Instance {
     int solve_nc;          // CTAs of the whole-solve cluster, 0 when solves run as launches
     size_t solve_smem;
     void *cl_inv;          // explicit inverse of the coarsest level (kClInvBytes)
-    void *cl_image;        // shared-memory images of the cluster's CTAs (cl_image_bytes)
+    void *cl_image;        // shared-memory images of the cluster's CTAs
+    size_t cl_image_need;  // bytes of the images of the present schedule
+    size_t cl_image_cap;   // bytes at cl_image: the default schedule's (part of the arena), or what a schedule needed since
+    void *cl_image_own;    // cl_image where it is not part of the arena
     cudaStream_t aux;      // branch of the operator set-up
     cudaEvent_t ev_fork, ev_join;
     int pending;           // kind (0 drag, 1 relax, 2 standard) of a launched step not yet waited for, or -1

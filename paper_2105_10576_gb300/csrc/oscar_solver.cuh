@@ -906,37 +906,35 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
-    int nc = I.cta_global ? kVcycleCtas : 1;
+    const int nc = I.cta_global ? kVcycleCtas : 1;
     const int keep = I.lc0;
     auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
-    auto stored = [&]() { return (size_t)P.img * P.nc <= cl_image_bytes(I.g); };
-    int lc0;
-    for (;; nc /= 2) {   // fewer CTAs when the images of more have no room (never below 4)
-        lc0 = I.nlev - 1;
-        for (;;) {   // the layout depends on which levels take mg_nu_cta sweeps
-            I.lc0 = lc0;
-            if (!fits(lc0)) break;
-            if (lc0 == 0 || I.lev[lc0 - 1].g.ncell > cap) { --lc0; break; }
-            --lc0;
-        }
-        I.lc0 = ++lc0;   // the last one that fitted
-        if (lc0 == I.nlev) { I.lc0 = keep; return OSCAR_E_INVALID_ARG; }
-        Impl<T>::cl_fill(I, P, lc0, nc);
-        if (stored() || nc == 1) break;
+    int lc0 = I.nlev - 1;
+    for (;;) {   // the layout depends on which levels take mg_nu_cta sweeps
+        I.lc0 = lc0;
+        if (!fits(lc0)) break;
+        if (lc0 == 0 || I.lev[lc0 - 1].g.ncell > cap) { --lc0; break; }
+        --lc0;
     }
+    I.lc0 = ++lc0;   // the last one that fitted
+    if (lc0 == I.nlev) { I.lc0 = keep; return OSCAR_E_INVALID_ARG; }
     int lg = lc0;
     if (I.cta_global)
-        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1) && stored() &&
+        while (lg - 1 >= 1 && I.lev[lg - 1].g.ncell <= ClRule<T>::vcycle_cells * cap && fits(lg - 1) &&
                Impl<T>::cl_rows(P) <= kVcycleRows)
             --lg;
     I.lg = lg < lc0 ? lg : -1;
     I.cl_smem = Impl<T>::cl_fill(I, P, lg, nc);
     I.cl_nc = P.nc;
+    I.cl_image_need = (size_t)P.img * P.nc;
     I.solve_nc = 0;
     if (I.cta_global && I.g.dim == 2 && I.g.ncell <= kSolveCells) {
         ClSolve A;
         I.solve_smem = Impl<T>::cl_fill(I, P, 0, solve_ctas<T>(I.g.ncell), &A);
-        if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) I.solve_nc = P.nc;   // even slab starts
+        if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) {   // even slab starts
+            I.solve_nc = P.nc;
+            I.cl_image_need = (size_t)P.img * P.nc;
+        }
     }
     return 0;
 }

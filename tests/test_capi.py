@@ -92,3 +92,13 @@ def test_footprint_is_host_only_and_scales(lib):
     assert 7 * mixed < big < 9 * mixed
     with pytest.raises(oscar.OscarError):
         oscar.oscar_footprint(dict(c.params, nx=0))
+
+
+def test_footprint_holds_no_more_than_the_images_need(lib):
+    """The images of the coarse levels are sized as they are laid out: a 128x16
+    channel holds its 2048 cells' fields and levels (about 70 values per cell,
+    1.2 MB) and 8 images of less than 40 KB."""
+    c = inputs.channel_bubble_2d()
+    assert oscar.oscar_footprint(dict(c.params, precision=inputs.PREC_MIXED)) < 1.6e6
+    c = inputs.constricted_channel_3d(nx=64, ny=22, nz=22)
+    assert oscar.oscar_footprint(dict(c.params, precision=inputs.PREC_MIXED)) < 12.5e6

@@ -121,3 +121,23 @@ def test_vcycle_cluster_levels(shape, level):
     g, p, dt_vd, N = _sim(shape, inputs.PREC_MIXED, 1e-8, 11, solid_frac=0.05)
     assert g.stats()["mg_cta_global_level"] == level
     g.close()
+
+
+# a schedule whose images need more than the default one's: room is made for
+# them, and the steps are those of the launched path; back to the default
+@pytest.mark.parametrize("shape", [(256, 32, 1), (257, 65, 1), (70, 24, 24)])
+def test_schedule_with_larger_images(shape):
+    wide = dict(mg_nu=4, mg_nu_mid=4, mg_nu_cta=6)
+    out, held = [], []
+    for flag in (1, 0):
+        g, p, dt_vd, N = _sim(shape, inputs.PREC_MIXED, 1e-8, 23, cta_global=flag)
+        assert flag == 0 or g.stats()["device_bytes"] == ox.oscar_footprint(p)
+        for sched in (wide, dict(mg_nu=2, mg_nu_mid=2, mg_nu_cta=2), wide):
+            g.set_schedule(sched)
+            g.drag_step(dt_vd)
+        held.append(g.stats()["device_bytes"] - ox.oscar_footprint(p))
+        out.append([g.field(w) for w in (ox.FIELD_ALPHA, ox.FIELD_P, ox.FIELD_U)])
+        g.close()
+    assert 0 < held[0] < 2.1e6 and held[1] == 0
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
