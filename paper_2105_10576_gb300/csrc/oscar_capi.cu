@@ -300,6 +300,7 @@ static void plan(Instance &I, const oscar_params *p) {
     I.block_x = 0;
     I.cta_global = 1;
     I.lg = -1;
+    I.cl_fit = I.solve_fit = 16;   // the solver set-up asks the device
     build_hierarchy(I);
     I.lc0 = I.nlev - 1;
     choose_cta(I, I.cta_cells);   // for the size of the images; the solver set-up reports what it returns
@@ -410,6 +411,7 @@ int oscar_create(const oscar_params *p, const uint8_t *solid, const double *alph
     cudaMemcpyAsync(sd, solid, (size_t)I.g.ncell, cudaMemcpyHostToDevice, I.stream);
     rc = I.prec == OSCAR_FP64 ? Solver<double>::setup(I, sd, a0d) : Solver<float>::setup(I, sd, a0d);
     int rc2 = sync_bounded(I.stream, kSyncTimeoutSec);
+    if (!rc) rc = reserve_images(I);
     cudaFree(tmp);
     if (rc || rc2) { oscar_destroy(H); return rc ? rc : rc2; }
     *out = H;

@@ -126,6 +126,7 @@ struct Instance {
     int red_stride;        // partials per slot: max(kRedBlocks, blocks of a cell launch)
     int lc0;               // first multigrid level of at most cta_cells cells
     int lg;                // first of the levels above lc0 that the cluster works too, -1 when none
+    int cl_fit, solve_fit; // CTAs of a cluster that the GPU can place, for the V-cycle and for whole solves
     int cl_nc;             // CTAs of the V-cycle's cluster
     size_t cl_smem;        // shared memory of each of them
     int solve_nc;          // CTAs of the whole-solve cluster, 0 when solves run as launches

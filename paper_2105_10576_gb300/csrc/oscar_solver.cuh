@@ -906,7 +906,7 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     ClLevels<T> P;
     const size_t budget = kClSmemBytes;
     if (cap > kCtaCells) cap = kCtaCells;
-    const int nc = I.cta_global ? kVcycleCtas : 1;
+    const int nc = I.cta_global ? std::min(kVcycleCtas, I.cl_fit) : 1;
     const int keep = I.lc0;
     auto fits = [&](int l) { return Impl<T>::cl_fill(I, P, l, nc) <= budget; };
     int lc0 = I.nlev - 1;
@@ -930,13 +930,37 @@ template <typename T> int Solver<T>::choose_cta(Instance &I, long long cap) {
     I.solve_nc = 0;
     if (I.cta_global && I.g.dim == 2 && I.g.ncell <= kSolveCells) {
         ClSolve A;
-        I.solve_smem = Impl<T>::cl_fill(I, P, 0, solve_ctas<T>(I.g.ncell), &A);
+        I.solve_smem = Impl<T>::cl_fill(I, P, 0, std::min(solve_ctas<T>(I.g.ncell), I.solve_fit), &A);
         if (I.solve_smem <= budget && (P.nc == 1 || P.L[0].sh > 0)) {   // even slab starts
             I.solve_nc = P.nc;
             I.cl_image_need = (size_t)P.img * P.nc;
         }
     }
     return 0;
+}
+
+// The CTAs, at most nc, of a cluster of kernel f that the GPU can place. A GPU
+// processing cluster with fewer SMs left than a cluster needs (16 CTAs of up to
+// 220 KB take 16 SMs; a device with SMs turned off or partitioned) cannot hold
+// it, and its launch would fail.
+inline int cluster_fit(const void *f, int threads, int nc) {
+    for (; nc > 1; nc /= 2) {
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3(nc);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = kClSmemBytes;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)nc;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) == cudaSuccess && n > 0) break;
+        cudaGetLastError();
+    }
+    return nc;
 }
 
 template <typename T> int Solver<T>::setup(Instance &I, const uint8_t *solid_dev, const double *alpha0_dev) {
@@ -954,7 +978,6 @@ template <typename T> int Solver<T>::setup(Instance &I, const uint8_t *solid_dev
                                                                F.fluid, Lv.fluid), ++I.nlaunch;
     }
     OSCAR_LAUNCH_CHECK();
-    OSCAR_TRY(choose_cta(I, I.cta_cells));
     // the attributes belong to the kernels, not to this instance: they are set
     // to the budget (never lowered), so that instances of other sizes, created
     // while this one runs, cannot shrink them below what this one launches with
@@ -966,6 +989,9 @@ template <typename T> int Solver<T>::setup(Instance &I, const uint8_t *solid_dev
             cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return OSCAR_E_CUDA;
     }
+    I.cl_fit = cluster_fit(vcy, kVcycleThreads, kVcycleCtas);
+    I.solve_fit = cluster_fit(sol, 512, kMaxCluster);
+    OSCAR_TRY(choose_cta(I, I.cta_cells));
     int rc = Impl<T>::interface_(I, I.alpha);
     I.nexec += I.nlaunch - l0;
     return rc;

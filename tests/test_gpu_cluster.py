@@ -7,6 +7,11 @@ the same operands, so the fields are bitwise equal. FP64 path: other orders of
 summation; with the solves converged to 1e-13 the fields agree to 1e-9 of
 their largest value.
 """
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -141,3 +146,46 @@ def test_schedule_with_larger_images(shape):
     assert 0 < held[0] < 2.1e6 and held[1] == 0
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+FAKE_OCCUPANCY = r"""
+#include <cuda_runtime.h>
+#include <stdlib.h>
+/* a device on which clusters of more than FAKE_CLUSTER CTAs cannot be placed */
+cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *f, const cudaLaunchConfig_t *cfg) {
+    unsigned nc = 1;
+    for (unsigned q = 0; q < cfg->numAttrs; ++q)
+        if (cfg->attrs[q].id == cudaLaunchAttributeClusterDimension) nc = cfg->attrs[q].val.clusterDim.x;
+    *n = nc <= (unsigned)atoi(getenv("FAKE_CLUSTER"));
+    return cudaSuccess;
+}
+"""
+FAKE_RUN = """
+import json, sys
+sys.path.insert(0, "."); sys.path.insert(0, "tests")
+import test_gpu_cluster as t
+g, p, dt_vd, N = t._sim(tuple(json.loads(sys.argv[1])), t.inputs.PREC_MIXED, 1e-8, 29)
+print("CTAS", json.dumps(t._clusters(g, dt_vd)), float(abs(g.field(t.ox.FIELD_P)).sum()).hex())
+"""
+
+
+# where the GPU cannot place a cluster, the next smaller one is taken (the query
+# is faked: a preloaded library answers it), with the same mixed fields
+@pytest.mark.parametrize("shape,kernel,ctas", [((256, 32, 1), "k_solve_cluster", 16), ((512, 128, 1), "k_mg_cluster", 8)])
+def test_clusters_that_cannot_be_placed(tmp_path, shape, kernel, ctas):
+    from paper_2105_10576_gb300 import build
+    src, lib = tmp_path / "fake.c", tmp_path / "fake.so"
+    src.write_text(FAKE_OCCUPANCY)
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-I" + inc, "-o", str(lib), str(src)], check=True)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    seen = []
+    for most in (16, ctas // 2, 1):
+        r = subprocess.run([sys.executable, "-c", FAKE_RUN, json.dumps(shape)], cwd=root, capture_output=True, text=True,
+                           env=dict(os.environ, LD_PRELOAD=str(lib), FAKE_CLUSTER=str(most)), timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        _, rest = r.stdout.split("CTAS ", 1)
+        seen.append((json.loads(rest[:rest.index("}") + 1]), rest.split()[-1]))
+    assert seen[0][0] == {kernel: ctas} and list(seen[1][0].values()) == [ctas // 2]
+    assert list(seen[2][0].values()) == [1]
+    assert seen[0][1] == seen[1][1] == seen[2][1]
