@@ -40,7 +40,7 @@ def _sim(shape, prec, rtol, seed, solid_frac=0.15, **sched):
 # one, two and three slab columns per CTA, ragged slabs, the line between 8 and
 # 16 CTAs (2048 cells) and between 256 and 512 threads (8192), the largest grid
 # solved whole (16384) and the first beyond it, larger grids' levels in 8 CTAs;
-# in 3D every coarsening ratio and slabs that end inside the grid
+# in 3D slabs that end inside the grid (every level coarsens all axes by 2 here)
 SHAPES = [(16, 8, 1), (37, 19, 1), (64, 32, 1), (129, 16, 1), (65, 33, 1), (256, 32, 1), (241, 35, 1), (257, 63, 1),
           (256, 64, 1), (257, 64, 1), (512, 128, 1), (513, 128, 1), (33, 9, 21), (48, 40, 7), (50, 27, 26), (70, 12, 12)]
 
@@ -189,3 +189,59 @@ def test_clusters_that_cannot_be_placed(tmp_path, shape, kernel, ctas):
     assert seen[0][0] == {kernel: ctas} and list(seen[1][0].values()) == [ctas // 2]
     assert list(seen[2][0].values()) == [1]
     assert seen[0][1] == seen[1][1] == seen[2][1]
+
+
+# every coarsening ratio inside the cluster (cells of several aspect ratios),
+# grids taller than wide, one to sixteen CTAs: the kernel and its CTAs on the
+# mixed and on the FP64 path (MG: the V-cycle, SOLVE: the whole solve)
+MG, SOLVE = "k_mg_cluster", "k_solve_cluster"
+LEVELS = [((24, 48, 40), (16, 2, 2), (MG, 8), (MG, 8)),       # (1, 2, 2) above 1024 cells
+          ((24, 48, 40), (32, 2, 2), (MG, 8), (MG, 8)),       # (1, 2, 2) below
+          ((48, 6, 40), (2, 32, 2), (MG, 2), (MG, 2)),        # (2, 1, 2)
+          ((48, 40, 6), (2, 2, 32), (MG, 2), (MG, 2)),        # (2, 2, 1)
+          ((256, 5, 6), (2, 32, 32), (MG, 8), (MG, 8)),       # (2, 1, 1), three in a row on the mixed path
+          ((6, 256, 5), (32, 2, 32), (MG, 2), (MG, 2)),       # (1, 2, 1)
+          ((5, 6, 256), (32, 32, 2), (MG, 2), (MG, 2)),       # (1, 1, 2)
+          ((256, 6, 40), (2, 32, 8), (MG, 8), (MG, 8)),
+          ((64, 128, 1), (32, 2, 2), (SOLVE, 16), (MG, 8)),   # (1, 2)
+          ((128, 64, 1), (2, 32, 2), (MG, 4), (MG, 4)),       # (2, 1)
+          ((19, 120, 1), (2, 1.5, 2), (SOLVE, 2), (MG, 2)), ((40, 200, 1), (2, 1.5, 2), (MG, 4), (MG, 4)),
+          ((16, 300, 1), (2, 1.5, 2), (MG, 2), (MG, 2)), ((12, 60, 1), (2, 1.5, 2), (SOLVE, 2), (SOLVE, 2)),
+          ((3, 90, 1), (2, 1.5, 2), (SOLVE, 2), (SOLVE, 2)), ((1, 100, 1), (2, 1.5, 2), (SOLVE, 1), (SOLVE, 1)),
+          ((9, 33, 21), (2, 1.5, 2), (MG, 2), (MG, 2)), ((12, 40, 40), (2, 1.5, 2), (MG, 2), (MG, 2)),
+          ((256, 32, 32), (2, 1.5, 2), (MG, 8), (MG, 8)), ((256, 32, 1), (2, 1.5, 2), (SOLVE, 16), (SOLVE, 16)),
+          ((129, 16, 1), (2, 1.5, 2), (SOLVE, 16), (SOLVE, 16)), ((240, 80, 9), (2, 2, 16), (MG, 8), (MG, 8))]
+
+
+# Mixed: against one CTA, the same bits and so the same PCG iterations. FP64:
+# against per-level launches down to the level that is solved exactly. The
+# V-cycle is the same but for the order of sums, which changes when a solve
+# stops only where its residual meets the target to rounding: at most once in
+# the nine solves. (A wrong ghost column, transfer or sweep changes every one.)
+@pytest.mark.parametrize("prec", [inputs.PREC_MIXED, inputs.PREC_FP64])
+@pytest.mark.parametrize("shape,h,mixed_kernel,fp64_kernel", LEVELS)
+def test_cluster_vcycle_is_the_launched_one(shape, h, mixed_kernel, fp64_kernel, prec):
+    mixed = prec == inputs.PREC_MIXED
+    nx, ny, nz = shape
+    c = inputs.random_small_case(31 + nx, nx, ny, nz=nz, dim=3 if nz > 1 else 2, solid_frac=0.1,
+                                 hx=h[0] * 1e-6, hy=h[1] * 1e-6, hz=h[2] * 1e-6)
+    p = dict(c.params, precision=prec, cg_rtol=1e-8 if mixed else 1e-10, conv_mode=inputs.CONV_PRES_RESID, conv_tol=0.0)
+    dt_cfl, dt_b, dt_vd, N = ox.oscar_timesteps(p, 0.02)
+    out, its = [], []
+    for sched in (dict(), dict(cta_global=0) if mixed else dict(cta_global=0, cta_cells=128)):
+        g = ox.Oscar(p, c.solid, c.alpha0)
+        g.set_schedule(sched)
+        g.drag_step(dt_vd)
+        g.relax(dt_vd / N, 2)
+        its.append(g.stats()["cg_iters_total"])
+        out.append([g.field(w) for w in (ox.FIELD_ALPHA, ox.FIELD_P, ox.FIELD_U, ox.FIELD_U + 1)])
+        if not sched:
+            kernel, ctas = mixed_kernel if mixed else fp64_kernel
+            assert _clusters(g, dt_vd) == {kernel: ctas}
+        g.close()
+    if mixed:
+        assert its[0] == its[1]
+        for x, y in zip(*out):
+            assert np.array_equal(x, y)
+    else:
+        assert abs(its[0] - its[1]) <= 1
