@@ -655,11 +655,15 @@ template <typename T> struct Impl {
                                                                         tp(cf[2]), tp(I.fst[2]), cf64_out(I, 2)), ++I.nlaunch;
         OSCAR_LAUNCH_CHECK();
         // the multigrid operators are first needed by the solve: they are built
-        // on a branch beside the first momentum prediction
-        if (cudaEventRecord(I.ev_fork, I.stream) != cudaSuccess || cudaStreamWaitEvent(I.aux, I.ev_fork, 0) != cudaSuccess)
+        // on a branch beside the first momentum prediction. A timed step keeps
+        // them on the instance's stream: no kernel is timed beside another, and the
+        // recording waits for that stream only
+        const bool branch = !t_prof;
+        if (branch && (cudaEventRecord(I.ev_fork, I.stream) != cudaSuccess ||
+                       cudaStreamWaitEvent(I.aux, I.ev_fork, 0) != cudaSuccess))
             return OSCAR_E_CUDA;
-        OSCAR_TRY(mg_coeffs_d<DIM>(I, I.aux));
-        if (cudaEventRecord(I.ev_join, I.aux) != cudaSuccess) return OSCAR_E_CUDA;
+        OSCAR_TRY(mg_coeffs_d<DIM>(I, branch ? I.aux : I.stream));
+        if (branch && cudaEventRecord(I.ev_join, I.aux) != cudaSuccess) return OSCAR_E_CUDA;
         P3<T> Gp0 = p3(&I.G[0]), Gp1 = p3(&I.G[3]), Gp2 = p3(&I.G[6]);
         C3<T> Gc0 = c3(&I.G[0]), Gc1 = c3(&I.G[3]), Gc2 = c3(&I.G[6]);
         for (int corr = 0; corr < I.P.n_piso; ++corr) {
@@ -672,7 +676,7 @@ template <typename T> struct Impl {
             // E_k, the normalised initial residual of the first corrector
             // (Section 3.2), is formed by the solve's initial-residual kernel
             if (corr == 0) {
-                if (cudaStreamWaitEvent(I.stream, I.ev_join, 0) != cudaSuccess) return OSCAR_E_CUDA;
+                if (branch && cudaStreamWaitEvent(I.stream, I.ev_join, 0) != cudaSuccess) return OSCAR_E_CUDA;
                 if (!(DIM == 2 && I.solve_nc))   // the one-launch solve sums q itself
                     launchx(false, 1, k_sum_to<double>, kRedBlocks, BS, 0, I.stream, g.ncell, q, 1.0, I.partials,
                             I.ticket, I.scal, S_QSUM), ++I.nlaunch;

@@ -148,6 +148,15 @@ def test_schedule_with_larger_images(shape):
         assert np.array_equal(x, y)
 
 
+def _preload(tmp_path, source):
+    from paper_2105_10576_gb300 import build
+    src, lib = tmp_path / "fake.c", tmp_path / "fake.so"
+    src.write_text(source)
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-I" + inc, "-o", str(lib), str(src), "-ldl"], check=True)
+    return str(lib)
+
+
 FAKE_OCCUPANCY = r"""
 #include <cuda_runtime.h>
 #include <stdlib.h>
@@ -173,16 +182,12 @@ print("CTAS", json.dumps(t._clusters(g, dt_vd)), float(abs(g.field(t.ox.FIELD_P)
 # is faked: a preloaded library answers it), with the same mixed fields
 @pytest.mark.parametrize("shape,kernel,ctas", [((256, 32, 1), "k_solve_cluster", 16), ((512, 128, 1), "k_mg_cluster", 8)])
 def test_clusters_that_cannot_be_placed(tmp_path, shape, kernel, ctas):
-    from paper_2105_10576_gb300 import build
-    src, lib = tmp_path / "fake.c", tmp_path / "fake.so"
-    src.write_text(FAKE_OCCUPANCY)
-    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
-    subprocess.run(["gcc", "-shared", "-fPIC", "-I" + inc, "-o", str(lib), str(src)], check=True)
+    lib = _preload(tmp_path, FAKE_OCCUPANCY)
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     seen = []
     for most in (16, ctas // 2, 1):
         r = subprocess.run([sys.executable, "-c", FAKE_RUN, json.dumps(shape)], cwd=root, capture_output=True, text=True,
-                           env=dict(os.environ, LD_PRELOAD=str(lib), FAKE_CLUSTER=str(most)), timeout=300)
+                           env=dict(os.environ, LD_PRELOAD=lib, FAKE_CLUSTER=str(most)), timeout=300)
         assert r.returncode == 0, r.stderr[-2000:]
         _, rest = r.stdout.split("CTAS ", 1)
         seen.append((json.loads(rest[:rest.index("}") + 1]), rest.split()[-1]))
@@ -245,3 +250,49 @@ def test_cluster_vcycle_is_the_launched_one(shape, h, mixed_kernel, fp64_kernel,
             assert np.array_equal(x, y)
     else:
         assert abs(its[0] - its[1]) <= 1
+
+
+COUNT_STREAMS = r"""
+#include <cuda_runtime.h>
+#include <dlfcn.h>
+#include <stdio.h>
+/* streams on which events are recorded */
+static cudaStream_t seen[64];
+static int n = 0;
+int streams_seen(void) { int m = n; n = 0; return m; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+    int q = 0;
+    while (q < n && seen[q] != s) ++q;
+    if (q == n && n < 64) seen[n++] = s;
+    char so[64];
+    snprintf(so, sizeof(so), "libcudart.so.%d", CUDART_VERSION / 1000);
+    void *f = dlsym(dlopen(so, RTLD_LAZY), "cudaEventRecord");
+    return f ? ((cudaError_t(*)(cudaEvent_t, cudaStream_t))f)(e, s) : cudaErrorUnknown;
+}
+"""
+STREAMS_RUN = """
+import ctypes, os, sys
+sys.path.insert(0, "."); sys.path.insert(0, "tests")
+import test_gpu_cluster as t
+streams = ctypes.CDLL(os.environ["LD_PRELOAD"]).streams_seen
+g, p, dt_vd, N = t._sim((40, 24, 16), t.inputs.PREC_MIXED, 1e-8, 37)
+g.profile(True)
+streams()
+g.drag_step(dt_vd)
+n = streams()
+g.profile(False)
+print("STREAMS", n, len(g.profile_read()))
+"""
+
+
+def test_timed_steps_run_on_one_stream(tmp_path):
+    """In-step timing puts an event pair around every launch; the launches of a
+    timed step run one after the other on the instance's stream, so that no
+    kernel is timed beside another (a graph step builds the multigrid operators
+    on a branch)."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", STREAMS_RUN], cwd=root, capture_output=True, text=True,
+                       env=dict(os.environ, LD_PRELOAD=_preload(tmp_path, COUNT_STREAMS)), timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    n, kinds = map(int, r.stdout.split("STREAMS ", 1)[1].split())
+    assert n == 1 and kinds > 20
