@@ -81,7 +81,9 @@ def grid_counts(c):
 def kernel_bytes(name: str, c, e: int):
     """Algorithmic bytes of one finest-level launch of kernel `name`
     ("k_x<args>"), or None for kernels without a streaming byte model (the
-    kernels that work in one thread-block cluster, set-up and control kernels)."""
+    kernels that work in one thread-block cluster, set-up and control kernels,
+    and k_cg_refine, which moves the vectors only in the launches that end a
+    defect-correction trip)."""
     n, F, R, d = grid_counts(c)
     base = name.split("<")[0]
     if base == "k_mg_rbgs":          # x of every cell, b and 1/diag of one colour, half of x written, each face once
@@ -108,8 +110,6 @@ def kernel_bytes(name: str, c, e: int):
         return n * (6 * e + 4)
     if base == "k_transport_update":
         return n * (5 * e + 4) + 2 * F * e
-    if base == "k_cg_refine":        # e, q, r64 and FP32 images in, q, r64, r, z out, FP32 faces once
-        return n * (e + 8 + 8 + 8 + 2 * e + 4) + F * e
     if base == "k_cg_init":          # q, b, r64 in/out, FP64 face coefficients
         return n * (8 + 8 + 8 + 2 * e + 4) + 8 * F
     if base == "k_correct":          # phi*, c_f, f_st in and phi out per face; q (FP64), info, HbyA, 1/A in, v out
@@ -146,7 +146,7 @@ def recorded_traffic(kernel: str):
              "k_cg_update": "k_cg_update_constriction_3d.md",
              "k_mg_resid_restrict": "k_mg_resid_restrict_constriction_3d.md",
              "k_momentum_H": "k_momentum_H_constriction_3d.md", "k_cg_init": "k_cg_init_constriction_3d.md",
-             "k_cg_refine": "k_cg_refine_constriction_3d.md", "k_correct": "k_correct_constriction_3d.md"}
+             "k_correct": "k_correct_constriction_3d.md"}
     base = kernel.split("<")[0]
     if base not in files:
         return None
