@@ -117,6 +117,15 @@ def kernel_bytes(name: str, c, e: int):
     return None
 
 
+def fine_sweep_name(c, e: int) -> str:
+    """The kernel of the plain finest-level half sweep: k_mg_rbgs<dimension,
+    type, folded prolongation, inverse diagonal formed>, the last where FP32
+    sweeps stream 80 MB or more."""
+    n, _, _, d = grid_counts(c)
+    formed = e == 4 and (d + 3) * n * e >= 80e6
+    return f"k_mg_rbgs<{d}, {'double' if e == 8 else 'float'}, false, {'true' if formed else 'false'}>"
+
+
 def kernel_source_sha1(base: str):
     """SHA-1 of the source text of kernel `base` (from its __global__
     signature to the closing brace of its body) in oscar_kernels.cuh, or None."""
@@ -890,7 +899,7 @@ def main():
         if roofline is not None and args.workload == "constriction_3d":
             ig = in_graph_sweep_time(ox, c, sched, dt_vd, dt_cr, min(nsub, 8), stream)
             if ig is not None:
-                fine = f"k_mg_rbgs<{c.params['dim']}, {'double' if es == 8 else 'float'}, false>"
+                fine = fine_sweep_name(c, es)
                 ab = kernel_bytes(fine, c, es)
                 ig.update({"kernel": fine + " (finest level)", "algorithmic_bytes_per_launch": ab,
                            "achieved": ab / (ig["avg_launch_us"] * 1e-6) / 1e9,
