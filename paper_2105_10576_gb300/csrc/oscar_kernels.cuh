@@ -1591,7 +1591,7 @@ __device__ __forceinline__ void poisson_row_comp(const GridD &g, uint32_t inf, i
 // 1.5 us of the iterations that only check. The values the decision reads are
 // written by the last block to finish at the earliest.
 template <int DIM>
-__global__ void k_cg_refine(GridD g, const uint32_t *__restrict__ info, C3<float> cf, const float *__restrict__ e,
+__global__ void __launch_bounds__(1024) k_cg_refine(GridD g, const uint32_t *__restrict__ info, C3<float> cf, const float *__restrict__ e,
                             double *__restrict__ q, double *__restrict__ r64, float *__restrict__ r,
                             const float *__restrict__ idiag0, float *__restrict__ z, const double *__restrict__ rr_part,
                             int nrr, double *__restrict__ part, int stride, unsigned *__restrict__ ticket, int nb,

@@ -102,3 +102,17 @@ def test_footprint_holds_no_more_than_the_images_need(lib):
     assert oscar.oscar_footprint(dict(c.params, precision=inputs.PREC_MIXED)) < 1.6e6
     c = inputs.constricted_channel_3d(nx=64, ny=22, nz=22)
     assert oscar.oscar_footprint(dict(c.params, precision=inputs.PREC_MIXED)) < 12.5e6
+
+
+def test_kernels_launched_with_1024_threads_are_compiled_for_them():
+    """launch_sms blocks have 1024 threads, 64 registers each: a kernel launched
+    with them declares so (without it one that needs more fails at its launch)."""
+    csrc = os.path.join(ROOT, "paper_2105_10576_gb300", "csrc")
+    kern, solver = (open(os.path.join(csrc, f)).read() for f in ("oscar_kernels.cuh", "oscar_solver.cuh"))
+    names = set()
+    for m in re.finditer(r"(?:const )?L3 (\w+) = launch_sms\(", solver):
+        rest = solver[m.end():]
+        names |= set(re.findall(r"launchk\((\w+)(?:<[^;]*?>)?, " + m.group(1) + r"\.grid", rest[:rest.index("return")]))
+    assert names == {"k_cg_refine"}
+    for name in names:
+        assert re.search(r"__launch_bounds__\(1024\) " + name + r"\(", kern), name
