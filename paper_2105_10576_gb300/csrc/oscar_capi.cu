@@ -293,7 +293,6 @@ static void plan(Instance &I, const oscar_params *p) {
     I.g = make_grid(p->dim, p->nx, p->ny, p->nz, p->hx, p->hy, p->hz);
     I.mg_nu = 2;
     I.mg_nu_c = 2;
-    I.mg_coarse_sweeps = 4;
     I.mg_nu_cta = 2;
     I.coarse_refresh = 8;
     I.cta_cells = 1024;

@@ -18,7 +18,7 @@ constexpr size_t kClInvBytes = 128 * 128 * sizeof(double);   // explicit inverse
 
 // Scalar slots in the device scalar array (double).
 enum Slot {
-    S_BB = 0, S_RR, S_RZ0, S_RZ1, S_PAP, S_QSUM, S_RES, S_NRM, S_DUMAX, S_VOL, S_TARGET, S_E, S_DU, S_TEST,
+    S_BB = 0, S_RR, S_RZ0, S_RZ1, S_QSUM, S_RES, S_NRM, S_DUMAX, S_VOL, S_TARGET, S_E, S_DU, S_TEST,
     S_ITARGET, S_AREA0, S_AREA1, S_COUNT
 };
 
@@ -154,7 +154,7 @@ struct Instance {
     long long cg_iters_total;
     int cg_iters_last;
     long long cell_updates;
-    int mg_nu, mg_nu_c, mg_coarse_sweeps;   // sweeps on the finest level, on coarser levels, on the coarsest
+    int mg_nu, mg_nu_c;    // sweeps on the finest level, on coarser levels
     int mg_nu_cta;         // sweeps on the levels of at most cta_cells cells
     int repeat_fine;       // measurement: finest-level plain half sweeps issued twice (oscar_profile_repeat)
     int coarse_refresh;    // the coarsest level's inverse is formed every this many PISO set-ups

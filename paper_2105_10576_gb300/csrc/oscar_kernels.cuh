@@ -70,12 +70,10 @@ template <typename T> struct GA;
 template <> struct GA<double> {
     __device__ static __forceinline__ double h(const GridD &g, int a) { return g.h[a]; }
     __device__ static __forceinline__ double S(const GridD &g, int a) { return g.S[a]; }
-    __device__ static __forceinline__ double V(const GridD &g) { return g.V; }
 };
 template <> struct GA<float> {
     __device__ static __forceinline__ float h(const GridD &g, int a) { return g.hf[a]; }
     __device__ static __forceinline__ float S(const GridD &g, int a) { return g.Sf[a]; }
-    __device__ static __forceinline__ float V(const GridD &g) { return g.Vf; }
 };
 
 // Divisions by grid constants and the time step. An FP64 division is about ten
@@ -174,20 +172,11 @@ inline L3 launch_sms(const GridH &g) {
 
 #define BLOCK_ID() ((int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)))
 
-// Blocks of launch3's shape over (x, rows) where each thread takes RPT rows,
-// row = blockIdx.y * blockDim.y * RPT + threadIdx.y + u * blockDim.y, u < RPT
+// Blocks of launch3's shape over (x, rows) where each thread takes rpt rows of a
+// group, row = group * blockDim.y * rpt + threadIdx.y + u * blockDim.y, u < rpt
 // (the kernels unroll u so that the loads of all their rows are in flight
-// together)
-inline L3 launch_rpt(const GridH &g, int rpt) {
-    L3 l = launch3(g.nx, g.ny * g.nz, 1);
-    const int by = (int)l.block.y, rows = g.ny * g.nz;
-    l.grid = dim3(l.grid.x, (rows + by * rpt - 1) / (by * rpt), 1);
-    l.nblocks = (int)(l.grid.x * l.grid.y);
-    return l;
-}
-
-// launch_rpt with at most about kDotBlocks blocks: a block takes the row
-// groups blockIdx.y, blockIdx.y + gridDim.y, ... (at most gy of them)
+// together). At most kDotBlocks blocks and one more per column of blocks: a
+// block takes the groups blockIdx.y, blockIdx.y + gridDim.y, ...
 constexpr int kDotBlocks = 608;   // 152 SMs x 4
 struct L3G : L3 { int groups; };
 inline L3G launch_groups(int nx, int rows, int rpt) {
@@ -1093,28 +1082,6 @@ __global__ void k_correct(GridD g, GR<T> gr, const uint32_t *__restrict__ info, 
 // acc + w x: a product and a sum in FP32, fused in FP64 (half the FP64 instructions)
 __device__ __forceinline__ float mg_madd(float w, float x, float acc) { return acc + w * x; }
 __device__ __forceinline__ double mg_madd(double w, double x, double acc) { return fma(w, x, acc); }
-// (M x)_P = sum_f c_f (x_P - x_N) + sum_outlet c_f x_P, evaluated in type V
-template <int DIM, typename T, typename V>
-__device__ __forceinline__ V poisson_row(const GridD &g, uint32_t inf, int c, int i, int j, int k, C3<T> cf,
-                                         const V *__restrict__ x) {
-    V acc = V(0);
-    V xc = x[c];
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        int off = noff(g, a);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            int t = ftype(inf, a, s);
-            if (t == FT_INTERIOR) {
-                int f = s ? fhi(g, a, i, j, k) : flo(g, a, i, j, k);
-                acc = mg_madd((V)cf.a[a][f], xc - x[s ? c + off : c - off], acc);
-            } else if (t == FT_OUTLET) {
-                acc = mg_madd((V)cf.a[a][fhi(g, a, i, j, k)], xc, acc);
-            }
-        }
-    }
-    return acc;
-}
 
 // The FP64 operator row, sum over the faces of w_f (q_c - q_nb) (interior)
 // and w_f q_c (outlet), from FP64 copies of the coefficients and with
@@ -1282,10 +1249,7 @@ __device__ __forceinline__ V cg_alpha(const double *pap_part, int npap, double *
     const double pap = dot_total<V>(pap_part, npap);
     if (block_leader()) alpha_s = (V)(rz / pap);
     __syncthreads();
-    if (block_leader() && BLOCK_ID() == 0) {
-        scal[S_PAP] = pap;
-        scal[S_RZ0] = rz;
-    }
+    if (block_leader() && BLOCK_ID() == 0) scal[S_RZ0] = rz;
     return alpha_s;
 }
 
@@ -1332,7 +1296,7 @@ __global__ void __launch_bounds__(256) k_cg_apply_dot(GridD g, C3<V> cf, const V
                 pn[2 * a + 1] = ijk[a] < n[a] - 1 ? p[c + off[a]] : V(0);
             }
 #pragma unroll
-            for (int q = 0; q < 2 * DIM; ++q) y = mg_madd(w[q], pc - pn[q], y);   // same terms and order as poisson_row
+            for (int q = 0; q < 2 * DIM; ++q) y = mg_madd(w[q], pc - pn[q], y);   // by axis, low face first
             Ap[c] = y;
             acc.add(pc * y);
         }
@@ -1412,7 +1376,7 @@ __global__ void __launch_bounds__(256) k_cg_pz_apply(GridD g, C3<T> cf, const V 
         for (int u = 0; u < RPT; ++u) {
             if (!in[u]) continue;
             const V pn = fresh ? zc[u] : zc[u] + be * po[u];
-            V y = V(0);   // same terms and order as poisson_row
+            V y = V(0);   // by axis, low face first
 #pragma unroll
             for (int q = 0; q < 2 * DIM; ++q) y += (V)w[u][q] * (zc[u] - zn[u][q]);
             const V an = fresh ? y : y + be * ao[u];
@@ -1546,7 +1510,7 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
 // formed without rounding error and the terms are summed with TwoSum, so the
 // pair matches the exact row value to about 2^-46 of the sum of the term
 // magnitudes -- FP64-grade, with FP32 instructions only. Same faces as
-// poisson_row.
+// poisson_row64.
 template <int DIM>
 __device__ __forceinline__ void poisson_row_comp(const GridD &g, uint32_t inf, int c, int i, int j, int k,
                                                  C3<float> cf, const float *__restrict__ e, float &s, float &cc) {

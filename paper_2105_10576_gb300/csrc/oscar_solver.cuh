@@ -985,10 +985,13 @@ template <typename T> int Solver<T>::setup(Instance &I, const uint8_t *solid_dev
     // the attributes belong to the kernels, not to this instance: they are set
     // to the budget (never lowered), so that instances of other sizes, created
     // while this one runs, cannot shrink them below what this one launches with
-    const void *inv = I.g.dim == 3 ? (const void *)k_mg_inverse_band<3, T> : (const void *)k_mg_inverse_band<2, T>;
+    const void *inv = nullptr;   // FP32: static shared memory only
+    if constexpr (sizeof(T) == sizeof(double))
+        inv = I.g.dim == 3 ? (const void *)k_mg_inverse_band<3, T> : (const void *)k_mg_inverse_band<2, T>;
     const void *vcy = I.g.dim == 3 ? (const void *)k_mg_cluster<3, T> : (const void *)k_mg_cluster<2, T>;
     const void *sol = (const void *)k_solve_cluster<T>;
     for (const void *f : {inv, vcy, sol}) {
+        if (!f) continue;
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClSmemBytes) != cudaSuccess ||
             cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
             return OSCAR_E_CUDA;
