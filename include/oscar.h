@@ -214,8 +214,9 @@ typedef struct {
     int block_x;        /* cap on the x extent of the 256-thread blocks of cell kernels: 0 (none), 32, 64,
                            128 or 256 */
     int cta_global;     /* 1: the cluster has several CTAs and also takes larger levels (not the finest) when
-                           they fit, and a small 2D grid's pressure solve runs whole in one cluster; 0: a
-                           cluster of one CTA, with the levels of at most cta_cells cells only */
+                           they fit and leave each CTA few enough rows, and a small 2D grid's pressure solve
+                           runs whole in one cluster; 0: a cluster of one CTA, with the levels of at most
+                           cta_cells cells only */
 } oscar_schedule;
 
 /* Read the schedule of an instance. */

@@ -3,16 +3,16 @@
 // The lower levels of the V-cycle are far too small to fill the GPU, and as
 // one launch per half sweep they are a chain of dependent launches (1.2 us
 // each); in a single CTA they are bound by that SM's issue rate and, in FP64,
-// by its two FP64 FMAs per clock. Here a cluster of up to 16 CTAs holds them
-// in distributed shared memory: each CTA owns a slab of columns (an x range)
-// of every level and works it with a wide margin of ghost columns. A cluster
-// barrier takes 0.26-0.31 us (256-512 threads per CTA), a block barrier a
-// quarter of that, so the ghosts are recomputed rather than exchanged: given
-// the right-hand side on D ghost columns, each half sweep is valid on one
-// column less, and a whole level (pre-smoothing, residual, prolongation,
-// post-smoothing) passes with block barriers only. What crosses CTAs is the
-// restricted right-hand side, once per level, stored into every CTA whose
-// margin covers it (st.shared::cluster), followed by one cluster barrier.
+// by its two FP64 FMAs per clock. Here a cluster of CTAs (up to 8 for a V-cycle,
+// 16 for a whole solve) holds them in distributed shared memory: each CTA owns
+// a slab of columns (an x range) of every level and works it with a wide margin
+// of ghost columns. A cluster barrier takes 0.26-0.31 us (256-512 threads per
+// CTA), a block barrier a quarter of that, so the ghosts are recomputed rather
+// than exchanged: given the right-hand side on D ghost columns, each half sweep
+// is valid on one column less, and a whole level (pre-smoothing, residual,
+// prolongation, post-smoothing) passes with block barriers only. What crosses
+// CTAs is the restricted right-hand side, once per level, stored into every CTA
+// whose margin covers it (st.shared::cluster), followed by one cluster barrier.
 // Slab boundaries are multiples of the x coarsening factor down to the
 // coarsest level, so restriction stays inside a CTA.
 //

@@ -8,13 +8,15 @@
 // fastest and one face array per direction. Cell and face kernels run on 3D
 // grids (x over threadIdx.x for coalesced rows, y over threadIdx.y /
 // blockIdx.y, z over blockIdx.z), so no thread divides to find its cell.
-// Reductions write one partial per block and finish in one block, in a
-// fixed order, so every sum is deterministic run to run.
+// Reductions write one partial per block. The last block to finish sums them,
+// or, for the dot products of the CG, every block of the kernel that needs the
+// total; always in a fixed order, so every sum is deterministic run to run.
 //
 // Element types: T is the field type (double for the FP64 path, float for
 // the mixed path); V the CG vector type (= T); the multigrid runs in T.
-// FP64 arithmetic is rare on GB300 silicon, so the mixed path keeps it to
-// dot-product accumulation, norms and the outer defect correction.
+// FP64 arithmetic is rare on GB300 silicon, so the mixed path keeps it to the
+// totals of dot products and norms (FP32 pairs below them) and the outer defect
+// correction.
 //
 // Included by exactly one translation unit per element type.
 #pragma once

@@ -2,13 +2,15 @@
 // Sections 2.2, 3.1, 3.2) as CUDA graphs.
 //
 // Each API call (drag step, relaxation, standard step) launches one
-// instantiated graph and synchronises once. Inside the graph every pressure
-// solve is a conditional WHILE node whose body ends in a one-thread control
-// kernel, and the relaxation loop is an outer WHILE node whose control kernel
-// applies the paper's early exit (E_k < tol or k = N) on the device. The
-// mixed path nests an FP32 PCG (FP64 dot products) inside an FP64
-// defect-correction WHILE loop. Graphs are captured from the same launch
-// sequence the eager mode issues, and rebuilt when the time step changes.
+// instantiated graph and synchronises once. Inside the graph a pressure solve
+// is one conditional WHILE node of PCG iterations, whose last kernel (k_cg_check
+// in FP64, k_cg_refine on the mixed path, which also ends the FP64
+// defect-correction trips) decides on the next one; a small 2D grid's solve is
+// one launch of k_solve_cluster, without a loop node. The relaxation is an outer
+// WHILE node whose last reduction applies the paper's early exit (E_k < tol or
+// k = N) on the device. Dot products of FP32 vectors are summed in compensated
+// pairs. Graphs are captured from the same launch sequence the eager mode
+// issues, and rebuilt when the time step changes.
 #pragma once
 #include <stdlib.h>
 #include <string.h>
@@ -171,12 +173,14 @@ template <class F> int loop_while(Instance &I, cudaGraphConditionalHandle h, F b
 // in FP32, where a launch per half sweep is still bound by its latency; in FP64
 // the cluster is bound by FP64 issue above 1024 cells), of which a CTA works at
 // most kVcycleRows. A 2D grid of at most kSolveCells is solved whole in one
-// cluster when its vectors fit the shared memory: beyond that a solve alone is
-// still shorter in the cluster (512x64 mixed 3.55 against 4.30 ms per five steps,
-// 5.90 launched without any cluster), but it holds 16 SMs for work that the
-// launches spread thinner, and instances stepped together wait for each other
-// (ten of 1024x128 to 128x16: 12.4 against 10.2 ms; 64: 392 against 419 M
-// cell-updates/s).
+// cluster when its vectors fit the shared memory and its slabs start at even
+// columns (r.z pairs the columns 2 i and 2 i + 1; grids of one level, at most 128
+// cells, have slabs of any width and go by launches, nx = 1 apart). Beyond that
+// a solve alone is still shorter in the cluster (512x64 mixed 3.55 against 4.30
+// ms per five steps, 5.90 launched without any cluster), but it holds 16 SMs for
+// work that the launches spread thinner, and instances stepped together wait for
+// each other (ten of 1024x128 to 128x16: 12.4 against 10.2 ms; 64: 392 against
+// 419 M cell-updates/s).
 constexpr int kSolveCells = 16384;
 constexpr int kVcycleThreads = 512;
 // CTAs of the V-cycle's cluster: at most 8. 16 make a V-cycle 1 to 2 us
@@ -203,7 +207,9 @@ constexpr int kVcycleRows = 4 * kVcycleThreads;
 inline int solve_threads(int ncell) { return ncell <= 8192 ? 256 : 512; }
 // CTAs of the cluster: fewer exchange less, more have shorter slabs. FP32 at
 // 128x16 (six sub-steps): 8 CTAs 2.48 ms, 16 2.55; at 211x26 3.92 and 3.56.
-// FP64, bound by the SM's FP64 rate: 128x16 4.74 and 4.52.
+// FP64, bound by the SM's FP64 rate: 128x16 4.74 and 4.52. Many instances
+// together are faster with 8 (64 of 256x32, mixed: 24.3 ms per step, with 16
+// 27.1, before there were clusters 44.7).
 template <typename T> inline int solve_ctas(int ncell) { return sizeof(T) == sizeof(float) && ncell <= 2048 ? 8 : 16; }
 template <typename T> struct ClRule;
 template <> struct ClRule<float> {
